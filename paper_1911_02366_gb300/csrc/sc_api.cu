@@ -108,6 +108,9 @@ void free_all(sc_ctx* c) {
   if (c->gj_scale) cudaFree(c->gj_scale);
   c->gj_scale = nullptr;
   c->packed = false;
+  if (c->tri_x) cudaFree(c->tri_x);
+  c->tri_x = nullptr;
+  c->ls_full = c->black_full = c->zinv_ready = false;
   if (c->Sls16) cudaFree(c->Sls16);
   c->Sls16 = nullptr;
   c->ls16_ok = false;
@@ -397,12 +400,18 @@ sc_status sc_set_mesh(sc_ctx* c, int n, double L, int N) {
   }
   const bool sweep = c->cfg.precond == SC_PC_RED_BLACK || c->cfg.precond == SC_PC_LEARNED ||
                      c->cfg.precond == SC_PC_RB_SCHUR;
+  c->ls_full = sc::solve_full_inverse(sweep ? G.K / 2 : G.K, sweep);
+  c->black_full = sc::solve_full_inverse(c->n_black, true);
+  {
+    const size_t len = (size_t)G.K * ((G.nb + 31) / 32 * 32);
+    A(cudaMalloc(&c->tri_x, len * (c->cfg.precision == SC_PREC_MIXED ? sizeof(float) : sizeof(double))));
+  }
   if (sweep) {
     A(dalloc(&c->d_colour, (size_t)G.K)); A(dalloc(&c->Trb, n1));
     if (c->cfg.precision == SC_PREC_MIXED) A(dalloc(&c->Zrb, n1));
   }
   if (c->cfg.precond == SC_PC_RB_SCHUR) {
-    A(dalloc(&c->Zinv, (size_t)c->n_red * G.nb * G.nb));
+    A(dalloc(&c->Zinv, (size_t)c->n_red * G.nb * G.lds));
     A(dalloc(&c->d_redidx, (size_t)G.K)); A(dalloc(&c->d_face_tab, c->face_tab.size()));
   }
   if (c->cfg.precond == SC_PC_LEARNED || c->cfg.precond == SC_PC_RB_SCHUR) {
@@ -525,6 +534,7 @@ sc_status sc_condense(sc_ctx* c) {
   if (c->cfg.precond == SC_PC_LEARNED && !c->weights_set)
     return fail(c, SC_ERR_STATE, "learned preconditioner without weights (sc_set_learned_weights)");
   c->Sdiag_valid = false;
+  c->zinv_ready = false;
   const int zero = 0;
   SC_CUDA(cudaMemcpyAsync(c->d_status + 1, &zero, sizeof(int), cudaMemcpyHostToDevice, c->stream));
   SC_CUDA(sc::launch_condense(c));

@@ -88,8 +88,8 @@ cudaError_t run_all(sc_batch* b, cudaStream_t st) {
     c->stream = own;
   }
   const int n = (int)b->items.size();
-  // grouped launches of this run: GJ, copy, 3 finishing kernels, the products and the panels
-  long long nl = sc::grouped_gj_launches(b->nbig_gj, n, b->max_ni) + 4 + 2 * (long long)b->cls.size();
+  // grouped launches of this run: GJ, copy, the products, the panels and the finishing kernels
+  long long nl = sc::grouped_gj_launches(b->nbig_gj, n, b->max_ni) + 1 + 2 * (long long)b->cls.size();
   for (int step = 0; 32 * step < b->max_nb; ++step) {
     nl += (b->nbig_lu > 0 ? 1 : 0) + (n > b->nbig_lu ? 1 : 0);
     for (const OrderClass& oc : b->cls) nl += step < (int)oc.off_t.size() ? 1 : 0;
@@ -106,7 +106,9 @@ cudaError_t run_all(sc_batch* b, cudaStream_t st) {
     for (const OrderClass& oc : b->cls)
       if (e == cudaSuccess && step < (int)oc.off_t.size()) e = run_trailing(b, st, oc, step, oc.bn_t);
   }
-  if (e == cudaSuccess) e = sc::grouped_finish(st, b->d_items, n, b->max_nb);
+  int fin = 0;
+  if (e == cudaSuccess) e = sc::grouped_finish(st, b->d_items, b->items, &fin);
+  b->grouped_launches += fin;
   return e;
 }
 
@@ -188,6 +190,7 @@ sc_status sc_batch_create(sc_ctx* const* ctxs, int nctx, sc_batch** out) {
       it.rowperm = c->rowperm + (size_t)e * G.nb;
       it.status = nullptr;  // set once the status word exists
       it.dsc = reinterpret_cast<float*>(c->gj_scale) + (size_t)e * G.ni;
+      it.full = c->ls_full ? 1 : 0;
       b->items.push_back(it);
     }
   }

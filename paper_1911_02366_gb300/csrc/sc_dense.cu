@@ -980,29 +980,35 @@ __global__ void __launch_bounds__(256) k_diag_inv_grouped(const CondItem* __rest
   diag_inv_body<float>(it.nb, it.See, it.lds);
 }
 
-// Sequential LAPACK-style row interchanges -> one gather permutation per element:
-// row i of P A is row rowperm[i] of A.
+// Sequential LAPACK-style row interchanges -> one gather permutation per element: row i of P A
+// is row rowperm[i] of A.  One CTA per element; the interchanges are a chain, so one thread
+// walks it, on shared memory (in global memory the chain took 0.48 ms at n_b = 1090).
 __device__ void piv_to_perm_body(int n, const int* __restrict__ piv, int* __restrict__ rp) {
-  for (int i = 0; i < n; ++i) rp[i] = i;
-  for (int k = 0; k < n; ++k) {
-    const int p = piv[k];
-    if (p != k) { const int t = rp[k]; rp[k] = rp[p]; rp[p] = t; }
+  extern __shared__ int pperm[];  // [2 n]: pivots, permutation
+  int* pv = pperm;
+  int* pm = pperm + n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) { pv[i] = piv[i]; pm[i] = i; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < n; ++k) {
+      const int p = pv[k];
+      const int t = pm[k];
+      pm[k] = pm[p];
+      pm[p] = t;
+    }
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) rp[i] = pm[i];
 }
 
-__global__ void k_piv_to_perm(int n, const int* __restrict__ piv_all, int* __restrict__ rowperm, int nelem) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nelem) return;
-  piv_to_perm_body(n, piv_all + (long long)e * n, rowperm + (long long)e * n);
+__global__ void __launch_bounds__(128) k_piv_to_perm(int n, const int* __restrict__ piv_all, int* __restrict__ rowperm) {
+  piv_to_perm_body(n, piv_all + (long long)blockIdx.x * n, rowperm + (long long)blockIdx.x * n);
 }
 
-__global__ void k_piv_to_perm_grouped(const CondItem* __restrict__ items, int nitems) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nitems) return;
-  const CondItem it = items[t];
+__global__ void __launch_bounds__(128) k_piv_to_perm_grouped(const CondItem* __restrict__ items) {
+  const CondItem it = items[blockIdx.x];
   piv_to_perm_body(it.nb, it.piv, it.rowperm);
 }
-
 
 // ---- block-Jacobi solve with partitioned inverses -----------------------------------
 // With D_b the 32 x 32 diagonal blocks of the factors (their triangles replaced by the
@@ -1180,10 +1186,6 @@ __device__ __forceinline__ void ls_solve_warp(int n, int nblk, const TS* __restr
   }
 }
 
-// The same substitutions by a CTA of W warps per element, for meshes with too few elements
-// to fill the GPU one warp each: in every block row the W warps share the off-diagonal
-// 4-column groups (strided), their partial dot products meet in shared memory, and warp
-// 0 adds the diagonal block's part and writes the row.  Two CTA barriers per block row.
 // ls_solve_warp with loads issued ahead of the dependence on s: each block row's diagonal
 // block quads are loaded before its long dot product, and the first 8 quads of the next
 // row's long part before the row's result is written.  The factor entries do not depend on
@@ -1304,127 +1306,9 @@ __device__ __forceinline__ void ls_solve_warp_pf(int n, int nblk, const TS* __re
   }
 }
 
-template <class T, class TS, int W>
-__device__ __forceinline__ void ls_solve_cta(int n, int nblk, const TS* __restrict__ Le, int npad, T* s, T* red) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int nq = npad / 4;
-  for (int b = 0; b < nblk; ++b) {  // forward
-    const int i0 = 32 * b, R = i0 + lane;
-    const bool live = R < n;
-    const TS* row = Le + (long long)b * 32 * npad + 4 * lane;
-    T a0 = T(0), a1 = T(0);
-    if (live) {
-#pragma unroll 4
-      for (int q = w; q < i0 / 4; q += W) {
-        Quad<T, TS> m;
-        m.load(row + (long long)q * 128);
-        a0 = fma(m.v[0], s[4 * q], a0);
-        a1 = fma(m.v[1], s[4 * q + 1], a1);
-        a0 = fma(m.v[2], s[4 * q + 2], a0);
-        a1 = fma(m.v[3], s[4 * q + 3], a1);
-      }
-    }
-    red[w * 32 + lane] = a0 + a1;
-    __syncthreads();
-    if (w == 0) {
-      T d = s[R];
-      const int qd = min(i0 / 4 + 8, nq);
-#pragma unroll
-      for (int q = i0 / 4; q < qd; ++q) {
-        if (live && 4 * q < R) {
-          Quad<T, TS> m;
-          m.load(row + (long long)q * 128);
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (4 * q + j < R) d = fma(m.v[j], s[4 * q + j], d);
-        }
-      }
-      T sum = T(0);
-#pragma unroll
-      for (int k = 0; k < W; ++k) sum += red[k * 32 + lane];
-      __syncwarp();
-      if (live) s[R] = d - sum;
-    }
-    __syncthreads();
-  }
-  for (int b = nblk - 1; b >= 0; --b) {  // backward
-    const int i0 = 32 * b, R = i0 + lane;
-    const bool live = R < n;
-    const TS* row = Le + (long long)b * 32 * npad + 4 * lane;
-    T a0 = T(0), a1 = T(0);
-    if (live) {
-#pragma unroll 4
-      for (int q = i0 / 4 + 8 + w; q < nq; q += W) {
-        Quad<T, TS> m;
-        m.load(row + (long long)q * 128);
-        a0 = fma(m.v[0], s[4 * q], a0);
-        a1 = fma(m.v[1], s[4 * q + 1], a1);
-        a0 = fma(m.v[2], s[4 * q + 2], a0);
-        a1 = fma(m.v[3], s[4 * q + 3], a1);
-      }
-    }
-    red[w * 32 + lane] = a0 + a1;
-    __syncthreads();
-    if (w == 0) {
-      T d = T(0);
-      const int qd = min(i0 / 4 + 8, nq);
-#pragma unroll
-      for (int q = i0 / 4; q < qd; ++q) {
-        if (live && 4 * q + 3 >= R) {
-          Quad<T, TS> m;
-          m.load(row + (long long)q * 128);
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (4 * q + j >= R) d = fma(m.v[j], s[4 * q + j], d);
-        }
-      }
-      T sum = T(0);
-#pragma unroll
-      for (int k = 0; k < W; ++k) sum += red[k * 32 + lane];
-      __syncwarp();
-      if (live) s[R] = d - sum;
-    }
-    __syncthreads();
-  }
-}
-
-constexpr int kSolveCtaWarps = 8;
-
-// Element lists (red-black sweep): CTA / warp i serves element elist[i] (all elements when
-// elist is null); its factors are number i of LS / rowperm when compact, else number e;
-// vsub (optional) is subtracted from v on input.
-template <class T, class TS, int W = kSolveCtaWarps>
-__global__ void __launch_bounds__(32 * W) k_lu_solve_cta(int n, int nblk, const TS* __restrict__ LS,
-                                                                      long long lsstride, int npad,
-                                                                      const int* __restrict__ rowperm,
-                                                                      const double* __restrict__ v,
-                                                                      double* __restrict__ z, T* __restrict__ zt,
-                                                                      const int* __restrict__ elist, int compact,
-                                                                      const double* __restrict__ vsub) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int e = elist ? __ldg(elist + blockIdx.x) : blockIdx.x, ls = nblk * 32;
-  const int f = compact ? blockIdx.x : e;
-  T* s = reinterpret_cast<T*>(smem_raw);
-  T* red = s + ls;
-  const int* rp = rowperm + (long long)f * n;
-  const double* ve = v + (long long)e * n;
-  const double* we = vsub ? vsub + (long long)e * n : nullptr;
-  for (int i = threadIdx.x; i < ls; i += blockDim.x) {
-    T val = T(0);
-    if (i < n) {
-      const int r = __ldg(rp + i);
-      val = we ? (T)(ve[r] - we[r]) : (T)ve[r];
-    }
-    s[i] = val;
-  }
-  __syncthreads();
-  ls_solve_cta<T, TS, W>(n, nblk, LS + (long long)f * lsstride, npad, s, red);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    if (z) z[(long long)e * n + i] = (double)s[i];
-    if (zt) zt[(long long)e * n + i] = s[i];
-  }
-}
-
+// Element lists (red-black sweep): warp i serves element elist[i] (all elements when elist is
+// null); its factors are number i of LS / rowperm when compact, else number e; vsub (optional)
+// is subtracted from v on input.
 // z = (P^T L U)^-1 v, one warp per element (4 per CTA); the running vector (v, then x,
 // then z) sits in shared memory.  Arithmetic in the factor precision T; v in double,
 // outputs z (double) and / or zt (T).
@@ -1650,7 +1534,7 @@ cudaError_t condense_t(sc_ctx* c, T* Aown, T* Ainv, T* Y, T* See, bool tc, bool 
       k_lu<T><<<K, 256, smem, c->stream>>>(nb, See, (long long)nb * lds, lds, c->piv, c->d_status);
     }
     count_launch(c, 2);
-    k_piv_to_perm<<<cdiv(K, 128), 128, 0, c->stream>>>(nb, c->piv, c->rowperm, K);
+    k_piv_to_perm<<<K, 128, 2 * nb * sizeof(int), c->stream>>>(nb, c->piv, c->rowperm);
     const size_t dsm = (size_t)8 * 2 * 32 * 33 * sizeof(T);
     err = cudaFuncSetAttribute(k_diag_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);
     if (err != cudaSuccess) return err;
@@ -1661,6 +1545,7 @@ cudaError_t condense_t(sc_ctx* c, T* Aown, T* Ainv, T* Y, T* See, bool tc, bool 
     const int nblk = (nb + 31) / 32, npad = (nb + 3) & ~3;
     __half* LS16 = nullptr;
     if constexpr (std::is_same<T, float>::value) LS16 = c->Sls16;
+    if (c->ls_full) return tri_inverse<T>(c, nb, See, (long long)nb * lds, lds, LS, K, LS16, c->d_status + 1);
     k_solve_prep<T><<<dim3(nblk, K), 256, 0, c->stream>>>(nb, See, (long long)nb * lds, lds, LS,
                                                            (long long)nblk * 32 * npad, npad, LS16, c->d_status + 1);
   }
@@ -1697,23 +1582,23 @@ inline int ls_nblk(const Geo& G) { return (G.nb + 31) / 32; }
 inline int ls_npad(const Geo& G) { return (G.nb + 3) & ~3; }
 inline long long ls_stride(const Geo& G) { return (long long)ls_nblk(G) * 32 * ls_npad(G); }
 
-// Meshes with fewer elements than this solve the block-Jacobi system with a CTA per element;
-// element lists (the red-black sweep's colours) below the second bound.
-constexpr int kSolveCtaMaxElems = 2048;
-constexpr int kSolveListCtaMaxElems = 1024;
+// Below these counts the warp-per-element solve cannot fill the chip and its chain of block rows
+// sets the time, so the condensation inverts the whole triangles (sc_trinv.cu): launches over
+// every element of the mesh, and over element lists (one colour of the sweep).  Above them the
+// chains of many elements overlap: a list of 2048 elements of n_b = 490 runs at 0.83 of the HBM
+// rate, and inverting the triangles would cost more per system than the solves gain.
+constexpr int kSolveFullMaxElems = 2048;
+constexpr int kSolveFullMaxList = 1024;
+bool solve_full_inverse(int per_launch, bool list) {
+  return per_launch < (list ? kSolveFullMaxList : kSolveFullMaxElems);
+}
 
 template <class T, class TS>
 cudaError_t lu_solve_t(sc_ctx* c, const TS* LS, const double* v, double* z, T* zt) {
   const Geo& G = c->G;
   ProfScope ps(c, SCK_LU_SOLVE);
+  if (c->ls_full) return tri_solve<T, TS>(c, LS, c->rowperm, 0, nullptr, G.K, v, nullptr, z, zt);
   const size_t smem = (size_t)4 * ls_nblk(G) * 32 * sizeof(T);
-  if (G.K < kSolveCtaMaxElems) {
-    const size_t csm = (size_t)(ls_nblk(G) + kSolveCtaWarps) * 32 * sizeof(T);
-    k_lu_solve_cta<T, TS><<<G.K, 32 * kSolveCtaWarps, csm, c->stream>>>(G.nb, ls_nblk(G), LS, ls_stride(G),
-                                                                       ls_npad(G), c->rowperm, v, z, zt, nullptr, 0,
-                                                                       nullptr);
-    return cudaGetLastError();
-  }
   k_lu_solve<T, TS><<<cdiv(G.K, 4), 128, smem, c->stream>>>(G.nb, ls_nblk(G), LS, ls_stride(G), ls_npad(G),
                                                             c->rowperm, v, z, zt, G.K, nullptr, 0, nullptr);
   return cudaGetLastError();
@@ -1721,39 +1606,29 @@ cudaError_t lu_solve_t(sc_ctx* c, const TS* LS, const double* v, double* z, T* z
 
 // Block solves of a list of elements (one colour of the red-black sweep): factors LS /
 // rowperm by element, or compact (number i for list entry i); vsub subtracted from v.
-template <class T, class TS>
-cudaError_t lu_solve_list_t(sc_ctx* c, const TS* LS, const int* rowperm, int compact, const int* elist, int nlist,
-                            const double* v, const double* vsub, double* z, T* zt) {
+template <class T>
+cudaError_t lu_solve_list_t(sc_ctx* c, const T* LS, const int* rowperm, int compact, bool full, const int* elist,
+                            int nlist, const double* v, const double* vsub, double* z, T* zt) {
   const Geo& G = c->G;
   if (nlist <= 0) return cudaSuccess;
   ProfScope ps(c, SCK_LU_SOLVE, nlist);
-  // lists of 1024 elements or more keep one warp per element: at 2048 elements (one colour of
-  // 16^3) it takes 0.49 ms per launch against 0.57 ms with 4 and 0.64 ms with 8 warps per
-  // element (CTA kernel)
-  if (nlist < kSolveListCtaMaxElems) {
-    const size_t csm = (size_t)(ls_nblk(G) + kSolveCtaWarps) * 32 * sizeof(T);
-    k_lu_solve_cta<T, TS><<<nlist, 32 * kSolveCtaWarps, csm, c->stream>>>(G.nb, ls_nblk(G), LS, ls_stride(G),
-                                                                         ls_npad(G), rowperm, v, z, zt, elist,
-                                                                         compact, vsub);
-    return cudaGetLastError();
-  }
+  if (full) return tri_solve<T, T>(c, LS, rowperm, compact, elist, nlist, v, vsub, z, zt);
   const size_t smem = (size_t)4 * ls_nblk(G) * 32 * sizeof(T);
   // FP32 factors: loads issued ahead (128 registers, 4 CTAs per SM hold one colour of 16^3)
-  constexpr bool pf = std::is_same<T, float>::value && std::is_same<TS, float>::value;
-  k_lu_solve<T, TS, pf><<<cdiv(nlist, 4), 128, smem, c->stream>>>(G.nb, ls_nblk(G), LS, ls_stride(G),
-                                                                  ls_npad(G), rowperm, v, z, zt, nlist, elist,
-                                                                  compact, vsub);
+  constexpr bool pf = std::is_same<T, float>::value;
+  k_lu_solve<T, T, pf><<<cdiv(nlist, 4), 128, smem, c->stream>>>(G.nb, ls_nblk(G), LS, ls_stride(G), ls_npad(G),
+                                                                 rowperm, v, z, zt, nlist, elist, compact, vsub);
   return cudaGetLastError();
 }
 
-cudaError_t lu_solve_list(sc_ctx* c, const double* LS, const int* rowperm, int compact, const int* elist, int nlist,
-                          const double* v, const double* vsub, double* z) {
-  return lu_solve_list_t<double, double>(c, LS, rowperm, compact, elist, nlist, v, vsub, z, nullptr);
+cudaError_t lu_solve_list(sc_ctx* c, const double* LS, const int* rowperm, int compact, bool full, const int* elist,
+                          int nlist, const double* v, const double* vsub, double* z) {
+  return lu_solve_list_t<double>(c, LS, rowperm, compact, full, elist, nlist, v, vsub, z, nullptr);
 }
 
-cudaError_t lu_solve_list32(sc_ctx* c, const float* LS, const int* rowperm, int compact, const int* elist, int nlist,
-                            const double* v, const double* vsub, double* z, float* zt) {
-  return lu_solve_list_t<float, float>(c, LS, rowperm, compact, elist, nlist, v, vsub, z, zt);
+cudaError_t lu_solve_list32(sc_ctx* c, const float* LS, const int* rowperm, int compact, bool full, const int* elist,
+                            int nlist, const double* v, const double* vsub, double* z, float* zt) {
+  return lu_solve_list_t<float>(c, LS, rowperm, compact, full, elist, nlist, v, vsub, z, zt);
 }
 
 cudaError_t precond_apply(sc_ctx* c, const double* v, double* z) {
@@ -1840,14 +1715,28 @@ cudaError_t grouped_lu_panel(cudaStream_t st, const CondItem* items, int n, int 
   return cudaGetLastError();
 }
 
-cudaError_t grouped_finish(cudaStream_t st, const CondItem* items, int n, int max_nb) {
-  k_piv_to_perm_grouped<<<cdiv(n, 128), 128, 0, st>>>(items, n);
+cudaError_t grouped_finish(cudaStream_t st, const CondItem* items, const std::vector<CondItem>& host, int* launches) {
+  const int n = (int)host.size(), max_nb = n ? host[0].nb : 0;  // sorted by decreasing block size
+  k_piv_to_perm_grouped<<<n, 128, 2 * max_nb * sizeof(int), st>>>(items);
   const size_t dsm = (size_t)8 * 2 * 32 * 33 * sizeof(float);
   cudaError_t e = cudaFuncSetAttribute(k_diag_inv_grouped, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);
   if (e != cudaSuccess) return e;
   k_diag_inv_grouped<<<n, 256, dsm, st>>>(items);
-  k_solve_prep_grouped<<<dim3((max_nb + 31) / 32, n), 256, 0, st>>>(items);
-  return cudaGetLastError();
+  *launches = 2;
+  for (int i = 0; i < n && e == cudaSuccess;) {  // runs of one block size and solve form
+    int k = i;
+    while (k < n && host[k].nb == host[i].nb && host[k].full == host[i].full) ++k;
+    if (host[i].full) {
+      e = grouped_tri_inverse(st, items + i, k - i, host[i].nb);
+      *launches += 2;
+    } else {
+      k_solve_prep_grouped<<<dim3((host[i].nb + 31) / 32, k - i), 256, 0, st>>>(items + i);
+      *launches += 1;
+      e = cudaGetLastError();
+    }
+    i = k;
+  }
+  return e;
 }
 
 cudaError_t to_float(sc_ctx* c, const double* a, float* b, size_t n) {
@@ -1880,7 +1769,7 @@ long long solve_layout_stride(const Geo& G) { return ls_stride(G); }
 // LU with partial pivoting of `batch` FP32 n x n blocks (row-major, lda, `stride` apart),
 // then the gather permutation and the partitioned-inverse solve layout LS.
 cudaError_t factor_batch32(sc_ctx* c, float* A, int n, int lda, long long stride, int batch, int* piv, int* rowperm,
-                           float* LS, int* status) {
+                           float* LS, int* status, bool full) {
   cudaError_t err;
   if (c->cfg.tensor_cores && n == c->G.nb && lda == c->G.lds && stride == (long long)n * lda) {
     err = lu_blocked_tf32_batch(c, A, batch, piv, status);  // element-block sized: TF32 trailing updates
@@ -1893,11 +1782,12 @@ cudaError_t factor_batch32(sc_ctx* c, float* A, int n, int lda, long long stride
     count_launch(c, 4);
     k_lu<float><<<batch, 256, smem, c->stream>>>(n, A, stride, lda, piv, status);
   }
-  k_piv_to_perm<<<cdiv(batch, 128), 128, 0, c->stream>>>(n, piv, rowperm, batch);
+  k_piv_to_perm<<<batch, 128, 2 * n * sizeof(int), c->stream>>>(n, piv, rowperm);
   const size_t dsm = (size_t)8 * 2 * 32 * 33 * sizeof(float);
   err = cudaFuncSetAttribute(k_diag_inv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);
   if (err != cudaSuccess) return err;
   k_diag_inv<float><<<batch, 256, dsm, c->stream>>>(n, A, stride, lda);
+  if (full) return tri_inverse<float>(c, n, A, stride, lda, LS, batch);
   const int nblk = (n + 31) / 32, npad = (n + 3) & ~3;
   k_solve_prep<float><<<dim3(nblk, batch), 256, 0, c->stream>>>(n, A, stride, lda, LS, (long long)nblk * 32 * npad,
                                                                npad, nullptr, nullptr);
@@ -1927,6 +1817,7 @@ __global__ void __launch_bounds__(128) k_inv_node_blocks(int n, int nblk, const 
 
 cudaError_t inverse_node_blocks32(sc_ctx* c, float* out) {
   const Geo& G = c->G;
+  if (c->ls_full || c->red_compact) return tri_node_blocks(c, c->Sls32, c->rowperm, out);
   const int nblk = ls_nblk(G);
   const size_t smem = (size_t)4 * nblk * 32 * sizeof(float);
   cudaError_t err = cudaFuncSetAttribute(k_inv_node_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1935,157 +1826,6 @@ cudaError_t inverse_node_blocks32(sc_ctx* c, float* out) {
   const long long nw = (long long)G.K * G.nbn * 5;
   k_inv_node_blocks<<<cdiv(nw, 4), 128, smem, c->stream>>>(G.nb, nblk, c->Sls32, ls_stride(G), ls_npad(G), c->rowperm,
                                                            (int)nw, out);
-  return cudaGetLastError();
-}
-
-
-// ls_solve_warp for R right-hand sides at once (s: R vectors of nblk * 32 entries, stride
-// ls, zero beyond n): every factor entry the warp loads serves all R columns.
-// The forward pass starts at block row b0: the right-hand sides are zero above row 32 b0.
-template <int R>
-__device__ __forceinline__ void ls_solve_warp_multi(int n, int nblk, const float* __restrict__ Le, int npad,
-                                                    float* s, int ls, int lane, int b0) {
-  const int nq = npad / 4;
-  for (int b = b0; b < nblk; ++b) {  // forward: x_b = L_bb^-1 v_b - M_b x_{<b}
-    const int i0 = 32 * b, Rw = i0 + lane;
-    const bool live = Rw < n;
-    const float* row = Le + (long long)b * 32 * npad + 4 * lane;
-    float a[R], d[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) a[r] = 0.f;
-    if (live) {
-#pragma unroll 2
-      for (int q = 8 * b0; q < i0 / 4; ++q) {
-        Quad<float, float> m;
-        m.load(row + (long long)q * 128);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const float4 x = *reinterpret_cast<const float4*>(s + r * ls + 4 * q);
-          a[r] = fmaf(m.v[0], x.x, a[r]);
-          a[r] = fmaf(m.v[1], x.y, a[r]);
-          a[r] = fmaf(m.v[2], x.z, a[r]);
-          a[r] = fmaf(m.v[3], x.w, a[r]);
-        }
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) d[r] = s[r * ls + Rw];
-    const int qd = min(i0 / 4 + 8, nq);
-    for (int q = i0 / 4; q < qd; ++q) {
-      if (live && 4 * q < Rw) {  // strictly lower part: columns < Rw
-        Quad<float, float> m;
-        m.load(row + (long long)q * 128);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (4 * q + j < Rw) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) d[r] = fmaf(m.v[j], s[r * ls + 4 * q + j], d[r]);
-          }
-      }
-    }
-    __syncwarp();
-    if (live) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) s[r * ls + Rw] = d[r] - a[r];
-    }
-    __syncwarp();
-  }
-  for (int b = nblk - 1; b >= 0; --b) {  // backward: z_b = U_bb^-1 x_b - N_b z_{>b}
-    const int i0 = 32 * b, Rw = i0 + lane;
-    const bool live = Rw < n;
-    const float* row = Le + (long long)b * 32 * npad + 4 * lane;
-    float a[R], d[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) a[r] = d[r] = 0.f;
-    const int qd = min(i0 / 4 + 8, nq);
-    for (int q = i0 / 4; q < qd; ++q) {
-      if (live && 4 * q + 3 >= Rw) {  // upper part: columns >= Rw
-        Quad<float, float> m;
-        m.load(row + (long long)q * 128);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (4 * q + j >= Rw) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) d[r] = fmaf(m.v[j], s[r * ls + 4 * q + j], d[r]);
-          }
-      }
-    }
-    if (live) {
-#pragma unroll 2
-      for (int q = i0 / 4 + 8; q < nq; ++q) {
-        Quad<float, float> m;
-        m.load(row + (long long)q * 128);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const float4 x = *reinterpret_cast<const float4*>(s + r * ls + 4 * q);
-          a[r] = fmaf(m.v[0], x.x, a[r]);
-          a[r] = fmaf(m.v[1], x.y, a[r]);
-          a[r] = fmaf(m.v[2], x.z, a[r]);
-          a[r] = fmaf(m.v[3], x.w, a[r]);
-        }
-      }
-    }
-    __syncwarp();
-    if (live) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) s[r * ls + Rw] = d[r] - a[r];
-    }
-    __syncwarp();
-  }
-}
-
-namespace {
-
-constexpr int kInvCols = 4;   // right-hand sides per warp in k_inv_columns
-constexpr int kInvWarps = 4;  // warps per CTA
-
-// Explicit inverses of the element blocks listed: warp w solves S_ee X = I[:, c0 .. c0 + R - 1]
-// (R = kInvCols) for element list[w / ngrp], c0 = R (w % ngrp), with the condensation's factors, and writes
-// the columns contiguously: out[(i n + c) n + r] = (S_ee^-1)[r][c], i the list index.
-__global__ void __launch_bounds__(32 * kInvWarps) k_inv_columns(int n, int nblk, const float* __restrict__ LS,
-                                                               long long lsstride, int npad,
-                                                               const int* __restrict__ rowperm,
-                                                               const int* __restrict__ list, int nlist,
-                                                               float* __restrict__ out) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-  const int ngrp = (n + kInvCols - 1) / kInvCols;
-  const long long w = (long long)blockIdx.x * kInvWarps + warp;
-  if (w >= (long long)nlist * ngrp) return;
-  const int li = (int)(w / ngrp), c0 = (int)(w % ngrp) * kInvCols;
-  const int e = list ? __ldg(list + li) : li;  // no list: entries in list order (compact factors)
-  const int ls = nblk * 32;
-  float* s = reinterpret_cast<float*>(smem_raw) + (size_t)warp * kInvCols * ls;
-  const int* rp = rowperm + (long long)e * n;
-  int first = n;  // the lowest row holding a one: the forward pass starts at its block
-  for (int i = lane; i < ls; i += 32) {
-    const int pi = i < n ? __ldg(rp + i) : -1;
-    if (pi >= c0 && pi < c0 + kInvCols) first = min(first, i);
-#pragma unroll
-    for (int r = 0; r < kInvCols; ++r) s[r * ls + i] = pi == c0 + r ? 1.f : 0.f;
-  }
-  first = __reduce_min_sync(0xffffffffu, first);
-  __syncwarp();
-  ls_solve_warp_multi<kInvCols>(n, nblk, LS + (long long)e * lsstride, npad, s, ls, lane, min(first, n - 1) / 32);
-  for (int r = 0; r < kInvCols && c0 + r < n; ++r) {
-    float* o = out + ((long long)li * n + c0 + r) * n;
-    for (int i = lane; i < n; i += 32) o[i] = s[r * ls + i];
-  }
-}
-
-}  // namespace
-
-cudaError_t inverse_columns32(sc_ctx* c, const int* list, int nlist, float* out) {
-  const Geo& G = c->G;
-  if (nlist == 0) return cudaSuccess;
-  const int nblk = ls_nblk(G);
-  const size_t smem = (size_t)kInvWarps * kInvCols * nblk * 32 * sizeof(float);
-  cudaError_t err = cudaFuncSetAttribute(k_inv_columns, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  count_launch(c);
-  const long long nw = (long long)nlist * cdiv(G.nb, kInvCols);
-  k_inv_columns<<<(unsigned)cdiv(nw, kInvWarps), 32 * kInvWarps, smem, c->stream>>>(G.nb, nblk, c->Sls32, ls_stride(G), ls_npad(G),
-                                                                 c->rowperm, list, nlist, out);
   return cudaGetLastError();
 }
 

@@ -320,6 +320,11 @@ struct sc_ctx {
   float* Sls32 = nullptr;
   __half* Sls16 = nullptr;  // FP16 copy of the mixed arm's layout, used when every entry is in range
   bool ls16_ok = false;
+  // block solves with the inverted triangles (sc_trinv.cu): of all elements, of the black ones in
+  // SlsL, and the dense inverses of the red ones in Zinv; tri_x: the vector between the two
+  // triangular products (K x 32 ceil(n_b / 32) values of the operator precision)
+  bool ls_full = false, black_full = false, zinv_ready = false;
+  void* tri_x = nullptr;
   bool packed = false;     // packed blocks match the assembled Jacobian
   // learned correction of the block-Jacobi preconditioner (mixed arm)
   std::vector<int> l_face, l_mirror;  // per boundary position: face, co-located position
@@ -353,8 +358,8 @@ struct sc_ctx {
   bool blackL_valid = false;  // SlsL holds the factors of the corrected black blocks
   bool red_compact = false;   // SC_PC_RB_SCHUR: Sls32 / rowperm hold only the red blocks' factors,
                               // entry i for the i-th red element (the black ones are in SlsL)
-  // Schur-corrected sweep (SC_PC_RB_SCHUR): the red blocks' inverses, column-major per red
-  // element (Zinv[r][j][i] = (S_rr^-1)[i][j], r the red list index), red index of every
+  // Schur-corrected sweep (SC_PC_RB_SCHUR): the red blocks' inverses, column-major with leading
+  // dimension lds per red element (Zinv[r][j][i] = (S_rr^-1)[i][j], r the red list index), red index of every
   // element (-1 for black), and per face f the (N+1)^2 boundary nodes on f with the slot of f
   // in each node's face list: face_tab[(2 f) P2 + t] = node, face_tab[(2 f + 1) P2 + t] = slot
   float* Zinv = nullptr;
@@ -417,6 +422,7 @@ struct CondItem {
   int *piv, *rowperm;
   int* status;
   float* dsc;                     // n_i row scales of the blocked Gauss-Jordan (n_i > 136)
+  int full;                       // 1: Sls holds the inverted triangles (sc_trinv.cu)
 };
 
 // Status word value written by a tensor-core kernel whose bounded wait ran out (element
@@ -467,7 +473,20 @@ size_t solve_layout_elems(const Geo& G);
 void build_packed_pattern(sc_ctx* c);
 long long solve_layout_stride(const Geo& G);
 cudaError_t factor_batch32(sc_ctx* c, float* A, int n, int lda, long long stride, int batch, int* piv, int* rowperm,
-                           float* LS, int* status);
+                           float* LS, int* status, bool full);
+// Meshes whose block solves use the inverted triangles: `per_launch` elements per solve launch.
+bool solve_full_inverse(int per_launch, bool list);
+template <class T>
+cudaError_t tri_inverse(sc_ctx* c, int n, const T* LU, long long stride, int lda, T* LS, int count,
+                        __half* LS16 = nullptr, int* ovf = nullptr);
+cudaError_t grouped_tri_inverse(cudaStream_t st, const CondItem* items, int count, int nb);
+template <class T, class TS>
+cudaError_t tri_solve(sc_ctx* c, const TS* LS, const int* rowperm, int compact, const int* elist, int count,
+                      const double* v, const double* vsub, double* z, T* zt);
+cudaError_t tri_dense_inverse(sc_ctx* c, const float* LS, const int* rowperm, int count, float* out);
+cudaError_t dense_inverse_apply(sc_ctx* c, const float* inv, const int* elist, int count, const double* v, double* z,
+                                float* zt);
+cudaError_t tri_node_blocks(sc_ctx* c, const float* LS, const int* rowperm, float* out);
 void build_learned_tables(sc_ctx* c);
 void build_explicit_tables(sc_ctx* c);
 cudaError_t upload_explicit_tables(sc_ctx* c);
@@ -482,7 +501,8 @@ bool gj_blocked_item(int ni);
 bool lu_panel_smem_item(int nb);
 cudaError_t grouped_copy_bb(cudaStream_t st, const CondItem* items, int n);
 cudaError_t grouped_lu_panel(cudaStream_t st, const CondItem* items, int n, int nbig, int k0, int max_nb);
-cudaError_t grouped_finish(cudaStream_t st, const CondItem* items, int n, int max_nb);
+// host: the same items; returns the launches made in *launches
+cudaError_t grouped_finish(cudaStream_t st, const CondItem* items, const std::vector<CondItem>& host, int* launches);
 cudaError_t to_float(sc_ctx* c, const double* a, float* b, size_t n);
 cudaError_t gemm_tf32_ptrs(cudaStream_t stream, int M, int N, int K, float alpha, const float* const* Ap, int lda,
                            bool ta, const float* const* Bp, int ldb, bool tb, float beta, float* const* Cp, int ldc,
@@ -512,10 +532,11 @@ cudaError_t cond_boundary_pk(sc_ctx* c, const T* Apk, const T* X, const T* xb, d
 cudaError_t vec_axpby(sc_ctx* c, double* y, double a, const double* x, double b, size_t n);
 // block solves of a list of elements (factors by element, or compact by list position), vsub
 // subtracted from the right-hand side
-cudaError_t lu_solve_list(sc_ctx* c, const double* LS, const int* rowperm, int compact, const int* elist, int nlist,
-                          const double* v, const double* vsub, double* z);
-cudaError_t lu_solve_list32(sc_ctx* c, const float* LS, const int* rowperm, int compact, const int* elist, int nlist,
-                            const double* v, const double* vsub, double* z, float* zt);
+// (full: the factors are the inverted triangles)
+cudaError_t lu_solve_list(sc_ctx* c, const double* LS, const int* rowperm, int compact, bool full, const int* elist,
+                          int nlist, const double* v, const double* vsub, double* z);
+cudaError_t lu_solve_list32(sc_ctx* c, const float* LS, const int* rowperm, int compact, bool full, const int* elist,
+                            int nlist, const double* v, const double* vsub, double* z, float* zt);
 template <class T>
 cudaError_t cond_boundary_pk_list(sc_ctx* c, const T* Apk, const T* X, const T* xb, const T* u, double* y,
                                   const int* elist, int nlist);
@@ -530,7 +551,6 @@ void build_face_tables(sc_ctx* c);
 cudaError_t schur_black_factor(sc_ctx* c);
 cudaError_t red_factor32(sc_ctx* c, const float* See);
 cudaError_t plain_black_factor(sc_ctx* c);
-cudaError_t inverse_columns32(sc_ctx* c, const int* list, int nlist, float* out);
 cudaError_t gather_black_see(sc_ctx* c, const float* See);
 template <class T>
 cudaError_t gemm_update(sc_ctx* c, int M, int N, int K, const T* A, int lda, const T* B, int ldb, T* C, int ldc);

@@ -1114,6 +1114,10 @@ sc_status sc_mixed_create(const sc_config* cfg, void* cuda_stream, int n, double
     c.view = new sc_ctx();
     c.view->G = Gc; c.view->stream = c.st; c.view->cfg = *cfg;
     c.view->rowperm = c.rowperm;
+    c.view->ls_full = sc::solve_full_inverse(c.count, true);
+    float* tx = nullptr;
+    A(mx_alloc(&tx, k * (size_t)((c.nb + 31) / 32 * 32)));
+    c.view->tri_x = tx;
     m->max_ni = std::max(m->max_ni, c.ni);
     m->max_nb = std::max(m->max_nb, c.nb);
   }
@@ -1134,6 +1138,7 @@ sc_status sc_mixed_create(const sc_config* cfg, void* cuda_stream, int n, double
         it.rowperm = c.rowperm + (size_t)i * c.nb;
         it.status = m->d_status;
         it.dsc = c.dsc + (size_t)i * c.ni;
+        it.full = c.view->ls_full ? 1 : 0;
         m->items.push_back(it);
       }
     for (const CondItem& it : m->items) {
@@ -1200,6 +1205,7 @@ void sc_mixed_destroy(sc_mixed* m) {
     for (void* p : cs) if (p) cudaFree(p);
     if (c.st) cudaStreamDestroy(c.st);
     if (c.done) cudaEventDestroy(c.done);
+    if (c.view && c.view->tri_x) cudaFree(c.view->tri_x);
     delete c.view;
   }
   if (m->fork) cudaEventDestroy(m->fork);
@@ -1323,7 +1329,9 @@ cudaError_t mx_condense_blocks(sc_mixed* m) {
       e = mx_products(m, c, c.off_t[step], rest, rest, 32, -1.0f, c.lds, false, c.lds, false, 1.0f, c.lds);
     }
   }
-  if (e == cudaSuccess) { e = sc::grouped_finish(st, m->d_items, n, m->max_nb); m->launches += 3; }
+  int fin = 0;
+  if (e == cudaSuccess) e = sc::grouped_finish(st, m->d_items, m->items, &fin);
+  m->launches += fin;
   return e;
 }
 
@@ -1383,7 +1391,8 @@ cudaError_t mx_precond(sc_mixed* m, const double* v, double* z) {
   cudaError_t e = mx_per_class(m, [&](MxClass& c) {
     const long long o = m->boff[c.slot0];
     m->launches += 1;
-    return sc::lu_solve_list32(c.view, c.Sls32, c.rowperm, 0, nullptr, c.count, v + o, nullptr, z + o, nullptr);
+    return sc::lu_solve_list32(c.view, c.Sls32, c.rowperm, 0, c.view->ls_full, nullptr, c.count, v + o, nullptr, z + o,
+                               nullptr);
   });
   if (m->prof) cudaEventRecord(m->prof_ev[2 * m->prof_used++ + 1], m->stream);
   return e;

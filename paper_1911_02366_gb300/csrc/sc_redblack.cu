@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) k_face_schur(Geo G, const int* __restrict
     const int m = __ldg(nbr + (long long)b * 18 + f);
     const int ri = __ldg(redidx + m);
     if (ri >= 0) {
-      const float* Z = Zinv + (long long)ri * nb * nb;
+      const float* Z = Zinv + (long long)ri * nb * G.lds;
       const int* fa = ftab + 2 * f * P2;
       const int* fs = fa + P2;
       for (int p = threadIdx.x; p < P2 * P2; p += blockDim.x) {
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(256) k_face_schur(Geo G, const int* __restrict
           for (int cc = 0; cc < 5; ++cc) T[5 * r + cc] = 0.f;
 #pragma unroll
         for (int t = 0; t < 5; ++t) {
-          const float* zc = Z + (long long)(5 * bm + t) * nb + 5 * am;  // column 5 l' + t, rows of k'
+          const float* zc = Z + (long long)(5 * bm + t) * G.lds + 5 * am;  // column 5 l' + t, rows of k'
           float zr[5], sr[5];
 #pragma unroll
           for (int r = 0; r < 5; ++r) zr[r] = __ldg(zc + r);
@@ -162,12 +162,12 @@ cudaError_t precond_rb(sc_ctx* c, const double* v, double* z) {
   const Geo& G = c->G;
   const size_t n1 = (size_t)G.K * G.nb;
   cudaError_t e = cudaMemsetAsync(z, 0, n1 * sizeof(double), c->stream);
-  if (e == cudaSuccess) e = lu_solve_list(c, c->Sls, c->rowperm, 0, c->d_colour, c->n_red, v, nullptr, z);
+  if (e == cudaSuccess) e = lu_solve_list(c, c->Sls, c->rowperm, 0, c->ls_full, c->d_colour, c->n_red, v, nullptr, z);
   if (e == cudaSuccess) e = cond_interior_sweep(c, z, c->Ui);
   if (e == cudaSuccess)
     e = cond_boundary_pk_list<double>(c, c->Apk, c->X, z, c->Ui, c->Trb, c->d_colour + c->n_red, c->n_black);
   if (e == cudaSuccess)
-    e = lu_solve_list(c, c->Sls, c->rowperm, 0, c->d_colour + c->n_red, c->n_black, v, c->Trb, z);
+    e = lu_solve_list(c, c->Sls, c->rowperm, 0, c->ls_full, c->d_colour + c->n_red, c->n_black, v, c->Trb, z);
   return e;
 }
 
@@ -180,15 +180,22 @@ cudaError_t precond_rb32(sc_ctx* c, const double* v, double* z, float* zf) {
                                              c->cfg.precond == SC_PC_RB_SCHUR);
   const int* black = c->d_colour + c->n_red;
   cudaError_t e = cudaMemsetAsync(zt, 0, n1 * sizeof(float), c->stream);
-  if (e == cudaSuccess)
-    e = lu_solve_list32(c, c->Sls32, c->rowperm, c->red_compact ? 1 : 0, c->d_colour, c->n_red, v, nullptr, z, zt);
+  if (e == cudaSuccess) {
+    if (c->zinv_ready) {  // the red inverses that the corrected black blocks were formed from
+      ProfScope ps(c, SCK_LU_SOLVE, c->n_red);
+      e = dense_inverse_apply(c, c->Zinv, c->d_colour, c->n_red, v, z, zt);
+    } else {
+      e = lu_solve_list32(c, c->Sls32, c->rowperm, c->red_compact ? 1 : 0, c->red_compact || c->ls_full, c->d_colour,
+                          c->n_red, v, nullptr, z, zt);
+    }
+  }
   if (e == cudaSuccess) e = cond_interior_sweep32(c, zt, c->Uf);
   if (e == cudaSuccess) e = cond_boundary_pk_list<float>(c, c->Apk32, c->X32, zt, c->Uf, c->Trb, black, c->n_black);
   if (e == cudaSuccess) {
     if (corrected)
-      e = lu_solve_list32(c, c->SlsL, c->rowpermL, 1, black, c->n_black, v, c->Trb, z, zt);
+      e = lu_solve_list32(c, c->SlsL, c->rowpermL, 1, c->black_full, black, c->n_black, v, c->Trb, z, zt);
     else
-      e = lu_solve_list32(c, c->Sls32, c->rowperm, 0, black, c->n_black, v, c->Trb, z, zt);
+      e = lu_solve_list32(c, c->Sls32, c->rowperm, 0, c->ls_full, black, c->n_black, v, c->Trb, z, zt);
   }
   return e;
 }
@@ -229,7 +236,7 @@ static cudaError_t black_factor(sc_ctx* c, const float* Ck, float scale, bool fa
     if (e != cudaSuccess) return e;
   }
   e = factor_batch32(c, c->SeeL, G.nb, G.lds, (long long)per, c->n_black, c->pivL, c->rowpermL, c->SlsL,
-                     c->d_status + 2);
+                     c->d_status + 2, c->black_full);
   if (e == cudaSuccess) c->blackL_valid = true;
   return e;
 }
@@ -238,18 +245,21 @@ cudaError_t learned_black_factor(sc_ctx* c, const float* Ck, float scale) { retu
 
 // SC_PC_RB_SCHUR after the condensation: couplings, red inverses, corrected black factors.
 cudaError_t schur_black_factor(sc_ctx* c) {
-  if (!c->Zinv || !c->SeeB || c->n_black == 0) {
+  c->zinv_ready = false;
+  if (!c->Zinv || !c->SeeB || c->n_black == 0 || !c->red_compact) {
     c->blackL_valid = false;
     return cudaSuccess;
   }
   cudaError_t e = learned_couplings(c);
-  if (e == cudaSuccess) e = inverse_columns32(c, c->red_compact ? nullptr : c->d_colour, c->n_red, c->Zinv);
+  if (e == cudaSuccess) e = tri_dense_inverse(c, c->Sls32, c->rowperm, c->n_red, c->Zinv);
   if (e == cudaSuccess) e = black_factor(c, nullptr, 0.f, true);
+  c->zinv_ready = e == cudaSuccess;
   return e;
 }
 
 // The red blocks alone (SC_PC_RB_SCHUR): gathered into SeeL (free until the black correction)
-// and factorised into the first n_red entries of the solve layout and of rowperm.
+// and factorised into the first n_red entries of the solve layout (inverted triangles, from which
+// the dense inverses follow) and of rowperm.
 cudaError_t red_factor32(sc_ctx* c, const float* See) {
   const Geo& G = c->G;
   if (c->n_red == 0) return cudaSuccess;
@@ -259,7 +269,7 @@ cudaError_t red_factor32(sc_ctx* c, const float* See) {
   if (e != cudaSuccess) return e;
   const size_t per = (size_t)G.nb * G.lds;
   return factor_batch32(c, c->SeeL, G.nb, G.lds, (long long)per, c->n_red, c->piv, c->rowperm, c->Sls32,
-                        c->d_status);
+                        c->d_status, true);
 }
 
 // The plain black blocks into SlsL: the Schur-corrected sweep's fallback when a corrected

@@ -1,0 +1,47 @@
+"""Block-Jacobi solves with the element Schur blocks against S_ee formed in FP64 from the
+assembled own blocks, at the block sizes of every order (n_b from 130 to 1090: one partial 32-row
+block, an odd and an even number of block rows)."""
+import numpy as np
+import pytest
+
+import oracle as O
+from gpu_common import case
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _schur_block(ctx, e, N):
+    p = N + 1
+    A = ctx.sc_get_jacobian_block(e, e)
+    i = np.arange(p)
+    inner1 = (i > 0) & (i < N)
+    inner = (inner1[:, None, None] & inner1[None, :, None] & inner1[None, None, :]).reshape(-1)
+    I = np.repeat(inner, 5)
+    Aii, Aib, Abi, Abb = A[np.ix_(I, I)], A[np.ix_(I, ~I)], A[np.ix_(~I, I)], A[np.ix_(~I, ~I)]
+    return Abb - Abi @ np.linalg.solve(Aii, Aib)
+
+
+@pytest.mark.parametrize("arm,N", [("fp64", 2), ("fp64", 3), ("fp64", 4), ("fp64", 5), ("mixed", 2), ("mixed", 3),
+                                   ("mixed", 4), ("mixed", 5), ("mixed", 6)])
+def test_block_jacobi_apply_solves_the_element_schur_blocks(arm, N):
+    """z = P v, S_ee z_e = v_e, as a backward error.  FP64: factors of S_ee to n_b eps (1e-12 leaves
+    a factor of several hundred for pivot growth and the inverted triangles).  Mixed: S_ee comes
+    from TF32 products (10-bit mantissas, 2^-11 relative per term), so 2e-3 of ||S|| ||z||."""
+    from paper_1911_02366_gb300 import sc
+    n = 2
+    Q, dt, p, ctx = case(n, N, cfl=10.0, precision=sc.SC_PREC_MIXED if arm == "mixed" else sc.SC_PREC_FP64)
+    ctx.sc_set_state(Q, Q)
+    ctx.sc_assemble()
+    ctx.sc_condense()
+    K, _, _, nb = ctx.sc_sizes()
+    v = np.random.default_rng(N).standard_normal(K * nb)
+    zt = torch.zeros(K * nb, dtype=torch.float64, device="cuda")
+    ctx.sc_precond_apply(torch.tensor(v, device="cuda"), zt)
+    z = zt.cpu().numpy()
+    tol = 1e-12 if arm == "fp64" else 2e-3
+    for e in (0, K - 1):
+        S = _schur_block(ctx, e, N)
+        ze, ve = z[e * nb:(e + 1) * nb], v[e * nb:(e + 1) * nb]
+        r = np.abs(S @ ze - ve).max()
+        assert r <= tol * (np.abs(S).sum(axis=1).max() * np.abs(ze).max() + np.abs(ve).max()), (e, r)
