@@ -239,7 +239,8 @@ sc_status sc_condensed_matvec(sc_ctx* ctx, const double* xb, double* yb);
    the call allocates nothing: the vectors that link the passes (the interior vector, and
    on the mixed arm the FP32 copy of xb) are kept in a fixed 8 MiB device array compiled
    into the library (held on every GPU that loads the library until the process exits)
-   instead of context-owned memory.  The paper has no counterpart.  It is for callers that
+   instead of context-owned memory (only the interior right-hand sides between the two
+   kernels of a split interior pass are the context's, allocated with the mesh).  The paper has no counterpart.  It is for callers that
    must not allocate device memory at the point of the call, e.g. a solver loop running
    under a memory pool or an allocator that forbids cudaMalloc/cudaFree once the
    simulation is running.

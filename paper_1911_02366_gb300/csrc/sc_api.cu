@@ -92,10 +92,10 @@ void free_all(sc_ctx* c) {
   sc::free_direct_factors(c);
   double** dps[] = {&c->Q, &c->Qh, &c->grad, &c->F, &c->B, &c->NJ, &c->RJ, &c->Aown, &c->X, &c->Ainv,
                     &c->Ytmp, &c->See, &c->V, &c->Wv, &c->Zv, &c->Xb, &c->Gb, &c->Rb, &c->Ui, &c->Tb,
-                    &c->Hd, &c->partial, &c->Xfull, &c->Rfull, &c->Cross, &c->Apk, &c->Sls, &c->dQn,
+                    &c->Hd, &c->partial, &c->Xfull, &c->Rfull, &c->Apk, &c->Sls, &c->dQn,
                     &c->OV, &c->OZ, &c->gloc, &c->NJL};
   for (auto p : dps) { if (*p) cudaFree(*p); *p = nullptr; }
-  float** fps[] = {&c->Aown32, &c->X32, &c->Ainv32, &c->Y32, &c->See32, &c->Zf, &c->Xbf, &c->Uf, &c->Cross32,
+  float** fps[] = {&c->Aown32, &c->Ainv32, &c->Y32, &c->See32, &c->Zf, &c->Xbf, &c->Uf,
                    &c->Apk32, &c->Sls32, &c->Sdiag, &c->Cpl, &c->Feat, &c->Snorm, &c->Ynet, &c->Hbuf,
                    &c->Ck, &c->Wbias, &c->ExIb, &c->ExBi, &c->ExY, &c->ExW, &c->Zrb, &c->SeeB, &c->SeeL, &c->SlsL,
                    &c->Zinv};
@@ -108,6 +108,8 @@ void free_all(sc_ctx* c) {
   if (c->gj_scale) cudaFree(c->gj_scale);
   c->gj_scale = nullptr;
   c->packed = false;
+  if (c->row_t) cudaFree(c->row_t);
+  c->row_t = nullptr;
   if (c->tri_x) cudaFree(c->tri_x);
   c->tri_x = nullptr;
   c->ls_full = c->black_full = c->zinv_ready = false;
@@ -118,8 +120,8 @@ void free_all(sc_ctx* c) {
   c->Wbf16 = nullptr;
   c->Sdiag_valid = c->weights_set = c->learned_on = false;
   int** ips[] = {&c->d_nbr, &c->d_perm, &c->d_iperm, &c->d_own_pairs, &c->d_prow, &c->d_pslot, &c->d_pcol, &c->d_pptr,
-                 &c->d_pinfo, &c->piv, &c->rowperm, &c->d_status, &c->d_pk_lptr, &c->d_pk_list,
-                 &c->d_pk_row_off, &c->d_pk_pos, &c->d_pk_nint, &c->d_lface, &c->d_lmirror, &c->d_ex_nbpos, &c->d_ex_face_idx,
+                 &c->d_pinfo, &c->piv, &c->rowperm, &c->d_status, &c->d_pk_node,
+                 &c->d_pk_own_code, &c->d_pk_cross_code, &c->d_lface, &c->d_lmirror, &c->d_ex_nbpos, &c->d_ex_face_idx,
                  &c->d_colour, &c->pivL, &c->rowpermL, &c->d_lnfaces, &c->d_lface3, &c->d_lmirror3,
                  &c->d_lrslot3, &c->d_redidx, &c->d_face_tab};
   for (auto p : ips) { if (*p) cudaFree(*p); *p = nullptr; }
@@ -347,12 +349,11 @@ sc_status sc_set_mesh(sc_ctx* c, int n, double L, int N) {
   if (G.visc_flux == SC_VISC_SIPG) { A(dalloc(&c->gloc, nodes * 15)); A(dalloc(&c->NJL, nodes * 375)); }
   A(dalloc(&c->Aown, (size_t)G.K * own_stride(G))); A(dalloc(&c->X, (size_t)G.K * G.NP * 25));
   if (c->cfg.precision == SC_PREC_MIXED) {
-    A(dalloc(&c->Aown32, (size_t)G.K * own_stride(G))); A(dalloc(&c->X32, (size_t)G.K * G.NP * 25));
+    A(dalloc(&c->Aown32, (size_t)G.K * own_stride(G)));
     A(dalloc(&c->Ainv32, (size_t)G.K * G.ni * G.ldi)); A(dalloc(&c->Y32, (size_t)G.K * G.nb * G.ldi));  // Y^T (nb x ldi) on the tensor-core path
     if (c->cfg.interior_fp64 && G.ni > sc::kGjRegRows) A(dalloc(&c->Ainv, (size_t)G.K * G.ni * G.ldi));  // FP64 A_ii^-1
     A(dalloc(&c->See32, (size_t)G.K * G.nb * G.lds)); A(dalloc(&c->Dfull, dofs));
     A(dalloc(&c->Zf, n1)); A(dalloc(&c->Xbf, n1)); A(dalloc(&c->Uf, (size_t)G.K * G.ni));
-    A(dalloc(&c->Cross32, n1 + (size_t)G.K * G.ni));
     if (c->cfg.outer_krylov > 0) {
       A(dalloc(&c->OV, dofs * (size_t)(c->cfg.outer_krylov + 1))); A(dalloc(&c->OZ, dofs * (size_t)c->cfg.outer_krylov));
     }
@@ -361,7 +362,7 @@ sc_status sc_set_mesh(sc_ctx* c, int n, double L, int N) {
     A(dalloc(&c->See, (size_t)G.K * G.nb * G.lds));
   }
   A(dalloc(&c->piv, (size_t)G.K * G.nb)); A(dalloc(&c->rowperm, (size_t)G.K * G.nb));
-  A(dalloc(&c->Cross, n1 + (size_t)G.K * G.ni));
+  A(cudaMalloc(&c->row_t, (size_t)G.K * G.ldi * (c->cfg.precision == SC_PREC_MIXED ? sizeof(float) : sizeof(double))));
   A(dalloc(&c->V, n1 * (m + 1))); A(dalloc(&c->Wv, n1)); A(dalloc(&c->Zv, n1)); A(dalloc(&c->Xb, n1));
   A(dalloc(&c->Gb, n1)); A(dalloc(&c->Rb, n1)); A(dalloc(&c->Tb, n1));
   A(dalloc(&c->Ui, (size_t)G.K * G.ni)); A(dalloc(&c->Hd, 3 * (size_t)(m + 2) + 16));
@@ -374,9 +375,8 @@ sc_status sc_set_mesh(sc_ctx* c, int n, double L, int N) {
   const int np = G.NP;
   A(dalloc(&c->d_prow, np)); A(dalloc(&c->d_pslot, np)); A(dalloc(&c->d_pcol, np));
   A(dalloc(&c->d_pptr, G.nn + 1)); A(dalloc(&c->d_pinfo, np));
-  A(dalloc(&c->d_pk_lptr, c->pk_lptr.size())); A(dalloc(&c->d_pk_list, c->pk_list.size()));
-  A(dalloc(&c->d_pk_row_off, c->pk_row_off.size())); A(dalloc(&c->d_pk_pos, c->pk_pos.size()));
-  A(dalloc(&c->d_pk_nint, c->pk_nint.size()));
+  A(dalloc(&c->d_pk_node, c->pk_node.size())); A(dalloc(&c->d_pk_own_code, c->pk_own_code.size()));
+  A(dalloc(&c->d_pk_cross_code, c->pk_cross_code.size()));
   A(dalloc(&c->d_lface, G.nbn)); A(dalloc(&c->d_lmirror, G.nbn)); A(dalloc(&c->d_lnfaces, G.nbn));
   A(dalloc(&c->d_lface3, 3 * (size_t)G.nbn)); A(dalloc(&c->d_lmirror3, 3 * (size_t)G.nbn));
   A(dalloc(&c->d_lrslot3, 3 * (size_t)G.nbn));
@@ -456,9 +456,7 @@ sc_status sc_set_mesh(sc_ctx* c, int n, double L, int N) {
     SC_CUDA(cudaMemcpy(c->d_redidx, c->red_index.data(), (size_t)G.K * sizeof(int), cudaMemcpyHostToDevice));
     SC_CUDA(cudaMemcpy(c->d_face_tab, c->face_tab.data(), c->face_tab.size() * sizeof(int), cudaMemcpyHostToDevice));
   }
-  // the alignment padding of the element blocks (dense and packed) must read as zero
-  if (c->Apk) SC_CUDA(cudaMemset(c->Apk, 0, (size_t)G.K * c->pk_stride * sizeof(double)));
-  if (c->Apk32) SC_CUDA(cudaMemset(c->Apk32, 0, (size_t)G.K * c->pk_stride * sizeof(float)));
+  // the alignment padding of the dense element blocks must read as zero (packing writes its own)
   SC_CUDA(cudaMemset(c->Aown, 0, (size_t)G.K * own_stride(G) * sizeof(double)));
   if (c->Ainv) SC_CUDA(cudaMemset(c->Ainv, 0, (size_t)G.K * G.ni * G.ldi * sizeof(double)));
   if (c->Ainv32) SC_CUDA(cudaMemset(c->Ainv32, 0, (size_t)G.K * G.ni * G.ldi * sizeof(float)));

@@ -1560,9 +1560,6 @@ cudaError_t launch_condense(sc_ctx* c) {
   if (pe != cudaSuccess) return pe;
   c->packed = true;
   if (c->cfg.precision == SC_PREC_MIXED) {  // the packing pass wrote the FP32 own blocks
-    count_launch(c);
-    const size_t nx = (size_t)G.K * G.NP * 25;
-    k_to_float<<<608, 256, 0, c->stream>>>(c->X, c->X32, nx);
     bool have_inv = false;
     if (c->cfg.interior_fp64 && c->Ainv && G.ni > GJR_N) {
       // A_ii^-1 in FP64 from the FP64 own blocks, rounded to FP32 for the operator
@@ -1737,12 +1734,6 @@ cudaError_t grouped_finish(cudaStream_t st, const CondItem* items, const std::ve
     i = k;
   }
   return e;
-}
-
-cudaError_t to_float(sc_ctx* c, const double* a, float* b, size_t n) {
-  count_launch(c);
-  k_to_float<<<608, 256, 0, c->stream>>>(a, b, n);
-  return cudaGetLastError();
 }
 
 // C = A B for `batch` row-major FP32 blocks on the CUDA cores.

@@ -19,7 +19,7 @@ namespace {
 
 // A_ib[e_int, E_e] (ni x ldm) and A_bi[E_e, e_int] (m x ldi) from the own block and the
 // neighbour couplings.  Buffers are zero on entry.
-__global__ void __launch_bounds__(256) k_gather_ext(Geo G, const float* __restrict__ Aown, const float* __restrict__ X,
+__global__ void __launch_bounds__(256) k_gather_ext(Geo G, const float* __restrict__ Aown, const double* __restrict__ X,
     const int* __restrict__ nbr, const int* __restrict__ pptr, const int* __restrict__ pinfo,
     const int* __restrict__ iperm, const int* __restrict__ ex_nbpos, const int* __restrict__ ex_face_idx, int F,
     int ldm, float* __restrict__ Aib, float* __restrict__ Abi, int* __restrict__ status) {
@@ -47,10 +47,10 @@ __global__ void __launch_bounds__(256) k_gather_ext(Geo G, const float* __restri
       int i = -1;
       if (slot < 6) i = __ldg(ex_face_idx + slot * nbn + pinfo_offset(info) / 5);
       if (i < 0) { atomicCAS(status, -1, SC_EXPLICIT_PATTERN); continue; }
-      const float* Xq = X + ((size_t)e * 5 * G.NP + q) * 5;
+      const double* Xq = X + ((size_t)e * 5 * G.NP + q) * 5;
       for (int kv = 0; kv < 5; ++kv)
         for (int l = 0; l < 5; ++l)
-          Ib[(size_t)(5 * pi + kv) * ldm + nb + slot * 5 * F + 5 * i + l] = __ldg(Xq + kv * xs + l);
+          Ib[(size_t)(5 * pi + kv) * ldm + nb + slot * 5 * F + 5 * i + l] = (float)__ldg(Xq + kv * xs + l);
     }
   }
   // face dofs of each neighbour -> interior of e (from the neighbour's couplings)
@@ -63,10 +63,10 @@ __global__ void __launch_bounds__(256) k_gather_ext(Geo G, const float* __restri
         const int info = __ldg(pinfo + q);
         if (!pinfo_interior(info) || pinfo_slot(info) != fb) continue;
         const int off = pinfo_offset(info);
-        const float* Xq = X + ((size_t)n * 5 * G.NP + q) * 5;
+        const double* Xq = X + ((size_t)n * 5 * G.NP + q) * 5;
         for (int kv = 0; kv < 5; ++kv)
           for (int l = 0; l < 5; ++l)
-            Bi[(size_t)(nb + f * 5 * F + 5 * i + kv) * G.ldi + off + l] = __ldg(Xq + kv * xs + l);
+            Bi[(size_t)(nb + f * 5 * F + 5 * i + kv) * G.ldi + off + l] = (float)__ldg(Xq + kv * xs + l);
       }
     }
   }
@@ -175,7 +175,7 @@ cudaError_t explicit_build(sc_ctx* c) {
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ExBi, 0, (size_t)K * m * G.ldi * sizeof(float), c->stream);
   if (e != cudaSuccess) return e;
   count_launch(c);
-  k_gather_ext<<<K, 256, 0, c->stream>>>(G, c->Aown32, c->X32, c->d_nbr, c->d_pptr, c->d_pinfo, c->d_iperm,
+  k_gather_ext<<<K, 256, 0, c->stream>>>(G, c->Aown32, c->X, c->d_nbr, c->d_pptr, c->d_pinfo, c->d_iperm,
                                          c->d_ex_nbpos, c->d_ex_face_idx, c->ex_F, ldm, c->ExIb, c->ExBi,
                                          c->d_status);
   e = cudaGetLastError();
@@ -202,7 +202,7 @@ cudaError_t explicit_build(sc_ctx* c) {
 // couplings), then the W_e products subtracted at the extended dofs.
 cudaError_t explicit_matvec32(sc_ctx* c, const float* x, double* y) {
   const Geo& G = c->G;
-  cudaError_t e = cond_boundary_pk<float>(c, c->Apk32, c->X32, x, 1.0, nullptr, 0.0, nullptr, y);
+  cudaError_t e = cond_boundary_pk<float>(c, c->Apk32, x, 1.0, nullptr, 0.0, nullptr, y);
   if (e != cudaSuccess) return e;
   ProfScope ps(c, SCK_EXPLICIT_APPLY);
   const size_t smem = (size_t)c->ex_ldm * sizeof(float);

@@ -301,18 +301,16 @@ struct sc_ctx {
   double *Ui = nullptr, *Tb = nullptr, *Hd = nullptr, *partial = nullptr, *Xfull = nullptr, *Rfull = nullptr;
   int restart_alloc = 0;
   // mixed-precision arm: FP32 copies of the element blocks and FP32 condensation
-  float *Aown32 = nullptr, *X32 = nullptr, *Ainv32 = nullptr, *Y32 = nullptr, *See32 = nullptr;
+  float *Aown32 = nullptr, *Ainv32 = nullptr, *Y32 = nullptr, *See32 = nullptr;
   float *Zf = nullptr, *Xbf = nullptr, *Uf = nullptr;  // FP32 vectors of the FP32 operator
-  double* Cross = nullptr;   // neighbour-coupling products of one pass, FP64 operator
-  float* Cross32 = nullptr;  // same, FP32 operator
+  void* row_t = nullptr;     // interior right-hand sides between the steps of a split interior pass (K x ldi)
   double* Dfull = nullptr;  // refinement correction
   double* dQn = nullptr;    // Newton update of sc_newton_step
   // pattern-packed own blocks of the condensed operator (A_ib rows, [A_bi A_bb] rows)
-  std::vector<int> pk_lptr, pk_list, pk_pos, pk_row_off;
-  std::vector<int> pk_nint;  // per node slot: packed entries of its rows in interior columns (listed first)
+  // and the couplings: per node slot 8 ints (sc_packed.cu, PkNode), codes of the rows' entries
+  std::vector<int> pk_node, pk_own_code, pk_cross_code;
   long long pk_stride = 0, pk_nnz_int = 0, pk_nnz_bnd = 0;
-  int *d_pk_lptr = nullptr, *d_pk_list = nullptr, *d_pk_row_off = nullptr, *d_pk_pos = nullptr;
-  int* d_pk_nint = nullptr;
+  int *d_pk_node = nullptr, *d_pk_own_code = nullptr, *d_pk_cross_code = nullptr;
   double* Apk = nullptr;   // FP64 arm
   float* Apk32 = nullptr;  // mixed arm
   // S_ee factors with partitioned inverses in the block-Jacobi solve layout
@@ -503,7 +501,6 @@ cudaError_t grouped_copy_bb(cudaStream_t st, const CondItem* items, int n);
 cudaError_t grouped_lu_panel(cudaStream_t st, const CondItem* items, int n, int nbig, int k0, int max_nb);
 // host: the same items; returns the launches made in *launches
 cudaError_t grouped_finish(cudaStream_t st, const CondItem* items, const std::vector<CondItem>& host, int* launches);
-cudaError_t to_float(sc_ctx* c, const double* a, float* b, size_t n);
 cudaError_t gemm_tf32_ptrs(cudaStream_t stream, int M, int N, int K, float alpha, const float* const* Ap, int lda,
                            bool ta, const float* const* Bp, int ldb, bool tb, float beta, float* const* Cp, int ldc,
                            int batch, int bn, int* status);
@@ -522,13 +519,13 @@ cudaError_t mlp_forward(cudaStream_t st, const uint16_t* Wbf16, const float* bia
 cudaError_t upload_packed_pattern(sc_ctx* c);
 cudaError_t pack_own(sc_ctx* c);
 template <class T>
-cudaError_t cond_interior_pk(sc_ctx* c, const T* Apk, const T* X, const T* Ainv, const T* xb, double beta,
-                             const double* Bfull, double alpha, T* u, int black_zero);
+cudaError_t cond_interior_pk(sc_ctx* c, const T* Apk, const T* Ainv, const T* xb, double beta, const double* Bfull,
+                             double alpha, T* u, int black_zero);
 cudaError_t cond_interior_sweep(sc_ctx* c, const double* xb, double* u);
 cudaError_t cond_interior_sweep32(sc_ctx* c, const float* xb, float* u);
 template <class T>
-cudaError_t cond_boundary_pk(sc_ctx* c, const T* Apk, const T* X, const T* xb, double delta, const double* Bfull,
-                             double gamma_, const T* u, double* y);
+cudaError_t cond_boundary_pk(sc_ctx* c, const T* Apk, const T* xb, double delta, const double* Bfull, double gamma_,
+                             const T* u, double* y);
 cudaError_t vec_axpby(sc_ctx* c, double* y, double a, const double* x, double b, size_t n);
 // block solves of a list of elements (factors by element, or compact by list position), vsub
 // subtracted from the right-hand side
@@ -538,8 +535,8 @@ cudaError_t lu_solve_list(sc_ctx* c, const double* LS, const int* rowperm, int c
 cudaError_t lu_solve_list32(sc_ctx* c, const float* LS, const int* rowperm, int compact, bool full, const int* elist,
                             int nlist, const double* v, const double* vsub, double* z, float* zt);
 template <class T>
-cudaError_t cond_boundary_pk_list(sc_ctx* c, const T* Apk, const T* X, const T* xb, const T* u, double* y,
-                                  const int* elist, int nlist);
+cudaError_t cond_boundary_pk_list(sc_ctx* c, const T* Apk, const T* xb, const T* u, double* y, const int* elist,
+                                  int nlist);
 // red-black sweep (precond SC_PC_RED_BLACK, or SC_PC_LEARNED while the learned correction is on)
 void build_colours(sc_ctx* c);
 bool rb_active(const sc_ctx* c);

@@ -5,9 +5,9 @@
 // passes do it:
 //   interior pass   u_e = A_ii,e^-1 ( alpha B_i,e + beta (A_ib x_b)_e )
 //   boundary pass   y_e = gamma B_b,e + delta (A_bb x_b)_e - (A_bi u)_e
-// where the own-element parts are dense row-major GEMVs on the stored element block and
-// the neighbour parts run over the structured coupling list.  The same two passes give
-// the condensed right-hand side (x_b = 0) and the back-substitution of eq. SC_step2.
+// from the pattern-packed rows of sc_packed.cu (own entries and neighbour couplings).  The same
+// two passes give the condensed right-hand side (x_b = 0) and the back-substitution of eq.
+// SC_step2.
 #include "sc_internal.cuh"
 
 namespace {
@@ -17,219 +17,21 @@ __device__ __forceinline__ double warp_sum(double s) {
   return s;
 }
 
-// 16-byte vector type of each storage precision.
-template <class T> struct Vec16;
-template <> struct Vec16<double> { using type = double2; static constexpr int n = 2; };
-template <> struct Vec16<float> { using type = float4; static constexpr int n = 4; };
-
 __device__ __forceinline__ void fma16(const double2& a, const double2& b, double& s0, double& s1) {
   s0 = fma(a.x, b.x, s0); s1 = fma(a.y, b.y, s1);
 }
-__device__ __forceinline__ void fma16(const float4& a, const float4& b, float& s0, float& s1) {
-  s0 = fmaf(a.x, b.x, s0); s1 = fmaf(a.y, b.y, s1); s0 = fmaf(a.z, b.z, s0); s1 = fmaf(a.w, b.w, s1);
-}
 
-// Dot product of a row segment (global, 16-byte aligned) with a vector in shared memory
-// (16-byte aligned), one warp, 16-byte loads, arithmetic in the storage precision T;
-// returns this lane's partial sum.
-template <class T>
-__device__ __forceinline__ T warp_dot(const T* __restrict__ row, const T* v, int len, int lane) {
-  using V = typename Vec16<T>::type;
-  constexpr int W = Vec16<T>::n;
-  const V* r = reinterpret_cast<const V*>(row);
-  const V* x = reinterpret_cast<const V*>(v);
-  const int nv = len / W;
-  T s0 = T(0), s1 = T(0);
+// Dot product of a row segment (global, 16-byte aligned) with a vector in shared memory (16-byte
+// aligned), one warp, 16-byte loads; returns this lane's partial sum.
+__device__ __forceinline__ double warp_dot(const double* __restrict__ row, const double* v, int len, int lane) {
+  const double2* r = reinterpret_cast<const double2*>(row);
+  const double2* x = reinterpret_cast<const double2*>(v);
+  const int nv = len / 2;
+  double s0 = 0.0, s1 = 0.0;
 #pragma unroll 4
   for (int i = lane; i < nv; i += 32) fma16(__ldg(r + i), x[i], s0, s1);
-  for (int i = nv * W + lane; i < len; i += 32) s0 = fma(__ldg(row + i), v[i], s0);
+  for (int i = nv * 2 + lane; i < len; i += 32) s0 = fma(__ldg(row + i), v[i], s0);
   return s0 + s1;
-}
-
-__device__ __forceinline__ float warp_sum(float s) {
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  return s;
-}
-
-// Two row dots at once (independent loads in flight): lane partial sums of
-// rowA . v and rowB . v over len entries.
-template <class T>
-__device__ __forceinline__ void warp_dot2(const T* __restrict__ rowA, const T* __restrict__ rowB, const T* v, int len,
-                                          int lane, T& sa, T& sb) {
-  using V = typename Vec16<T>::type;
-  constexpr int W = Vec16<T>::n;
-  const V* ra = reinterpret_cast<const V*>(rowA);
-  const V* rb = reinterpret_cast<const V*>(rowB);
-  const V* x = reinterpret_cast<const V*>(v);
-  const int nv = len / W;
-  T a0 = T(0), a1 = T(0), b0 = T(0), b1 = T(0);
-#pragma unroll 2
-  for (int i = lane; i < nv; i += 32) {
-    const V xa = x[i];
-    fma16(__ldg(ra + i), xa, a0, a1);
-    fma16(__ldg(rb + i), xa, b0, b1);
-  }
-  for (int i = nv * W + lane; i < len; i += 32) { a0 = fma(__ldg(rowA + i), v[i], a0); b0 = fma(__ldg(rowB + i), v[i], b0); }
-  sa = a0 + a1; sb = b0 + b1;
-}
-
-// Neighbour couplings of row (node j, variable k) of element e.  The couplings of one
-// row are contiguous in X (layout X[e][k][pair][l]); vb / vi are the condensed
-// boundary / interior vectors of all elements in the storage precision T (either may
-// be null), scaled by cb / ci.
-template <class T>
-__device__ __forceinline__ T cross_row(const Geo& G, int e, int j, int k, const T* __restrict__ X,
-                                       const int* nbr_s, const int* __restrict__ pptr,
-                                       const int* __restrict__ pinfo, const T* __restrict__ vb, T cb,
-                                       const T* __restrict__ vi, T ci, int lane) {
-  const int q0 = __ldg(pptr + j), q1 = __ldg(pptr + j + 1);
-  const T* Xr = X + (((size_t)e * 5 + k) * G.NP + q0) * 5;
-  T s = T(0);
-  for (int f = lane; f < 5 * (q1 - q0); f += 32) {
-    const int q = q0 + f / 5, l = f % 5;
-    const int info = __ldg(pinfo + q);
-    const int nb = nbr_s[pinfo_slot(info)];
-    const int off = pinfo_offset(info) + l;
-    T xv;
-    if (pinfo_interior(info)) {
-      if (!vi) continue;
-      xv = ci * vi[(size_t)nb * G.ni + off];
-    } else {
-      if (!vb) continue;
-      xv = cb * vb[(size_t)nb * G.nb + off];
-    }
-    s = fma(__ldg(Xr + f), xv, s);
-  }
-  return s;
-}
-
-// Neighbour couplings of a set of rows, one thread per (element, row): rows are the
-// permuted positions [row0, row0 + nrows) of every element; out[e][r - row0] =
-// sum over the row's couplings of X * (cb x_b or ci v_i) of the neighbour.
-template <class T>
-__global__ void __launch_bounds__(256) k_cross_rows(Geo G, const T* __restrict__ X, const int* __restrict__ nbr,
-    const int* __restrict__ pptr, const int* __restrict__ pinfo, const int* __restrict__ iperm, int row0, int nrows,
-    const T* __restrict__ vb, T cb, const T* __restrict__ vi, T ci, T* __restrict__ out) {
-  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (t >= (size_t)G.K * nrows) return;
-  const int e = (int)(t / nrows), r = row0 + (int)(t % nrows);
-  const int j = __ldg(iperm + r / 5), k = r % 5;
-  const int q0 = __ldg(pptr + j), q1 = __ldg(pptr + j + 1);
-  const T* Xr = X + (((size_t)e * 5 + k) * G.NP + q0) * 5;
-  const int* nb_e = nbr + e * 18;
-  T s = T(0);
-  for (int q = q0; q < q1; ++q) {
-    const int info = __ldg(pinfo + q);
-    const int nb = __ldg(nb_e + pinfo_slot(info));
-    const int off = pinfo_offset(info);
-    const T* vec;
-    T coef;
-    if (pinfo_interior(info)) { vec = vi ? vi + (size_t)nb * G.ni + off : nullptr; coef = ci; }
-    else { vec = vb ? vb + (size_t)nb * G.nb + off : nullptr; coef = cb; }
-    if (!vec) continue;
-    const T* xq = Xr + (q - q0) * 5;
-    T a = T(0);
-#pragma unroll
-    for (int l = 0; l < 5; ++l) a = fma(__ldg(xq + l), vec[l], a);
-    s = fma(coef, a, s);
-  }
-  out[t] = s;
-}
-
-// Interior pass: u_e = A_ii,e^-1 (alpha B_i,e + beta (A_ib x_b)_e).  Matrices and the
-// vectors x_b, u in precision T; the full right-hand side B in double.
-template <class T>
-__global__ void __launch_bounds__(256) k_cond_interior(Geo G, const T* __restrict__ Aown,
-    const T* __restrict__ X, const T* __restrict__ Ainv, const int* __restrict__ nbr,
-    const int* __restrict__ pptr, const int* __restrict__ pinfo, const int* __restrict__ iperm,
-    const T* __restrict__ xb, double beta, const double* __restrict__ Bfull, double alpha,
-    T* __restrict__ u, const T* __restrict__ cross) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int e = blockIdx.x, ni = G.ni, nb = G.nb;
-  T* v = reinterpret_cast<T*>(smem_raw);  // nb: x_e
-  T* t = v + ((nb + 3) & ~3);             // ldi: right-hand side of the interior solve, zero padded,
-                                          // 16-byte aligned for the vector loads of warp_dot
-  __shared__ int nbr_s[18];
-  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, nw = blockDim.x / 32;
-  if (threadIdx.x < 18) nbr_s[threadIdx.x] = nbr[e * 18 + threadIdx.x];
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) v[i] = xb ? xb[(size_t)e * nb + i] : T(0);
-  for (int i = ni + threadIdx.x; i < G.ldi; i += blockDim.x) t[i] = T(0);
-  __syncthreads();
-  const T* Ae = Aown + (size_t)e * own_stride(G);
-  for (int ri = warp; ri < ni; ri += nw) {
-    const int j = __ldg(iperm + ri / 5), k = ri % 5;
-    T s = T(0);
-    if (xb) {
-      s = warp_dot(Ae + (size_t)ri * G.lda + G.cb0, v, nb, lane);
-      if (!cross) s += cross_row(G, e, j, k, X, nbr_s, pptr, pinfo, xb, T(1), (const T*)nullptr, T(0), lane);
-      s = warp_sum(s);
-      if (cross) s += cross[(size_t)e * ni + ri];
-    }
-    if (lane == 0) {
-      T val = T(beta) * s;
-      if (Bfull) val += T(alpha * Bfull[((size_t)e * G.nn + j) * 5 + k]);
-      t[ri] = val;
-    }
-  }
-  __syncthreads();
-  const T* Ie = Ainv + (size_t)e * ni * G.ldi;
-  for (int ri = 2 * warp; ri < ni; ri += 2 * nw) {
-    const bool two = ri + 1 < ni;
-    T sa, sb;
-    warp_dot2(Ie + (size_t)ri * G.ldi, Ie + (size_t)(two ? ri + 1 : ri) * G.ldi, t, G.ldi, lane, sa, sb);
-    sa = warp_sum(sa); sb = warp_sum(sb);
-    if (lane == 0) {
-      u[(size_t)e * ni + ri] = sa;
-      if (two) u[(size_t)e * ni + ri + 1] = sb;
-    }
-  }
-}
-
-// Boundary pass: y_e = gamma B_b,e + delta (A_bb x_b)_e - (A_bi u)_e.  Matrices and x_b, u
-// in precision T; B and y in double.
-template <class T>
-__global__ void __launch_bounds__(256) k_cond_boundary(Geo G, const T* __restrict__ Aown,
-    const T* __restrict__ X, const int* __restrict__ nbr,
-    const int* __restrict__ pptr, const int* __restrict__ pinfo, const int* __restrict__ iperm,
-    const T* __restrict__ xb, double delta, const double* __restrict__ Bfull, double gamma_,
-    const T* __restrict__ u, double* __restrict__ y, const T* __restrict__ cross) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int e = blockIdx.x, ni = G.ni, nb = G.nb, ne = G.ne, lda = G.lda, cb0 = G.cb0;
-  T* v = reinterpret_cast<T*>(smem_raw);  // lda: [-u_e | 0 | delta x_e | 0] in own-column order
-  __shared__ int nbr_s[18];
-  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, nw = blockDim.x / 32;
-  const T dT = T(delta);
-  if (threadIdx.x < 18) nbr_s[threadIdx.x] = nbr[e * 18 + threadIdx.x];
-  for (int i = threadIdx.x; i < lda; i += blockDim.x) {
-    T val = T(0);
-    if (i < ni) { if (u) val = -u[(size_t)e * ni + i]; }
-    else if (i >= cb0 && i < cb0 + nb) { if (xb) val = dT * xb[(size_t)e * nb + i - cb0]; }
-    v[i] = val;
-  }
-  __syncthreads();
-  const T* Ae = Aown + (size_t)e * own_stride(G);
-  const int c0 = u ? 0 : cb0;                 // skip the A_bi columns when u is absent
-  const int len = (xb ? cb0 + nb : ni) - c0;  // and the A_bb columns when x_b is absent
-  for (int ra = ni + 2 * warp; ra < ne; ra += 2 * nw) {
-    const int rb2 = ra + 1 < ne ? ra + 1 : ra;
-    T sa = T(0), sb = T(0);
-    if (xb || u) warp_dot2(Ae + (size_t)ra * lda + c0, Ae + (size_t)rb2 * lda + c0, v + c0, len, lane, sa, sb);
-    if (!cross) {
-      sa += cross_row(G, e, __ldg(iperm + ra / 5), ra % 5, X, nbr_s, pptr, pinfo, xb, dT, u, T(-1), lane);
-      sb += cross_row(G, e, __ldg(iperm + rb2 / 5), rb2 % 5, X, nbr_s, pptr, pinfo, xb, dT, u, T(-1), lane);
-    }
-    sa = warp_sum(sa); sb = warp_sum(sb);
-    if (cross) { sa += cross[(size_t)e * nb + ra - ni]; sb += cross[(size_t)e * nb + rb2 - ni]; }
-    if (lane == 0) {
-      double va = (double)sa, vb = (double)sb;
-      if (Bfull) {
-        va += gamma_ * Bfull[((size_t)e * G.nn + __ldg(iperm + ra / 5)) * 5 + ra % 5];
-        vb += gamma_ * Bfull[((size_t)e * G.nn + __ldg(iperm + rb2 / 5)) * 5 + rb2 % 5];
-      }
-      y[(size_t)e * nb + ra - ni] = va;
-      if (rb2 != ra) y[(size_t)e * nb + rb2 - ni] = vb;
-    }
-  }
 }
 
 // y = A x on the full system, natural global dof order.
@@ -401,87 +203,43 @@ constexpr int kDotChunks = 152;
 
 namespace sc {
 
-// The condensed operator's passes: fused kernels on the pattern-packed blocks once the
-// condensation has packed them, otherwise a coupling pass followed by the dense kernels.
+// The condensed operator's passes on the pattern-packed blocks.
 template <class T>
-cudaError_t cond_interior_t(sc_ctx* c, const T* Aown, const T* Apk, const T* X, const T* Ainv, T* crossbuf,
-                            const T* xb, double beta, const double* Bfull, double alpha, T* u) {
-  const Geo& G = c->G;
-  if (G.ni == 0) return cudaSuccess;
-  if (Apk) {
-    ProfScope ps(c, SCK_COND_INTERIOR);
-    return cond_interior_pk<T>(c, Apk, X, Ainv, xb, beta, Bfull, alpha, u, 0);
-  }
-  if (xb) {
-    count_launch(c);
-    const size_t rows = (size_t)G.K * G.ni;
-    k_cross_rows<T><<<(unsigned)((rows + 255) / 256), 256, 0, c->stream>>>(G, X, c->d_nbr, c->d_pptr, c->d_pinfo,
-        c->d_iperm, 0, G.ni, xb, T(1), (const T*)nullptr, T(0), crossbuf);
-  }
+cudaError_t cond_interior_t(sc_ctx* c, const T* Apk, const T* Ainv, const T* xb, double beta, const double* Bfull,
+                            double alpha, T* u, int black_zero) {
+  if (c->G.ni == 0) return cudaSuccess;
   ProfScope ps(c, SCK_COND_INTERIOR);
-  const size_t smem = (size_t)(((G.nb + 3) & ~3) + G.ldi) * sizeof(T);
-  k_cond_interior<T><<<G.K, 256, smem, c->stream>>>(G, Aown, X, Ainv, c->d_nbr, c->d_pptr, c->d_pinfo, c->d_iperm,
-                                                    xb, beta, Bfull, alpha, u, xb ? crossbuf : (const T*)nullptr);
-  return cudaGetLastError();
-}
-
-template <class T>
-cudaError_t cond_boundary_t(sc_ctx* c, const T* Aown, const T* Apk, const T* X, T* crossbuf, const T* xb,
-                            double delta, const double* Bfull, double gamma_, const T* u, double* y) {
-  const Geo& G = c->G;
-  if (G.ni == 0) u = nullptr;
-  if (Apk) {
-    ProfScope ps(c, SCK_COND_BOUNDARY);
-    return cond_boundary_pk<T>(c, Apk, X, xb, delta, Bfull, gamma_, u, y);
-  }
-  const bool need = xb || u;
-  if (need) {
-    count_launch(c);
-    const size_t rows = (size_t)G.K * G.nb;
-    k_cross_rows<T><<<(unsigned)((rows + 255) / 256), 256, 0, c->stream>>>(G, X, c->d_nbr, c->d_pptr, c->d_pinfo,
-        c->d_iperm, G.ni, G.nb, xb, T(delta), u, T(-1), crossbuf);
-  }
-  ProfScope ps(c, SCK_COND_BOUNDARY);
-  const size_t smem = (size_t)G.lda * sizeof(T);
-  k_cond_boundary<T><<<G.K, 256, smem, c->stream>>>(G, Aown, X, c->d_nbr, c->d_pptr, c->d_pinfo, c->d_iperm, xb,
-                                                    delta, Bfull, gamma_, u, y, need ? crossbuf : (const T*)nullptr);
-  return cudaGetLastError();
+  return cond_interior_pk<T>(c, Apk, Ainv, xb, beta, Bfull, alpha, u, black_zero);
 }
 
 cudaError_t cond_interior(sc_ctx* c, const double* xb, double beta, const double* Bfull, double alpha, double* u) {
-  return cond_interior_t<double>(c, c->Aown, c->packed ? c->Apk : nullptr, c->X, c->Ainv, c->Cross, xb, beta, Bfull,
-                                 alpha, u);
+  return cond_interior_t<double>(c, c->Apk, c->Ainv, xb, beta, Bfull, alpha, u, 0);
 }
 
 cudaError_t cond_boundary(sc_ctx* c, const double* xb, double delta, const double* Bfull, double gamma_,
                           const double* u, double* y) {
-  return cond_boundary_t<double>(c, c->Aown, c->packed ? c->Apk : nullptr, c->X, c->Cross, xb, delta, Bfull, gamma_,
-                                 u, y);
+  ProfScope ps(c, SCK_COND_BOUNDARY);
+  return cond_boundary_pk<double>(c, c->Apk, xb, delta, Bfull, gamma_, u, y);
 }
 
 cudaError_t cond_interior32(sc_ctx* c, const float* xb, double beta, const double* Bfull, double alpha, float* u) {
-  return cond_interior_t<float>(c, c->Aown32, c->packed ? c->Apk32 : nullptr, c->X32, c->Ainv32, c->Cross32, xb, beta,
-                                Bfull, alpha, u);
+  return cond_interior_t<float>(c, c->Apk32, c->Ainv32, xb, beta, Bfull, alpha, u, 0);
 }
 
 // Interior pass of the red-black sweep: u = A_ii^-1 (A_ib x_b) with x_b zero on the black
-// elements, whose own part is then skipped (packed blocks; otherwise the general pass).
+// elements, whose own part is then skipped.
 cudaError_t cond_interior_sweep(sc_ctx* c, const double* xb, double* u) {
-  if (!c->packed || c->G.ni == 0) return cond_interior(c, xb, 1.0, nullptr, 0.0, u);
-  ProfScope ps(c, SCK_COND_INTERIOR);
-  return cond_interior_pk<double>(c, c->Apk, c->X, c->Ainv, xb, 1.0, nullptr, 0.0, u, 1);
+  return cond_interior_t<double>(c, c->Apk, c->Ainv, xb, 1.0, nullptr, 0.0, u, 1);
 }
 
 cudaError_t cond_interior_sweep32(sc_ctx* c, const float* xb, float* u) {
-  if (!c->packed || c->G.ni == 0) return cond_interior32(c, xb, 1.0, nullptr, 0.0, u);
-  ProfScope ps(c, SCK_COND_INTERIOR);
-  return cond_interior_pk<float>(c, c->Apk32, c->X32, c->Ainv32, xb, 1.0, nullptr, 0.0, u, 1);
+  return cond_interior_t<float>(c, c->Apk32, c->Ainv32, xb, 1.0, nullptr, 0.0, u, 1);
 }
 
 cudaError_t cond_boundary32(sc_ctx* c, const float* xb, double delta, const double* Bfull, double gamma_,
                             const float* u, double* y) {
-  return cond_boundary_t<float>(c, c->Aown32, c->packed ? c->Apk32 : nullptr, c->X32, c->Cross32, xb, delta, Bfull,
-                                gamma_, u, y);
+  ProfScope ps(c, SCK_COND_BOUNDARY);
+  return cond_boundary_pk<float>(c, c->Apk32, xb, delta, Bfull, gamma_, u, y);
 }
 
 cudaError_t global_apply(sc_ctx* c, const double* x, double* y) {

@@ -42,7 +42,7 @@ __global__ void k_extract_sdiag(int nb, const float* __restrict__ See, long long
 
 // S_(k,k') for every (element, boundary node): one warp per sample.
 __global__ void __launch_bounds__(256) k_learned_coupling(Geo G, const float* __restrict__ Aown, const float* __restrict__ Ainv,
-    const float* __restrict__ X, const int* __restrict__ pptr, const int* __restrict__ pinfo,
+    const double* __restrict__ X, const int* __restrict__ pptr, const int* __restrict__ pinfo,
     const int* __restrict__ iperm, const int* __restrict__ nbr, const int* __restrict__ lface3,
     const int* __restrict__ lmirror3, const int* __restrict__ nfaces, const float* __restrict__ Y, int y_transposed,
     float* __restrict__ out) {
@@ -82,13 +82,13 @@ __global__ void __launch_bounds__(256) k_learned_coupling(Geo G, const float* __
   const size_t xs = (size_t)G.NP * 5;  // X stride between row variables
   for (int h = 0; h < nh; ++h) {
     const int pi = hits[2 * h], q = hits[2 * h + 1];
-    const float* Xq = X + ((size_t)e * 5 * G.NP + q) * 5;
+    const double* Xq = X + ((size_t)e * 5 * G.NP + q) * 5;
     for (int r = lane; r < ni; r += 32) {
 #pragma unroll
       for (int kv = 0; kv < 5; ++kv) {
         const float av = Ie[(size_t)r * G.ldi + 5 * pi + kv];
 #pragma unroll
-        for (int l = 0; l < 5; ++l) t[r * 5 + l] = fmaf(av, __ldg(Xq + kv * xs + l), t[r * 5 + l]);
+        for (int l = 0; l < 5; ++l) t[r * 5 + l] = fmaf(av, (float)__ldg(Xq + kv * xs + l), t[r * 5 + l]);
       }
     }
   }
@@ -113,13 +113,13 @@ __global__ void __launch_bounds__(256) k_learned_coupling(Geo G, const float* __
     const int info = __ldg(pinfo + q);
     if (pinfo_slot(info) != f) continue;
     const int off = pinfo_offset(info);
-    const float* Xq = X + ((size_t)e * 5 * G.NP + q) * 5;
+    const double* Xq = X + ((size_t)e * 5 * G.NP + q) * 5;
     if (!pinfo_interior(info)) {
       if (off == 5 * am)
 #pragma unroll
         for (int kv = 0; kv < 5; ++kv)
 #pragma unroll
-          for (int l = 0; l < 5; ++l) acc[kv * 5 + l] += __ldg(Xq + kv * xs + l);
+          for (int l = 0; l < 5; ++l) acc[kv * 5 + l] += (float)__ldg(Xq + kv * xs + l);
     } else {
       // - A_bi[k, n_int(off..off+4)] Y_n[off.., k']
 #pragma unroll
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(256) k_learned_coupling(Geo G, const float* __
           const float yv = y_transposed ? Yn[(size_t)(5 * am + kk) * G.ldi + off + l]
                                         : Y[(size_t)n * ni * nb + (size_t)(off + l) * nb + 5 * am + kk];
 #pragma unroll
-          for (int kv = 0; kv < 5; ++kv) acc[kv * 5 + kk] = fmaf(-__ldg(Xq + kv * xs + l), yv, acc[kv * 5 + kk]);
+          for (int kv = 0; kv < 5; ++kv) acc[kv * 5 + kk] = fmaf(-(float)__ldg(Xq + kv * xs + l), yv, acc[kv * 5 + kk]);
         }
     }
   }
@@ -325,7 +325,7 @@ cudaError_t learned_couplings(sc_ctx* c) {
   cudaError_t e = cudaFuncSetAttribute(k_learned_coupling, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   count_launch(c);
-  k_learned_coupling<<<(3 * nsmp + 7) / 8, 256, smem, c->stream>>>(G, c->Aown32, c->Ainv32, c->X32, c->d_pptr,
+  k_learned_coupling<<<(3 * nsmp + 7) / 8, 256, smem, c->stream>>>(G, c->Aown32, c->Ainv32, c->X, c->d_pptr,
       c->d_pinfo, c->d_iperm, c->d_nbr, c->d_lface3, c->d_lmirror3, c->d_lnfaces, c->Y32,
       c->cfg.tensor_cores ? 1 : 0, c->Cpl);
   return cudaGetLastError();

@@ -165,7 +165,7 @@ cudaError_t precond_rb(sc_ctx* c, const double* v, double* z) {
   if (e == cudaSuccess) e = lu_solve_list(c, c->Sls, c->rowperm, 0, c->ls_full, c->d_colour, c->n_red, v, nullptr, z);
   if (e == cudaSuccess) e = cond_interior_sweep(c, z, c->Ui);
   if (e == cudaSuccess)
-    e = cond_boundary_pk_list<double>(c, c->Apk, c->X, z, c->Ui, c->Trb, c->d_colour + c->n_red, c->n_black);
+    e = cond_boundary_pk_list<double>(c, c->Apk, z, c->Ui, c->Trb, c->d_colour + c->n_red, c->n_black);
   if (e == cudaSuccess)
     e = lu_solve_list(c, c->Sls, c->rowperm, 0, c->ls_full, c->d_colour + c->n_red, c->n_black, v, c->Trb, z);
   return e;
@@ -190,7 +190,7 @@ cudaError_t precond_rb32(sc_ctx* c, const double* v, double* z, float* zf) {
     }
   }
   if (e == cudaSuccess) e = cond_interior_sweep32(c, zt, c->Uf);
-  if (e == cudaSuccess) e = cond_boundary_pk_list<float>(c, c->Apk32, c->X32, zt, c->Uf, c->Trb, black, c->n_black);
+  if (e == cudaSuccess) e = cond_boundary_pk_list<float>(c, c->Apk32, zt, c->Uf, c->Trb, black, c->n_black);
   if (e == cudaSuccess) {
     if (corrected)
       e = lu_solve_list32(c, c->SlsL, c->rowpermL, 1, c->black_full, black, c->n_black, v, c->Trb, z, zt);
