@@ -43,38 +43,238 @@ __global__ void k_history(Geo G, const double* __restrict__ Qs, const double* __
   Qh[t] = (bdf == 2) ? (4.0 * Qs[t] - Qsm1[t]) / 3.0 : Qs[t];
 }
 
-// Lifted gradients, one thread per node.
-SC_HD void lift_body(const Geo& G, const double* Q, const int* nbr, int t, double* grad, int lifted) {
-  const int e = t / G.nn, m = t % G.nn, p = G.p, N = G.N;
-  int c[3]; node_coords(m, p, c);
-  const double* qe = Q + (size_t)e * G.nn * 5;
-  const double* qm = qe + (size_t)m * 5;
-  for (int a = 0; a < 3; ++a) {
-    double acc[5] = {0, 0, 0, 0, 0};
-    int cc[3] = {c[0], c[1], c[2]};
-    for (int b = 0; b < p; ++b) {
-      cc[a] = b;
-      const double Dab = G.D[c[a]][b];
-      const double* qb = qe + (size_t)node_index(cc, p) * 5;
-      for (int k = 0; k < 5; ++k) acc[k] = fma(Dab, qb[k], acc[k]);
-    }
-    if (lifted && (c[a] == N || c[a] == 0)) {
-      const int s = (c[a] == N) ? 1 : -1;
-      const int nb = nbr[e * 18 + face_slot(a, s)];
-      int cn[3] = {c[0], c[1], c[2]}; cn[a] = N - c[a];
-      const double* qn = Q + ((size_t)nb * G.nn + node_index(cn, p)) * 5;
-      const double coef = 0.5 * s / G.w[c[a]];
-      for (int k = 0; k < 5; ++k) acc[k] = fma(coef, qn[k] - qm[k], acc[k]);
-    }
-    for (int k = 0; k < 5; ++k) grad[(size_t)t * 15 + a * 5 + k] = G.dx * acc[k];
+// ---- residual ---------------------------------------------------------------------------
+// Two kernels, one thread per node, CTAs of whole elements (four of order 2, two of order 3, else
+// one) whose values sit in shared memory:
+//   k_point  lifted gradients and point fluxes F_d = f^a_d - f^nu_d
+//   k_rows   rows of the residual: divergence lines, face terms, and what becomes of them
+// Face terms: with the central part of the numerical flux s (f^a(+) + f^a(-)) / 2 and the viscous
+// average s (f^nu(+) + f^nu(-)) / 2, fhat = s (F(+) + F(-)) / 2 - diss / 2 with the point fluxes
+// that are there already, so a face node costs one dissipation and no viscous flux.  Face
+// nodes are their own work items (6 (N+1)^2 per element, equal work), summed by their nodes
+// afterwards.  FP64-pipe bound: 46 + 54 us per Runge-Kutta stage at 8^3, N = 4 (the stage's update
+// included) against 22 + 22 + 215 + 16 us in five kernels with one thread per node doing its up to
+// three faces (Roe and two viscous fluxes each, 16 % of the warps resident).
+inline int group_elems(const Geo& G) { return G.nn <= 32 ? 4 : G.nn <= 64 ? 2 : 1; }
+inline int group_threads(const Geo& G) { return (group_elems(G) * G.nn + 31) / 32 * 32; }
+
+// Fluxes F_d = f^a_d - f^nu_d of one node along all directions.
+__device__ __forceinline__ void point_fluxes(const Geo& G, const double q[5], const double g[3][5], double F[3][5]) {
+  flux_viscous_all(G, q, g, F);
+  const double ir = 1.0 / q[0];
+  const double u[3] = {q[1] * ir, q[2] * ir, q[3] * ir};
+  const double pr = (G.gamma - 1.0) * (q[4] - 0.5 * (q[1] * u[0] + q[2] * u[1] + q[3] * u[2]));
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    F[d][0] = q[1 + d] - F[d][0];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) F[d][1 + i] = q[1 + i] * u[d] + (i == d ? pr : 0.0) - F[d][1 + i];
+    F[d][4] = (q[4] + pr) * u[d] - F[d][4];
   }
 }
 
-// lifted = 1: the BR1 lifted gradient g; 0: the element's own gradient Dq.
-__global__ void k_lift(Geo G, const double* __restrict__ Q, const int* __restrict__ nbr,
-                       double* __restrict__ grad, int lifted) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < G.K * G.nn) lift_body(G, Q, nbr, t, grad, lifted);
+__device__ __forceinline__ double warp_max_d(double v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+// Non-negative doubles order like their bit patterns; NaN is mapped to +inf.
+__device__ __forceinline__ void warp_max_into(double v, unsigned long long* out) {
+  v = warp_max_d(v == v ? v : INFINITY);
+  if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(v));
+}
+
+// Values of each thread (n per node) through shared memory to out[node][n], coalesced.
+template <int n>
+__device__ __forceinline__ void store_nodes(const double (&v)[n], double* buf, double* __restrict__ out, size_t first,
+                                            int nodes, bool live) {
+  __syncthreads();
+  if (live)
+#pragma unroll
+    for (int i = 0; i < n; ++i) buf[threadIdx.x * n + i] = v[i];
+  __syncthreads();
+  for (int i = threadIdx.x; i < nodes * n; i += blockDim.x) out[first * n + i] = buf[i];
+}
+
+// spd (or null): the largest signal speed |v| + c and the largest diffusivity
+// max(4/3, gamma/Pr) mu / (rho Re) of all nodes, folded in as bit patterns.
+template <bool IP>
+__global__ void __launch_bounds__(352) k_point(Geo G, int ge, const double* __restrict__ Q, const int* __restrict__ nbr,
+                                               double* __restrict__ F, double* __restrict__ grad,
+                                               double* __restrict__ Floc, double* __restrict__ gloc,
+                                               unsigned long long* __restrict__ spd) {
+  extern __shared__ __align__(16) double sm[];
+  const int p = G.p, N = G.N, nn = G.nn, e0 = blockIdx.x * ge, ne = min(ge, G.K - e0), nodes = ne * nn;
+  double* Ds = sm;               // p x p
+  double* qs = Ds + 64;          // [nodes][5]
+  double* buf = qs + ge * nn * 5;  // [nodes][15]
+  const size_t first = (size_t)e0 * nn;
+  for (int i = threadIdx.x; i < p * p; i += blockDim.x) Ds[i] = G.D[i / p][i % p];
+  for (int i = threadIdx.x; i < nodes * 5; i += blockDim.x) qs[i] = Q[first * 5 + i];
+  __syncthreads();
+  const bool live = threadIdx.x < nodes;
+  const int t = live ? threadIdx.x : 0, el = t / nn, m = t - el * nn, e = e0 + el;
+  const double* qe = qs + el * nn * 5;
+  const int c[3] = {m % p, (m / p) % p, m / (p * p)};
+  double q[5], g[15], gl[15];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) q[k] = qe[m * 5 + k];
+  const int stride[3] = {1, p, p * p};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    double acc[5] = {0, 0, 0, 0, 0};
+    const double* line = qe + (m - c[a] * stride[a]) * 5;
+    for (int b = 0; b < p; ++b) {
+      const double Dab = Ds[c[a] * p + b];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) acc[k] = fma(Dab, line[b * stride[a] * 5 + k], acc[k]);
+    }
+    if (IP)
+#pragma unroll
+      for (int k = 0; k < 5; ++k) gl[a * 5 + k] = G.dx * acc[k];
+    if (live && (c[a] == N || c[a] == 0)) {
+      const int s = c[a] == N ? 1 : -1;
+      const int nb = __ldg(nbr + e * 18 + face_slot(a, s));
+      const double* qn = Q + ((size_t)nb * nn + m + (N - 2 * c[a]) * stride[a]) * 5;
+      const double coef = 0.5 * s / G.w[0];  // the end weights are equal
+#pragma unroll
+      for (int k = 0; k < 5; ++k) acc[k] = fma(coef, __ldg(qn + k) - q[k], acc[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) g[a * 5 + k] = G.dx * acc[k];
+  }
+  if (grad) store_nodes(g, buf, grad, first, nodes, live);
+  double f[15];
+  point_fluxes(G, q, reinterpret_cast<const double(*)[5]>(g), reinterpret_cast<double(*)[5]>(f));
+  store_nodes(f, buf, F, first, nodes, live);
+  if (IP) {
+    store_nodes(gl, buf, gloc, first, nodes, live);
+    point_fluxes(G, q, reinterpret_cast<const double(*)[5]>(gl), reinterpret_cast<double(*)[5]>(f));
+    store_nodes(f, buf, Floc, first, nodes, live);
+  }
+  if (spd) {
+    const double ir = 1.0 / q[0];
+    const double u = q[1] * ir, v = q[2] * ir, w = q[3] * ir, vv = u * u + v * v + w * w;
+    const double pr = (G.gamma - 1.0) * (q[4] - 0.5 * q[0] * vv);
+    double mu = 1.0;
+    if (G.sutherland) {
+      const double T = G.gamma * G.Ma * G.Ma * pr * ir;
+      mu = (1.0 + G.Ts) * T * sqrt(T) / (T + G.Ts);
+    }
+    warp_max_into(sqrt(vv) + sqrt(G.gamma * pr * ir), spd);
+    warp_max_into(fmax(4.0 / 3.0, G.gamma / G.Pr) / G.Re * mu * ir, spd + 1);
+  }
+}
+
+// Rows of the residual.  RK = false: out = -R(Q); RK = true: the Runge-Kutta stage st with
+// rhs = -M^-1 H(Q), out the stage's new state.
+template <bool IP, bool RK>
+__global__ void __launch_bounds__(352) k_rows(Geo G, int ge, const double* __restrict__ Q, const double* __restrict__ Qh,
+                                              const double* __restrict__ F, const double* __restrict__ Floc,
+                                              const int* __restrict__ nbr, double* __restrict__ out, sc::RkStage st) {
+  extern __shared__ __align__(16) double sm[];
+  const int p = G.p, N = G.N, nn = G.nn, pp = p * p, e0 = blockIdx.x * ge, ne = min(ge, G.K - e0), nodes = ne * nn;
+  double* Ds = sm;                   // p x p
+  double* qs = Ds + 64;              // [nodes][5]
+  double* Fs = qs + ge * nn * 5;     // [nodes][15]
+  double* fs = Fs + ge * nn * 15;    // [ge][6][pp][5]: face terms fhat - s F_d
+  const size_t first = (size_t)e0 * nn;
+  for (int i = threadIdx.x; i < p * p; i += blockDim.x) Ds[i] = G.D[i / p][i % p];
+  for (int i = threadIdx.x; i < nodes * 5; i += blockDim.x) qs[i] = Q[first * 5 + i];
+  for (int i = threadIdx.x; i < nodes * 15; i += blockDim.x) Fs[i] = F[first * 15 + i];
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * 6 * pp; i += blockDim.x) {
+    const int el = i / (6 * pp), f = i / pp % 6, ia = i % pp, d = f >> 1, s = (f & 1) ? 1 : -1;
+    const int a = ia % p, b = ia / p, end = s > 0 ? N : 0;
+    const int sd = d == 0 ? 1 : d == 1 ? p : pp, s1 = d == 0 ? p : 1, s2 = d == 2 ? p : pp;  // in-face strides
+    const int m = end * sd + a * s1 + b * s2;
+    const size_t tn = (size_t)__ldg(nbr + (e0 + el) * 18 + f) * nn + m + (N - 2 * end) * sd;
+    const int k1 = 1 + d, k2 = d == 0 ? 2 : 1, k3 = d == 2 ? 2 : 3;  // momenta, normal one first
+    const double* qa = qs + (el * nn + m) * 5;
+    const double* qb = Q + tn * 5;
+    const double ra[5] = {qa[0], qa[k1], qa[k2], qa[k3], qa[4]};
+    const double rb[5] = {__ldg(qb), __ldg(qb + k1), __ldg(qb + k2), __ldg(qb + k3), __ldg(qb + 4)};
+    const double* Fa = Fs + (el * nn + m) * 15 + d * 5;
+    const double* Fb = (IP ? Floc : F) + tn * 15 + d * 5;
+    double fb[5], diss[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) fb[k] = __ldg(Fb + k);
+    adv_dissipation_x(G, ra, rb, (double)s, diss);
+    double* o = fs + (size_t)i * 5;
+    const int kk[5] = {0, k1, k2, k3, 4};
+    if (IP) {
+      const double* Fl = Floc + (first + el * nn + m) * 15 + d * 5;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const int v = kk[k];
+        o[v] = 0.5 * s * (__ldg(Fl + v) + __ldg(Fb + v)) - 0.5 * diss[k] + G.sigma * (ra[k] - rb[k]) - s * Fa[v];
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) o[k] = 0.5 * s * (fb[k] - Fa[k]);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) o[kk[k]] -= 0.5 * diss[k];
+    }
+  }
+  __syncthreads();
+  const bool live = threadIdx.x < nodes;
+  const int t = live ? threadIdx.x : 0, el = t / nn, m = t - el * nn;
+  const int c[3] = {m % p, (m / p) % p, m / pp};
+  const int stride[3] = {1, p, pp};
+  const double Wj = G.w[c[0]] * G.w[c[1]] * G.w[c[2]];
+  double r[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const double* line = Fs + (el * nn + m - c[d] * stride[d]) * 15 + d * 5;
+    for (int b = 0; b < p; ++b) {
+      const double coef = Ds[c[d] * p + b];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) r[k] = fma(coef, line[b * stride[d] * 15 + k], r[k]);
+    }
+    if (c[d] == 0 || c[d] == N) {
+      const int f = face_slot(d, c[d] == N ? 1 : -1);
+      const int ia = d == 0 ? c[1] + p * c[2] : d == 1 ? c[0] + p * c[2] : c[0] + p * c[1];
+      const double* o = fs + ((size_t)(el * 6 + f) * pp + ia) * 5;
+      const double iw = 1.0 / G.w[0];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) r[k] = fma(iw, o[k], r[k]);
+    }
+  }
+  // r is now the strong-form divergence over (h/2)^2 W_j per row: R = (h/2)^2 W_j r + time term
+  const double* q = qs + t * 5;
+  double y[5];
+  if (!RK) {
+    const double tcoef = G.c0 * G.Jf * 0.5 * G.h * Wj / G.dt, JW = G.Jf * Wj;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const double h = G.c0 != 0.0 ? __ldg(Qh + (first + t) * 5 + k) : q[k];
+      y[k] = -fma(JW, r[k], tcoef * (q[k] - h));
+    }
+  } else {
+    double dt;
+    if (st.first) {
+      const double smax = __longlong_as_double((long long)st.spd[0]), nmax = __longlong_as_double((long long)st.spd[1]);
+      const double dx = G.h / G.N;
+      dt = st.cfl * dx / smax;
+      if (st.dfl > 0.0 && nmax > 0.0) dt = fmin(dt, st.dfl * dx * dx / nmax);
+      if (blockIdx.x == 0 && threadIdx.x == 0) *st.dt = dt;
+    } else {
+      dt = *st.dt;
+    }
+    double mx = 0.0;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const double rhs = -G.dx * r[k];  // M_jj = (h/2)^3 W_j
+      mx = rhs == rhs ? fmax(mx, fabs(rhs)) : INFINITY;
+      const size_t i = (first + t) * 5 + k;
+      double dq = st.dt ? dt * rhs : 0.0;
+      if (st.a != 0.0 && live) dq = fma(st.a, st.dq[i], dq);
+      if (live) st.dq[i] = dq;
+      y[k] = fma(st.b, dq, q[k]);
+    }
+    if (st.rmax) warp_max_into(live ? mx : 0.0, st.rmax);
+  }
+  store_nodes(y, Fs, out, first, nodes, live);
 }
 
 SC_HD inline void load_node(const double* __restrict__ Q, const double* __restrict__ grad,
@@ -82,67 +282,6 @@ SC_HD inline void load_node(const double* __restrict__ Q, const double* __restri
   for (int k = 0; k < 5; ++k) q[k] = Q[t * 5 + k];
   for (int a = 0; a < 3; ++a)
     for (int k = 0; k < 5; ++k) g[a][k] = grad[t * 15 + a * 5 + k];
-}
-
-// Point fluxes F_d = f^a_d - f^nu_d, one thread per node.
-__global__ void k_flux(Geo G, const double* __restrict__ Q, const double* __restrict__ grad,
-                       double* __restrict__ F) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= G.K * G.nn) return;
-  double q[5], g[3][5];
-  load_node(Q, grad, t, q, g);
-  for (int d = 0; d < 3; ++d) {
-    double fa[5], fv[5];
-    flux_inviscid(G, q, d, fa);
-    flux_viscous(G, q, g, d, fv);
-    for (int k = 0; k < 5; ++k) F[(size_t)t * 15 + d * 5 + k] = fa[k] - fv[k];
-  }
-}
-
-// Residual rows; writes B = -R.  One thread per node.
-// gface: the gradients the face flux takes (lifted for BR1, unlifted for the interior penalty).
-__global__ void k_resid(Geo G, const double* __restrict__ Q, const double* __restrict__ Qh,
-                        const double* __restrict__ gface, const double* __restrict__ F,
-                        const int* __restrict__ nbr, double* __restrict__ Bout) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= G.K * G.nn) return;
-  const int e = t / G.nn, j = t % G.nn, p = G.p, N = G.N;
-  int c[3]; node_coords(j, p, c);
-  const double Wj = G.w[c[0]] * G.w[c[1]] * G.w[c[2]];
-  double r[5];
-  const double tcoef = G.c0 * G.Jf * 0.5 * G.h * Wj / G.dt;
-  for (int k = 0; k < 5; ++k) r[k] = tcoef * (Q[(size_t)t * 5 + k] - Qh[(size_t)t * 5 + k]);
-  const size_t e0 = (size_t)e * G.nn;
-  for (int d = 0; d < 3; ++d) {
-    int cc[3] = {c[0], c[1], c[2]};
-    for (int b = 0; b < p; ++b) {
-      cc[d] = b;
-      const double coef = G.Jf * Wj * G.D[c[d]][b];
-      const double* Fm = F + (e0 + node_index(cc, p)) * 15 + d * 5;
-      for (int k = 0; k < 5; ++k) r[k] = fma(coef, Fm[k], r[k]);
-    }
-  }
-  for (int d = 0; d < 3; ++d) {
-    if (c[d] != 0 && c[d] != N) continue;
-    const int s = (c[d] == N) ? 1 : -1;
-    const int nb = nbr[e * 18 + face_slot(d, s)];
-    int cn[3] = {c[0], c[1], c[2]}; cn[d] = N - c[d];
-    const size_t tn = (size_t)nb * G.nn + node_index(cn, p);
-    double qa[5], ga[3][5], qb[5], gb[3][5];
-    load_node(Q, gface, t, qa, ga);
-    load_node(Q, gface, tn, qb, gb);
-    double fr[5], fva[5], fvb[5];
-    flux_adv(G, qa, qb, d, s, fr);
-    flux_viscous(G, qa, ga, d, fva);
-    flux_viscous(G, qb, gb, d, fvb);
-    const double Sf = G.Jf * Wj / G.w[c[d]];
-    for (int k = 0; k < 5; ++k) {
-      double fhat = fr[k] - 0.5 * s * (fva[k] + fvb[k]);
-      if (G.visc_flux == 1) fhat = fma(G.sigma, qa[k] - qb[k], fhat);
-      r[k] = fma(Sf, fhat - s * F[(size_t)t * 15 + d * 5 + k], r[k]);
-    }
-  }
-  for (int k = 0; k < 5; ++k) Bout[(size_t)t * 5 + k] = -r[k];
 }
 
 // Point flux Jacobians of every node: NJ[e][comp][m].
@@ -497,15 +636,47 @@ inline unsigned blocks_for(size_t n, int bs) { return (unsigned)((n + bs - 1) / 
 
 namespace sc {
 
-cudaError_t launch_residual_geo(sc_ctx* c, const Geo& G, const double* Q, const double* Qh, double* out) {
-  const size_t nodes = (size_t)G.K * G.nn;
-  const bool ip = G.visc_flux == 1;
-  count_launch(c, ip ? 4 : 3);
-  k_lift<<<blocks_for(nodes, 128), 128, 0, c->stream>>>(G, Q, c->d_nbr, c->grad, 1);
-  if (ip) k_lift<<<blocks_for(nodes, 128), 128, 0, c->stream>>>(G, Q, c->d_nbr, c->gloc, 0);
-  k_flux<<<blocks_for(nodes, 128), 128, 0, c->stream>>>(G, Q, c->grad, c->F);
-  k_resid<<<blocks_for(nodes, 128), 128, 0, c->stream>>>(G, Q, Qh, ip ? c->gloc : c->grad, c->F, c->d_nbr, out);
+// Shared memory of the residual kernels per CTA.
+static size_t point_smem(const Geo& G) { return (64 + (size_t)group_elems(G) * G.nn * 20) * sizeof(double); }
+static size_t rows_smem(const Geo& G) {
+  return (64 + (size_t)group_elems(G) * (G.nn * 20 + 30 * G.p * G.p)) * sizeof(double);
+}
+
+template <bool IP>
+static cudaError_t launch_point(sc_ctx* c, const Geo& G, const double* Q, bool store_grad, unsigned long long* spd) {
+  const int ge = group_elems(G);
+  cudaError_t e = cudaFuncSetAttribute(k_point<IP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)point_smem(G));
+  if (e != cudaSuccess) return e;
+  count_launch(c);
+  k_point<IP><<<(G.K + ge - 1) / ge, group_threads(G), point_smem(G), c->stream>>>(
+      G, ge, Q, c->d_nbr, c->F, store_grad ? c->grad : nullptr, c->Floc, c->gloc, spd);
   return cudaGetLastError();
+}
+
+template <bool IP, bool RK>
+static cudaError_t launch_rows(sc_ctx* c, const Geo& G, const double* Q, const double* Qh, double* out, const RkStage& st) {
+  const int ge = group_elems(G);
+  cudaError_t e = cudaFuncSetAttribute(k_rows<IP, RK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem(G));
+  if (e != cudaSuccess) return e;
+  count_launch(c);
+  k_rows<IP, RK><<<(G.K + ge - 1) / ge, group_threads(G), rows_smem(G), c->stream>>>(G, ge, Q, Qh, c->F, c->Floc, c->d_nbr,
+                                                                                     out, st);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_residual_geo(sc_ctx* c, const Geo& G, const double* Q, const double* Qh, double* out) {
+  const bool ip = G.visc_flux == 1;
+  const cudaError_t e = ip ? launch_point<true>(c, G, Q, true, nullptr) : launch_point<false>(c, G, Q, true, nullptr);
+  if (e != cudaSuccess) return e;
+  return ip ? launch_rows<true, false>(c, G, Q, Qh, out, RkStage{}) : launch_rows<false, false>(c, G, Q, Qh, out, RkStage{});
+}
+
+cudaError_t launch_rk_stage(sc_ctx* c, const Geo& G, const double* q, double* qout, const RkStage& st) {
+  const bool ip = G.visc_flux == 1;
+  unsigned long long* spd = st.first ? st.spd : nullptr;
+  const cudaError_t e = ip ? launch_point<true>(c, G, q, false, spd) : launch_point<false>(c, G, q, false, spd);
+  if (e != cudaSuccess) return e;
+  return ip ? launch_rows<true, true>(c, G, q, nullptr, qout, st) : launch_rows<false, true>(c, G, q, nullptr, qout, st);
 }
 
 cudaError_t launch_residual(sc_ctx* c) { return launch_residual_geo(c, c->G, c->Q, c->Qh, c->B); }

@@ -184,6 +184,43 @@ SC_HD inline T abs_harten(const T& lam, const T& del) {
   return (lam * lam + del * del) * recip(2.0 * del);
 }
 
+// Dissipation of the advective numerical fluxes at a face with normal s e_x, momenta rotated so
+// that the normal component comes first: fhat . n = s (f(qa) + f(qb)) / 2 - diss / 2.  The same
+// waves as flux_roe and flux_lf below, without the central flux.
+SC_HD inline void adv_dissipation_x(const Geo& G, const double qa[5], const double qb[5], double s, double diss[5]) {
+  const double gm1 = G.gamma - 1.0;
+  const double ira = 1.0 / qa[0], irb = 1.0 / qb[0];
+  const double ua[3] = {qa[1] * ira, qa[2] * ira, qa[3] * ira}, ub[3] = {qb[1] * irb, qb[2] * irb, qb[3] * irb};
+  const double pa = gm1 * (qa[4] - 0.5 * (qa[1] * ua[0] + qa[2] * ua[1] + qa[3] * ua[2]));
+  const double pb = gm1 * (qb[4] - 0.5 * (qb[1] * ub[0] + qb[2] * ub[1] + qb[3] * ub[2]));
+  if (G.adv_flux == 1) {
+    const double wa = fabs(ua[0]) + sqrt(G.gamma * pa * ira), wb = fabs(ub[0]) + sqrt(G.gamma * pb * irb);
+    const double lam = wa >= wb ? wa : wb;
+    for (int k = 0; k < 5; ++k) diss[k] = lam * (qb[k] - qa[k]);
+    return;
+  }
+  const double ra = sqrt(qa[0]), rb = sqrt(qb[0]);
+  const double iw = 1.0 / (ra + rb);
+  double um[3];
+  for (int i = 0; i < 3; ++i) um[i] = (ra * ua[i] + rb * ub[i]) * iw;
+  const double Hm = (ra * (qa[4] + pa) * ira + rb * (qb[4] + pb) * irb) * iw;
+  const double vsq = um[0] * um[0] + um[1] * um[1] + um[2] * um[2];
+  const double c2 = gm1 * (Hm - 0.5 * vsq), cm = sqrt(c2), ic2 = 1.0 / c2;
+  const double rhom = ra * rb, un = um[0] * s;
+  const double jr = qb[0] - qa[0], jp = pb - pa;
+  const double jun = (ub[0] - ua[0]) * s, jv = ub[1] - ua[1], jw = ub[2] - ua[2];
+  const double wm = 0.5 * (jp - rhom * cm * jun) * ic2, wp = 0.5 * (jp + rhom * cm * jun) * ic2, we = jr - jp * ic2;
+  const double del = G.roe_delta * cm;
+  const double i2d = 0.5 / del;
+  auto fix = [&](double lam) { return fabs(lam) >= del ? fabs(lam) : (lam * lam + del * del) * i2d; };
+  const double am = fix(un - cm) * wm, ap = fix(un + cm) * wp, a0 = fix(un);
+  diss[0] = am + ap + a0 * we;
+  diss[1] = (am + ap + a0 * we) * um[0] + (ap - am) * cm * s;
+  diss[2] = (am + ap) * um[1] + a0 * (we * um[1] + rhom * jv);
+  diss[3] = (am + ap) * um[2] + a0 * (we * um[2] + rhom * jw);
+  diss[4] = (am + ap) * Hm + (ap - am) * cm * un + a0 * (0.5 * we * vsq + rhom * (um[1] * jv + um[2] * jw));
+}
+
 // Roe numerical flux fhat(qa, qb, n) . n, n = s e_d outward from qa's element,
 // with Roe-averaged wave decomposition and Harten's entropy fix on every wave.
 template <class T>
@@ -289,7 +326,7 @@ struct sc_ctx {
   double *NJ = nullptr, *RJ = nullptr, *Aown = nullptr, *X = nullptr;
   // interior penalty only: the elements' own (unlifted) gradients and the point-flux
   // Jacobians at them, same layouts as grad and NJ
-  double *gloc = nullptr, *NJL = nullptr;
+  double *gloc = nullptr, *NJL = nullptr, *Floc = nullptr;
   int *d_nbr = nullptr, *d_perm = nullptr, *d_iperm = nullptr, *d_own_pairs = nullptr;
   double* gj_scale = nullptr;      // [K][n_i] row scaling of the blocked Gauss-Jordan (T-typed)
   double *OV = nullptr, *OZ = nullptr;  // outer FGMRES: Arnoldi basis (m+1 global vectors), preconditioned (m)
@@ -438,8 +475,20 @@ namespace sc {
 void gl_basis(int N, std::vector<double>& x, std::vector<double>& w, double D[SC_MAXP][SC_MAXP]);
 cudaError_t launch_residual(sc_ctx* c);
 // -R(Q) with the geometry G (c0 = 0 gives -H(Q), the spatial operator alone) into out;
-// uses c->grad and c->F as scratch.
+// fills c->grad (and c->gloc) and uses c->F as scratch.
 cudaError_t launch_residual_geo(sc_ctx* c, const Geo& G, const double* Q, const double* Qh, double* out);
+// One stage of the low-storage Runge-Kutta scheme on dq/dt = -M^-1 H(q): dq <- a dq + dt rhs,
+// qout <- q + b dq (qout != q).  first: this stage reads the step's signal speeds (spd[0], spd[1],
+// zero on entry) and leaves dt = min(cfl (h/N) / spd[0], dfl (h/N)^2 / spd[1]) in *dt; the later
+// stages read *dt.  max |rhs| is folded into *rmax (or not: null).
+struct RkStage {
+  double a, b, cfl, dfl;
+  unsigned long long *spd, *rmax;
+  double* dt;
+  double* dq;
+  int first;
+};
+cudaError_t launch_rk_stage(sc_ctx* c, const Geo& G, const double* q, double* qout, const RkStage& st);
 cudaError_t launch_history(sc_ctx* c, const double* Qs, const double* Qsm1);
 cudaError_t launch_assembly(sc_ctx* c);
 cudaError_t launch_condense(sc_ctx* c);

@@ -49,10 +49,8 @@ __device__ void block_max_into(double v, unsigned long long* out) {
   }
 }
 
-// rhs = B / (J W_j), B = -H(Q): the right-hand side -M^-1 H(Q) of the semi-discrete system;
-// max |rhs| (the steady-state residual ||M^-1 H||_inf) into *rmax.  rhs may be null.
-__global__ void __launch_bounds__(kThreads) k_rhs(Geo G, const double* __restrict__ B, double* __restrict__ rhs,
-                                                  unsigned long long* rmax) {
+// Steady-state residual ||M^-1 H||_inf = max |B / (J W_j)| of B = -H(Q), folded into *rmax.
+__global__ void __launch_bounds__(kThreads) k_rhs(Geo G, const double* __restrict__ B, unsigned long long* rmax) {
   const size_t n = (size_t)G.K * G.nn * 5;
   double mx = 0.0;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
@@ -60,64 +58,9 @@ __global__ void __launch_bounds__(kThreads) k_rhs(Geo G, const double* __restric
     const int i0 = j % G.p, i1 = (j / G.p) % G.p, i2 = j / (G.p * G.p);
     const double MJ = G.Jf * 0.5 * G.h * G.w[i0] * G.w[i1] * G.w[i2];
     const double v = B[t] / MJ;
-    if (rhs) rhs[t] = v;
     mx = (v == v) ? fmax(mx, fabs(v)) : INFINITY;
   }
   block_max_into(mx, rmax);
-}
-
-// Largest signal speed |v| + c and largest diffusivity max(4/3, gamma/Pr) mu / (rho Re) over
-// all nodes (App. B nondimensionalisation: p = (gamma - 1)(rho E - rho |v|^2 / 2),
-// c^2 = gamma p / rho, T = gamma Ma^2 p / rho, Sutherland mu(T)).
-__global__ void __launch_bounds__(kThreads) k_speeds(Geo G, const double* __restrict__ Q,
-                                                     unsigned long long* __restrict__ out) {
-  const size_t nodes = (size_t)G.K * G.nn;
-  double smax = 0.0, nmax = 0.0;
-  const double dcoef = fmax(4.0 / 3.0, G.gamma / G.Pr) / G.Re;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < nodes; t += (size_t)gridDim.x * blockDim.x) {
-    const double* q = Q + t * 5;
-    const double ir = 1.0 / q[0];
-    const double u = q[1] * ir, v = q[2] * ir, w = q[3] * ir;
-    const double vv = u * u + v * v + w * w;
-    const double p = (G.gamma - 1.0) * (q[4] - 0.5 * q[0] * vv);
-    const double s = sqrt(vv) + sqrt(G.gamma * p * ir);
-    double mu = 1.0;
-    if (G.sutherland) {
-      const double T = G.gamma * G.Ma * G.Ma * p * ir;
-      mu = (1.0 + G.Ts) * T * sqrt(T) / (T + G.Ts);
-    }
-    const double nu = dcoef * mu * ir;
-    smax = (s == s) ? fmax(smax, s) : INFINITY;
-    nmax = (nu == nu) ? fmax(nmax, nu) : INFINITY;
-  }
-  block_max_into(smax, out);
-  __syncthreads();
-  block_max_into(nmax, out + 1);
-}
-
-// dt = min(cfl (h/N) / smax, dfl (h/N)^2 / numax) (dfl <= 0: no diffusive limit); clears
-// the speed maxima for the next step.
-__global__ void k_dt(Geo G, double cfl, double dfl, unsigned long long* spd, double* dt_out) {
-  const double smax = __longlong_as_double((long long)spd[0]);
-  const double nmax = __longlong_as_double((long long)spd[1]);
-  const double dx = G.h / G.N;
-  double dt = cfl * dx / smax;
-  if (dfl > 0.0 && nmax > 0.0) dt = fmin(dt, dfl * dx * dx / nmax);
-  *dt_out = dt;
-  spd[0] = 0ull;
-  spd[1] = 0ull;
-}
-
-// One stage of the two-register scheme: dq <- a dq + dt rhs, q <- q + b dq.
-__global__ void __launch_bounds__(kThreads) k_rk_stage(size_t n, double a, double b, const double* __restrict__ rhs,
-                                                       const double* __restrict__ dtp, double* __restrict__ dq,
-                                                       double* __restrict__ q) {
-  const double dt = *dtp;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-    const double d = a * dq[t] + dt * rhs[t];
-    dq[t] = d;
-    q[t] += b * d;
-  }
 }
 
 __global__ void k_axpy(size_t n, double a, const double* __restrict__ x, double* __restrict__ y) {
@@ -164,7 +107,7 @@ sc_status sc_steady_residual(sc_ctx* c, double* res_inf) {
   MC_CUDA(cudaMemsetAsync(r.p, 0, sizeof(unsigned long long), c->stream));
   MC_CUDA(sc::launch_residual_geo(c, Gs, c->Q, c->Q, c->Rfull));
   count_launch(c);
-  k_rhs<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->Rfull, nullptr, (unsigned long long*)r.p);
+  k_rhs<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->Rfull, (unsigned long long*)r.p);
   unsigned long long b = 0;
   MC_CUDA(cudaMemcpyAsync(&b, r.p, sizeof(b), cudaMemcpyDeviceToHost, c->stream));
   MC_CUDA(cudaStreamSynchronize(c->stream));
@@ -181,38 +124,36 @@ sc_status sc_explicit_march(sc_ctx* c, double cfl, double dfl, int nsteps, doubl
   const size_t dofs = (size_t)G.K * G.ne;
   Geo Gs = G;
   Gs.c0 = 0.0;  // the spatial operator alone
-  DevBuf dq, rhs, r, spd, dtv;
-  MC_CUDA(cudaMalloc(&dq.p, dofs * sizeof(double)));
-  MC_CUDA(cudaMalloc(&rhs.p, dofs * sizeof(double)));
-  MC_CUDA(cudaMalloc(&r.p, (size_t)(nsteps + 2) * sizeof(unsigned long long)));
-  MC_CUDA(cudaMalloc(&spd.p, 2 * sizeof(unsigned long long)));
-  MC_CUDA(cudaMalloc(&dtv.p, (size_t)std::max(nsteps, 1) * sizeof(double)));
-  unsigned long long* rd = (unsigned long long*)r.p;
-  double* dqd = (double*)dq.p;
-  double* rhsd = (double*)rhs.p;
-  double* dtd = (double*)dtv.p;
-  MC_CUDA(cudaMemsetAsync(r.p, 0, (size_t)(nsteps + 2) * sizeof(unsigned long long), c->stream));
-  MC_CUDA(cudaMemsetAsync(spd.p, 0, 2 * sizeof(unsigned long long), c->stream));
-  MC_CUDA(cudaMemsetAsync(dq.p, 0, dofs * sizeof(double), c->stream));
+  // one allocation: the second register, the speeds of every step, the residual maxima, the steps
+  const size_t ns = (size_t)std::max(nsteps, 1), words = dofs + 2 * ns + (size_t)(nsteps + 2) + ns;
+  DevBuf mem;
+  MC_CUDA(cudaMalloc(&mem.p, words * sizeof(double)));
+  double* dqd = (double*)mem.p;
+  unsigned long long* spd = (unsigned long long*)(dqd + dofs);
+  unsigned long long* rd = spd + 2 * ns;
+  double* dtd = (double*)(rd + nsteps + 2);
+  MC_CUDA(cudaMemsetAsync(spd, 0, (2 * ns + (size_t)(nsteps + 2)) * sizeof(unsigned long long), c->stream));
   cudaEvent_t e0, e1;
   MC_CUDA(cudaEventCreate(&e0));
   MC_CUDA(cudaEventCreate(&e1));
   struct Ev { cudaEvent_t a, b; ~Ev() { cudaEventDestroy(a); cudaEventDestroy(b); } } evg{e0, e1};
   MC_CUDA(cudaEventRecord(e0, c->stream));
+  // every stage reads one state buffer (neighbours' values included) and writes the other
+  double *qin = c->Q, *qout = c->Xfull;
   for (int st = 0; st < nsteps; ++st) {
-    count_launch(c, 2);
-    k_speeds<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->Q, (unsigned long long*)spd.p);
-    k_dt<<<1, 1, 0, c->stream>>>(Gs, cfl, dfl, (unsigned long long*)spd.p, dtd + st);
     for (int k = 0; k < 3; ++k) {
-      MC_CUDA(sc::launch_residual_geo(c, Gs, c->Q, c->Q, c->Rfull));
-      count_launch(c, 2);
-      k_rhs<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->Rfull, rhsd, k == 0 ? rd + st : rd + nsteps + 1);
-      k_rk_stage<<<kBlocks, kThreads, 0, c->stream>>>(dofs, kRkA[k], kRkB[k], rhsd, dtd + st, dqd, c->Q);
+      sc::RkStage s3{};
+      s3.a = kRkA[k]; s3.b = kRkB[k]; s3.cfl = cfl; s3.dfl = dfl;
+      s3.spd = spd + 2 * st; s3.rmax = k == 0 ? rd + st : nullptr;
+      s3.dt = dtd + st; s3.dq = dqd; s3.first = k == 0;
+      MC_CUDA(sc::launch_rk_stage(c, Gs, qin, qout, s3));
+      std::swap(qin, qout);
     }
   }
+  if (qin != c->Q) MC_CUDA(cudaMemcpyAsync(c->Q, qin, dofs * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
   MC_CUDA(sc::launch_residual_geo(c, Gs, c->Q, c->Q, c->Rfull));
   count_launch(c);
-  k_rhs<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->Rfull, nullptr, rd + nsteps);
+  k_rhs<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->Rfull, rd + nsteps);
   MC_CUDA(cudaEventRecord(e1, c->stream));
   // the new state is also the BDF1 history of a following implicit step
   MC_CUDA(sc::launch_history(c, c->Q, c->Q));
@@ -271,7 +212,7 @@ sc_status sc_implicit_march(sc_ctx* c, double dt, int nsteps, int jacobian_every
       MC_CUDA(sc::launch_residual(c));  // B = -R(Q) with the frozen Jacobian kept
     }
     count_launch(c);
-    k_rhs<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->B, nullptr, rd + st);
+    k_rhs<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->B, rd + st);
     if (steady_tol > 0.0) {  // stop once the state at the start of the step is steady
       unsigned long long b = 0;
       MC_CUDA(cudaMemcpyAsync(&b, rd + st, sizeof(b), cudaMemcpyDeviceToHost, c->stream));
@@ -290,7 +231,7 @@ sc_status sc_implicit_march(sc_ctx* c, double dt, int nsteps, int jacobian_every
   MC_CUDA(sc::launch_residual_geo(c, Gs, c->Q, c->Q, c->Rfull));
   count_launch(c);
   MC_CUDA(cudaMemsetAsync(rd + taken, 0, sizeof(unsigned long long), c->stream));
-  k_rhs<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->Rfull, nullptr, rd + taken);
+  k_rhs<<<kBlocks, kThreads, 0, c->stream>>>(Gs, c->Rfull, rd + taken);
   MC_CUDA(sc::launch_history(c, c->Q, c->Q));
   MC_CUDA(cudaGetLastError());
   std::vector<unsigned long long> rb(nsteps + 1);
