@@ -385,8 +385,7 @@ sc_status sc_hessenberg_eigvals(int m, const double* H, double* re, double* im);
    SC_ERR_ARG for null pointers or bad sizes, SC_ERR_CUDA for launch failures. */
 
 /* y[n x 25] = net(X[n x 128]).  cache: NULL, or 4 n x 256 floats that receive z1, h1, z2,
-   h2 (pre- and post-activations) for sc_mlp_backward; with NULL the call allocates
-   temporaries on the stream. */
+   h2 (pre- and post-activations) for sc_mlp_backward. */
 sc_status sc_mlp_forward(const uint16_t* Wbf16, const float* bias, const float* X, int n, float* Y, float* cache,
                          void* cuda_stream);
 

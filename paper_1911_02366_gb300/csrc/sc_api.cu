@@ -96,7 +96,7 @@ void free_all(sc_ctx* c) {
                     &c->OV, &c->OZ, &c->gloc, &c->NJL, &c->Floc};
   for (auto p : dps) { if (*p) cudaFree(*p); *p = nullptr; }
   float** fps[] = {&c->Aown32, &c->Ainv32, &c->Y32, &c->See32, &c->Zf, &c->Xbf, &c->Uf,
-                   &c->Apk32, &c->Sls32, &c->Sdiag, &c->Cpl, &c->Feat, &c->Snorm, &c->Ynet, &c->Hbuf,
+                   &c->Apk32, &c->Sls32, &c->Sdiag, &c->Cpl, &c->Feat, &c->Snorm, &c->Ynet,
                    &c->Ck, &c->Wbias, &c->ExIb, &c->ExBi, &c->ExY, &c->ExW, &c->Zrb, &c->SeeB, &c->SeeL, &c->SlsL,
                    &c->Zinv};
   for (auto p : fps) { if (*p) cudaFree(*p); *p = nullptr; }
@@ -385,7 +385,7 @@ sc_status sc_set_mesh(sc_ctx* c, int n, double L, int N) {
     A(dalloc(&c->Sdiag, nsmp * 25)); A(dalloc(&c->Cpl, nsmp * 75));  // 3 face slots per node
     if (c->cfg.precond == SC_PC_LEARNED) {
       A(dalloc(&c->Feat, nsmp * sc::kMlpInputs)); A(dalloc(&c->Snorm, nsmp)); A(dalloc(&c->Ynet, nsmp * 25));
-      A(dalloc(&c->Hbuf, nsmp * 512)); A(dalloc(&c->Ck, nsmp * 25)); A(dalloc(&c->Wbias, (size_t)sc::kMlpBiases));
+      A(dalloc(&c->Ck, nsmp * 25)); A(dalloc(&c->Wbias, (size_t)sc::kMlpBiases));
       A(dalloc(&c->Wbf16, (size_t)sc::kMlpWeights));
     }
     A(dalloc(&c->Apk32, (size_t)G.K * c->pk_stride)); A(dalloc(&c->Sls32, sc::solve_layout_elems(G)));

@@ -371,7 +371,7 @@ struct sc_ctx {
   int *d_lface3 = nullptr, *d_lmirror3 = nullptr, *d_lrslot3 = nullptr;
   int *d_lface = nullptr, *d_lmirror = nullptr;
   float *Sdiag = nullptr, *Cpl = nullptr;  // [K nbn][25] [S_ee]_kk; [K nbn][3][25] S_(k,k'_f) per face of k
-  float *Feat = nullptr, *Snorm = nullptr, *Ynet = nullptr, *Hbuf = nullptr, *Ck = nullptr, *Wbias = nullptr;
+  float *Feat = nullptr, *Snorm = nullptr, *Ynet = nullptr, *Ck = nullptr, *Wbias = nullptr;
   uint16_t* Wbf16 = nullptr;
   bool Sdiag_valid = false, weights_set = false, learned_on = false;
   int learned_fallbacks = 0;
@@ -563,8 +563,7 @@ cudaError_t assemble_correction(sc_ctx* c, const float* Y, float scale);
 constexpr int kGjRegRows = 136;
 constexpr int kMlpInputs = 128;
 constexpr int kMlpWeights = 256 * kMlpInputs + 256 * 256 + 25 * 256, kMlpBiases = 2 * 256 + 25;
-cudaError_t mlp_forward(cudaStream_t st, const uint16_t* Wbf16, const float* bias, const float* X, int n, float* Y,
-                        float* h1, float* h2);
+cudaError_t mlp_forward(cudaStream_t st, const uint16_t* Wbf16, const float* bias, const float* X, int n, float* Y);
 cudaError_t upload_packed_pattern(sc_ctx* c);
 cudaError_t pack_own(sc_ctx* c);
 template <class T>

@@ -373,7 +373,7 @@ cudaError_t learned_correction(sc_ctx* c) {
   const int nsmp = G.K * G.nbn;
   cudaError_t e = learned_features(c, c->Feat, c->Snorm);
   if (e == cudaSuccess)
-    e = mlp_forward(c->stream, c->Wbf16, c->Wbias, c->Feat, nsmp, c->Ynet, c->Hbuf, c->Hbuf + (size_t)nsmp * 256);
+    e = mlp_forward(c->stream, c->Wbf16, c->Wbias, c->Feat, nsmp, c->Ynet);
   if (e == cudaSuccess) e = assemble_correction(c, c->Ynet, kNetworkDamping);
   return e;
 }

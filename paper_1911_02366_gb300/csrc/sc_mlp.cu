@@ -3,14 +3,12 @@
 // learned part of the condensed-system preconditioner of Sec. 2.2/4), with its training loop
 // (shuffled mini-batch Adam) and a file format for its parameters.
 //
-// All layers run through one SIMT tile kernel, C (+)= op(A) op(B), 64 x 64 tiles, 16-deep
-// K chunks staged in shared memory (BF16 operands widened to FP32 on the way), 4 x 4
-// outputs per thread, with the epilogue each use needs:
-//   forward      Z = X W^T + b, H = relu(Z)          (A = X, B = W stored out x in)
+// The forward pass is one tensor-core kernel, 128 samples per CTA through all layers with the
+// activations in TMEM.  The backward pass runs through a SIMT tile kernel, C (+)= op(A) op(B), K
+// chunks staged in shared memory (BF16 operands widened to FP32 on the way):
 //   backward dX  dZ_prev = (dZ W) * [Z_prev > 0]      (A = dZ, B = W)
 //   backward dW  gW += dZ^T X, split over samples     (A = dZ stored n x out)
-// plus the loss, bias-gradient and Adam kernels.  Tensor cores stay with the Schur
-// products; the network is ~0.2 MFLOP per boundary node.
+// plus the loss, bias-gradient and Adam kernels.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -20,6 +18,7 @@
 #include <vector>
 
 #include "sc_internal.cuh"
+#include "sc_tcgen.cuh"
 
 namespace {
 
@@ -33,67 +32,354 @@ template <> __device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloa
   return __bfloat162float(*p);
 }
 
-enum Epi { EPI_BIAS = 0, EPI_BIAS_RELU = 1, EPI_MASK = 2, EPI_ATOMIC = 3 };
+enum Epi { EPI_MASK = 0, EPI_ATOMIC = 1 };
 
-// C[M x N] from op(A)[M x K] op(B)[K x N]; A stored M x K (lda) or K x M when TA;
-// B stored K x N (ldb) or N x K when TB.  gridDim.z splits K (EPI_ATOMIC only).
-template <class TA_, class TB_, bool TA, bool TB, int EPI>
-__global__ void __launch_bounds__(256) k_mlp_gemm(int M, int N, int K, const TA_* __restrict__ A, int lda,
+// C[M x N] from op(A)[M x K] op(B)[K x N], B stored K x N (ldb); A stored M x K (lda) or K x M
+// when TA.  gridDim.z splits K (EPI_ATOMIC only).  BT x BT tiles, BK deep; the next K chunk is
+// loaded while the current one is multiplied.  A training batch is latency bound: with 64 x 64
+// tiles a layer of 256 samples has 16 CTAs, so small products take 32 x 32 tiles.
+template <class TB_, bool TA, int EPI, int BT, int BK>
+__global__ void __launch_bounds__(256) k_mlp_gemm(int M, int N, int K, const float* __restrict__ A, int lda,
                                                   const TB_* __restrict__ B, int ldb, float* __restrict__ C, int ldc,
-                                                  const float* __restrict__ bias, float* __restrict__ Zout,
                                                   const float* __restrict__ mask, int kchunk) {
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
+  constexpr int PT = BT / 16, LD = BT * BK / 256;  // outputs per thread and direction, loads per thread
+  __shared__ float As[BK][BT + 4];
+  __shared__ float Bs[BK][BT + 4];
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+  const int m0 = blockIdx.y * BT, n0 = blockIdx.x * BT;
   const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
-  float acc[4][4] = {};
-  for (int k0 = kb; k0 < ke; k0 += 16) {
-    for (int t = threadIdx.x; t < 16 * 64; t += 256) {
-      const int kk = t / 64, mm = t % 64;
-      const int gk = k0 + kk, gm = m0 + mm, gn = n0 + mm;
-      float a = 0.f, b = 0.f;
-      if (gk < ke && gm < M) a = TA ? ldf(A + (size_t)gk * lda + gm) : ldf(A + (size_t)gm * lda + gk);
-      if (gk < ke && gn < N) b = TB ? ldf(B + (size_t)gn * ldb + gk) : ldf(B + (size_t)gk * ldb + gn);
-      As[kk][mm] = a;
-      Bs[kk][mm] = b;
+  float acc[PT][PT] = {}, ra[LD], rb[LD];
+  // A stored M x K is contiguous in k, everything else in the tile's rows
+  auto a_pos = [&](int i, int& kk, int& mm) {
+    const int t = threadIdx.x + 256 * i;
+    if (TA) { kk = t / BT; mm = t % BT; } else { kk = t % BK; mm = t / BK; }
+  };
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < LD; ++i) {
+      int kk, mm;
+      a_pos(i, kk, mm);
+      const int ga = k0 + kk, gm = m0 + mm;
+      ra[i] = ga < ke && gm < M ? (TA ? ldf(A + (size_t)ga * lda + gm) : ldf(A + (size_t)gm * lda + ga)) : 0.f;
+      const int t = threadIdx.x + 256 * i, gk = k0 + t / BT, gn = n0 + t % BT;
+      rb[i] = gk < ke && gn < N ? ldf(B + (size_t)gk * ldb + gn) : 0.f;
     }
+  };
+  load(kb);
+  for (int k0 = kb; k0 < ke; k0 += BK) {
     __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty + 16 * i]; b[i] = Bs[kk][tx + 16 * i]; }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    for (int i = 0; i < LD; ++i) {
+      int kk, mm;
+      a_pos(i, kk, mm);
+      As[kk][mm] = ra[i];
+      const int t = threadIdx.x + 256 * i;
+      Bs[t / BT][t % BT] = rb[i];
     }
     __syncthreads();
+    if (k0 + BK < ke) load(k0 + BK);
+#pragma unroll
+    for (int kk = 0; kk < BK; ++kk) {
+      float a[PT], b[PT];
+#pragma unroll
+      for (int i = 0; i < PT; ++i) { a[i] = As[kk][ty + 16 * i]; b[i] = Bs[kk][tx + 16 * i]; }
+#pragma unroll
+      for (int i = 0; i < PT; ++i)
+#pragma unroll
+        for (int j = 0; j < PT; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < PT; ++i) {
     const int r = m0 + ty + 16 * i;
     if (r >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < PT; ++j) {
       const int cc = n0 + tx + 16 * j;
       if (cc >= N) continue;
       float v = acc[i][j];
       if (EPI == EPI_ATOMIC) {
         atomicAdd(C + (size_t)r * ldc + cc, v);
       } else {
-        if (EPI == EPI_BIAS || EPI == EPI_BIAS_RELU) {
-          v += bias[cc];
-          if (Zout) Zout[(size_t)r * ldc + cc] = v;
-          if (EPI == EPI_BIAS_RELU) v = fmaxf(v, 0.f);
-        } else if (EPI == EPI_MASK) {
-          if (!(mask[(size_t)r * ldc + cc] > 0.f)) v = 0.f;
-        }
+        if (!(mask[(size_t)r * ldc + cc] > 0.f)) v = 0.f;
         C[(size_t)r * ldc + cc] = v;
       }
     }
   }
+}
+
+// ---- forward pass on the tensor cores -------------------------------------------------
+// One CTA takes 128 samples through all three layers: C = A W^T as tcgen05.mma (kind::f16, BF16
+// operands, M = 128).  The FP32 inputs of a layer are split exactly into three BF16 parts of 8
+// significand bits each (cut, not rounded) and the weights are BF16 already, so every product is
+// exact.  The tensor cores' FP32 accumulation cuts where FMA rounds: over a whole layer that
+// costs four times the error of an FMA chain (1.4e-6 against 3.5e-7 of the largest output), so
+// the accumulator (TMEM columns 0 .. 255) is started anew for every 64 inputs, the small parts first, and the
+// partial sums are added up in registers.  The activations wait in TMEM columns 256 .. 511 for the
+// next layer and leave the SM only if the caller asks for them (z1 .. h2).  Inputs and weights are
+// staged in two shared-memory buffers (three 128 x 64 parts and a 256 x 64 piece of the weights,
+// K-major core matrices of 8 rows x 16 bytes): while the tensor cores work on one chunk, the threads split
+// and store the next and load the one after.  Thread t holds row t % 128 (its TMEM lane) and of every
+// 64 columns the half t / 128.  A wait that runs out leaves NaN in its samples' outputs.
+// 100,352 samples: 0.20 ms against 1.84 ms in three SIMT products (and 0.6 ms of host time for their
+// temporaries); 256 samples: 52 against 82 us.  Bound by the chain of one CTA's chunks (split, store,
+// multiply, collect) more than by the tensor cores.
+constexpr int kFwStage = 3 * 128 * 64 * 2 + 256 * 64 * 2;  // bytes
+constexpr int kCoreLbo = 128, kCoreSbo = 8 * kCoreLbo;
+__device__ __forceinline__ uint32_t bf16_core(int row, int k) {
+  return (uint32_t)((row >> 3) * kCoreSbo + (k >> 3) * kCoreLbo + (row & 7) * 16);
+}
+__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                         uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// D = F32, A = B = BF16, both K-major, M = 128.
+constexpr uint32_t idesc_bf16(int N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+__device__ __forceinline__ bool wait_bounded(uint64_t* bar, uint32_t parity) {
+  for (long long it = 0; it <= kWaitLimit; ++it)
+    if (mbar_try_wait(bar, parity)) return true;
+  return false;
+}
+// x = p[0] + p[1] + p[2] in BF16 (bit patterns); infinities and NaN stay in the first part.
+__device__ __forceinline__ void split3(float x, uint32_t p[3]) {
+  const uint32_t b = __float_as_uint(x);
+  p[0] = b >> 16;
+  if ((b & 0x7f800000u) == 0x7f800000u) {
+    if (b & 0x007fffffu) p[0] |= 0x40u;
+    p[1] = p[2] = 0u;
+    return;
+  }
+  const float r1 = x - __uint_as_float(b & 0xffff0000u);
+  p[1] = __float_as_uint(r1) >> 16;
+  p[2] = __float_as_uint(r1 - __uint_as_float(__float_as_uint(r1) & 0xffff0000u)) >> 16;
+}
+
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float* v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
+               "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+               "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
+               "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
+               : "memory");
+}
+// 32 accumulator columns added to acc.
+__device__ __forceinline__ void tmem_add32(uint32_t taddr, float* acc) {
+  uint32_t r[4][8];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) tmem_ld8_async(taddr + 8 * g, r[g]);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) acc[i] += __uint_as_float(r[i >> 3][i & 7]);
+}
+
+struct FwLane {  // what a thread of k_mlp_forward works on
+  const __nv_bfloat16* W;
+  const float* X;
+  unsigned char* stage;
+  uint64_t* bar;
+  uint32_t tmem, lanes;
+  int tid, row, half, gr, n, flags, step;
+};
+
+// Piece k0 .. k0 + 63 of a layer's weights: one row per thread (256 rows), or one 16-byte piece
+// (32 rows, 25 of them real).
+template <int L>
+__device__ __forceinline__ void fw_load_w(const FwLane& f, int k0, uint4 w[8]) {
+  constexpr int K = L == 0 ? NI : NH;
+  const __nv_bfloat16* Wl = f.W + (L == 0 ? 0 : L == 1 ? OFF_W2 : OFF_W3);
+  auto piece = [&](int r, int k) {
+    const __nv_bfloat16* p = Wl + (size_t)r * K + k0 + k;
+    if (f.flags & 2) return __ldg(reinterpret_cast<const uint4*>(p));
+    const unsigned short* q = reinterpret_cast<const unsigned short*>(p);
+    return make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16, q[4] | (uint32_t)q[5] << 16,
+                      q[6] | (uint32_t)q[7] << 16);
+  };
+  if (L < 2) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = piece(f.tid, 8 * i);
+  } else {
+    w[0] = (f.tid & 31) < NO ? piece(f.tid & 31, 8 * (f.tid >> 5)) : make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+__device__ __forceinline__ void fw_load_x(const FwLane& f, int k0, float a[32]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (f.gr < f.n) {
+      const float* p = f.X + (size_t)f.gr * NI + k0 + 32 * f.half + 4 * i;
+      if (f.flags & 1) v = __ldg(reinterpret_cast<const float4*>(p));
+      else v = make_float4(p[0], p[1], p[2], p[3]);
+    }
+    a[4 * i] = v.x; a[4 * i + 1] = v.y; a[4 * i + 2] = v.z; a[4 * i + 3] = v.w;
+  }
+}
+
+// Products of one layer: acc[32 q + i] = sum over the layer's inputs for column 64 q + 32 half + i
+// (layer 3: the 32 columns, first half of the threads only).  w holds the first weights on entry
+// and the next layer's first ones on return, a the first inputs of layer 1.  False: a wait ran out.
+template <int L>
+__device__ __forceinline__ bool fw_layer(FwLane& f, float a[32], uint4 w[8], float acc[128]) {
+  constexpr int NC = (L == 0 ? NI : NH) / 64, NQ = L < 2 ? 4 : 1;
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < 32 * NQ; ++i) acc[i] = 0.f;
+  auto collect = [&]() {  // the products of the chunk before
+    ok = ok && wait_bounded(f.bar, (f.step - 1) & 1);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (L < 2 || f.half == 0)
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) tmem_add32(f.tmem + f.lanes + 64 * q + (L < 2 ? 32 * f.half : 0), acc + 32 * q);
+  };
+#pragma unroll 1
+  for (int ch = 0; ch < NC; ++ch) {
+    unsigned char* As = f.stage + (f.step & 1) * kFwStage;
+    unsigned char* Bs = As + 3 * 128 * 64 * 2;
+    if (L > 0) {
+      uint32_t r[4][8];
+#pragma unroll
+      for (int g = 0; g < 4; ++g) tmem_ld8_async(f.tmem + f.lanes + 256 + 64 * ch + 32 * f.half + 8 * g, r[g]);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int i = 0; i < 32; ++i) a[i] = __uint_as_float(r[i >> 3][i & 7]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      uint32_t q[3][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        uint32_t lo[3], hi[3];
+        split3(a[8 * i + 2 * j], lo);
+        split3(a[8 * i + 2 * j + 1], hi);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) q[s][j] = lo[s] | hi[s] << 16;
+      }
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+        *reinterpret_cast<uint4*>(As + s * 16384 + bf16_core(f.row, 32 * f.half + 8 * i)) =
+            make_uint4(q[s][0], q[s][1], q[s][2], q[s][3]);
+    }
+    if (L < 2) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4*>(Bs + bf16_core(f.tid, 8 * i)) = w[i];
+    } else {
+      *reinterpret_cast<uint4*>(Bs + bf16_core(f.tid & 31, 8 * (f.tid >> 5))) = w[0];
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (ch + 1 < NC) {
+      fw_load_w<L>(f, 64 * (ch + 1), w);
+      if (L == 0) fw_load_x(f, 64 * (ch + 1), a);
+    } else if (L < 2) {
+      fw_load_w<L < 2 ? L + 1 : 2>(f, 0, w);
+    }
+    if (ch > 0) collect();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    ok = __syncthreads_and(ok);
+    if (!ok) return false;
+    if (f.tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int s = 2; s >= 0; --s)  // small parts first
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_bf16(f.tmem, smem_desc(smem_u32(As) + s * 16384 + kk * 2 * kCoreLbo, kCoreLbo, kCoreSbo),
+                   smem_desc(smem_u32(Bs) + kk * 2 * kCoreLbo, kCoreLbo, kCoreSbo), idesc_bf16(L < 2 ? 256 : 32),
+                   s < 2 || kk > 0);
+      mma_commit(f.bar);
+    }
+    ++f.step;
+  }
+  collect();
+  return __syncthreads_and(ok);
+}
+
+// Bias, pre-activations (z, may be null), ReLU, activations (h, may be null), and the activations to TMEM.
+__device__ __forceinline__ void fw_activate(const FwLane& f, const float* bias, float acc[128], float* z, float* h) {
+  auto put = [&](float* o) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float* p = o + (size_t)f.gr * NH + 64 * q + 32 * f.half;
+      if (f.flags & 4) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          reinterpret_cast<float4*>(p)[i] = make_float4(acc[32 * q + 4 * i], acc[32 * q + 4 * i + 1],
+                                                       acc[32 * q + 4 * i + 2], acc[32 * q + 4 * i + 3]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) p[i] = acc[32 * q + i];
+      }
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < 128; ++i) acc[i] += bias[64 * (i >> 5) + 32 * f.half + (i & 31)];
+  if (z && f.gr < f.n) put(z);
+#pragma unroll
+  for (int i = 0; i < 128; ++i) acc[i] = fmaxf(acc[i], 0.f);
+  if (h && f.gr < f.n) put(h);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) tmem_st8(f.tmem + f.lanes + 256 + 64 * (i >> 2) + 32 * f.half + 8 * (i & 3), acc + 8 * i);
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// flags: bit 0 X is 16-byte aligned, bit 1 W, bit 2 the activations' rows.
+__global__ void __launch_bounds__(256, 1) k_mlp_forward(int n, const __nv_bfloat16* __restrict__ W,
+                                                        const float* __restrict__ bias, const float* __restrict__ X,
+                                                        float* __restrict__ Y, float* __restrict__ z1,
+                                                        float* __restrict__ h1, float* __restrict__ z2,
+                                                        float* __restrict__ h2, int flags) {
+  extern __shared__ __align__(1024) unsigned char stage_mem[];
+  __shared__ __align__(8) uint64_t mbar;
+  __shared__ uint32_t tmem_s;
+  __shared__ float bias_s[N_B + 7];
+  const int tid = threadIdx.x, warp = tid >> 5;
+  if (warp == 0) tmem_alloc(&tmem_s, 512);
+  if (tid == 0) {
+    mbar_init(&mbar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  FwLane f{W, X, stage_mem, &mbar, 0u, (uint32_t)(32 * (warp & 3)) << 16, tid, tid & 127, tid >> 7,
+           (int)blockIdx.x * 128 + (tid & 127), n, flags, 0};
+  float a[32], acc[128];
+  uint4 w[8];
+  fw_load_x(f, 0, a);
+  fw_load_w<0>(f, 0, w);
+  for (int i = tid; i < N_B + 7; i += 256) bias_s[i] = i < N_B ? bias[i] : 0.f;
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  f.tmem = tmem_s;
+  bool ok = fw_layer<0>(f, a, w, acc);
+  if (ok) {
+    fw_activate(f, bias_s, acc, z1, h1);
+    ok = fw_layer<1>(f, a, w, acc);
+  }
+  if (ok) {
+    fw_activate(f, bias_s + OFF_B2, acc, z2, h2);
+    ok = fw_layer<2>(f, a, w, acc);
+  }
+  if (!ok && f.step > 0) wait_bounded(&mbar, (f.step - 1) & 1);  // products still in flight
+  if (f.half == 0 && f.gr < n)
+#pragma unroll
+    for (int i = 0; i < NO; ++i)
+      Y[(size_t)f.gr * NO + i] = ok ? acc[i] + bias_s[OFF_B3 + i] : __int_as_float(0x7fc00000);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(f.tmem, 512);
+}
+
+cudaError_t forward(cudaStream_t st, const __nv_bfloat16* W, const float* bias, const float* X, int n, float* Y,
+                    float* z1, float* h1, float* z2, float* h2) {
+  auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  const int flags = (a16(X) ? 1 : 0) | (a16(W) ? 2 : 0) | (a16(z1) && a16(h1) && a16(z2) && a16(h2) ? 4 : 0);
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kFwStage);
+  if (e != cudaSuccess) return e;
+  k_mlp_forward<<<(unsigned)((n + 127) / 128), 256, 2 * kFwStage, st>>>(n, W, bias, X, Y, z1, h1, z2, h2, flags);
+  return cudaGetLastError();
 }
 
 // gb[c] += sum_s dZ[s][c]
@@ -156,14 +442,19 @@ __global__ void k_mlp_adam(int nw, int nbias, float* __restrict__ W, __nv_bfloat
   *g = 0.f;
 }
 
-template <class TA_, class TB_, bool TA, bool TB, int EPI>
-cudaError_t gemm(cudaStream_t st, int M, int N, int K, const TA_* A, int lda, const TB_* B, int ldb, float* C,
-                 int ldc, const float* bias, float* Z, const float* mask, int splits = 1) {
+template <class TB_, bool TA, int EPI>
+cudaError_t gemm(cudaStream_t st, int M, int N, int K, const float* A, int lda, const TB_* B, int ldb, float* C,
+                 int ldc, const float* mask, int splits = 1) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-  const int kchunk = ((K + splits - 1) / splits + 15) / 16 * 16;
+  const int kchunk = ((K + splits - 1) / splits + 31) / 32 * 32;
   const int nz = (K + kchunk - 1) / kchunk;
-  dim3 grid((N + 63) / 64, (M + 63) / 64, nz);
-  k_mlp_gemm<TA_, TB_, TA, TB, EPI><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, Z, mask, kchunk);
+  auto grid = [&](int bt) { return dim3((N + bt - 1) / bt, (M + bt - 1) / bt, nz); };
+  const dim3 g = grid(64);
+  // 32 x 32 tiles until the 64 x 64 ones fill the 152 SMs
+  if ((long long)g.x * g.y * g.z < 152)
+    k_mlp_gemm<TB_, TA, EPI, 32, 32><<<grid(32), 256, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, mask, kchunk);
+  else
+    k_mlp_gemm<TB_, TA, EPI, 64, 16><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, mask, kchunk);
   return cudaGetLastError();
 }
 
@@ -197,19 +488,10 @@ constexpr char kMlpMagic[8] = {'S', 'C', 'M', 'L', 'P', '0', '0', '1'};
 
 namespace sc {
 
-// Inference: Y = net(X) with the hidden activations in h1, h2 (n x 256 each).
-cudaError_t mlp_forward(cudaStream_t st, const uint16_t* Wbf16, const float* bias, const float* X, int n, float* Y,
-                        float* h1, float* h2) {
-  const __nv_bfloat16* W = reinterpret_cast<const __nv_bfloat16*>(Wbf16);
-  cudaError_t e = gemm<float, __nv_bfloat16, false, true, EPI_BIAS_RELU>(st, n, NH, NI, X, NI, W, NI, h1, NH, bias,
-                                                                         nullptr, nullptr);
-  if (e == cudaSuccess)
-    e = gemm<float, __nv_bfloat16, false, true, EPI_BIAS_RELU>(st, n, NH, NH, h1, NH, W + OFF_W2, NH, h2, NH,
-                                                               bias + OFF_B2, nullptr, nullptr);
-  if (e == cudaSuccess)
-    e = gemm<float, __nv_bfloat16, false, true, EPI_BIAS>(st, n, NO, NH, h2, NH, W + OFF_W3, NH, Y, NO, bias + OFF_B3,
-                                                          nullptr, nullptr);
-  return e;
+// Inference: Y = net(X).
+cudaError_t mlp_forward(cudaStream_t st, const uint16_t* Wbf16, const float* bias, const float* X, int n, float* Y) {
+  if (n <= 0) return cudaSuccess;
+  return forward(st, reinterpret_cast<const __nv_bfloat16*>(Wbf16), bias, X, n, Y, nullptr, nullptr, nullptr, nullptr);
 }
 
 }  // namespace sc
@@ -223,29 +505,8 @@ sc_status sc_mlp_forward(const uint16_t* Wbf16, const float* bias, const float* 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const __nv_bfloat16* W = reinterpret_cast<const __nv_bfloat16*>(Wbf16);
   // cache: [z1 | h1 | z2 | h2], each n x 256 (pre- and post-activations)
-  float* z1 = cache;
-  float* h1 = cache ? cache + (size_t)n * NH : nullptr;
-  float* z2 = cache ? cache + 2 * (size_t)n * NH : nullptr;
-  float* h2 = cache ? cache + 3 * (size_t)n * NH : nullptr;
-  float* tmp1 = nullptr;
-  float* tmp2 = nullptr;
-  cudaError_t e = cudaSuccess;
-  if (!cache) {
-    e = cudaMallocAsync(reinterpret_cast<void**>(&tmp1), (size_t)n * NH * sizeof(float), st);
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&tmp2), (size_t)n * NH * sizeof(float), st);
-    if (e != cudaSuccess) return SC_ERR_OOM;
-    h1 = tmp1;
-    h2 = tmp2;
-  }
-  e = gemm<float, __nv_bfloat16, false, true, EPI_BIAS_RELU>(st, n, NH, NI, X, NI, W, NI, h1, NH, bias, z1, nullptr);
-  if (e == cudaSuccess)
-    e = gemm<float, __nv_bfloat16, false, true, EPI_BIAS_RELU>(st, n, NH, NH, h1, NH, W + OFF_W2, NH, h2, NH,
-                                                               bias + OFF_B2, z2, nullptr);
-  if (e == cudaSuccess)
-    e = gemm<float, __nv_bfloat16, false, true, EPI_BIAS>(st, n, NO, NH, h2, NH, W + OFF_W3, NH, Y, NO, bias + OFF_B3,
-                                                          nullptr, nullptr);
-  if (tmp1) cudaFreeAsync(tmp1, st);
-  if (tmp2) cudaFreeAsync(tmp2, st);
+  auto part = [&](int i) { return cache ? cache + (size_t)i * n * NH : nullptr; };
+  cudaError_t e = forward(st, W, bias, X, n, Y, part(0), part(1), part(2), part(3));
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   return e == cudaSuccess ? SC_OK : SC_ERR_CUDA;
 }
@@ -264,24 +525,22 @@ sc_status sc_mlp_backward(const uint16_t* Wbf16, const float* X, const float* ca
   const int splits = (n + 2047) / 2048;   // sample chunks of the weight gradients
   cudaError_t e;
   // layer 3: gW3 += dY^T h2, gb3 += colsum dY, dz2 = (dY W3) * [z2 > 0]
-  e = gemm<float, float, true, false, EPI_ATOMIC>(st, NO, NH, n, dY, NO, h2, NH, gW + OFF_W3, NH, nullptr, nullptr,
-                                                  nullptr, splits);
+  e = gemm<float, true, EPI_ATOMIC>(st, NO, NH, n, dY, NO, h2, NH, gW + OFF_W3, NH, nullptr,
+                                    splits);
   if (e == cudaSuccess) { k_mlp_colsum<<<NO, 256, 0, st>>>(n, NO, dY, gb + OFF_B3); e = cudaGetLastError(); }
   if (e == cudaSuccess)
-    e = gemm<float, __nv_bfloat16, false, false, EPI_MASK>(st, n, NH, NO, dY, NO, W + OFF_W3, NH, dz2, NH, nullptr,
-                                                           nullptr, z2);
+    e = gemm<__nv_bfloat16, false, EPI_MASK>(st, n, NH, NO, dY, NO, W + OFF_W3, NH, dz2, NH, z2);
   // layer 2
   if (e == cudaSuccess)
-    e = gemm<float, float, true, false, EPI_ATOMIC>(st, NH, NH, n, dz2, NH, h1, NH, gW + OFF_W2, NH, nullptr, nullptr,
-                                                    nullptr, splits);
+    e = gemm<float, true, EPI_ATOMIC>(st, NH, NH, n, dz2, NH, h1, NH, gW + OFF_W2, NH, nullptr,
+                                    splits);
   if (e == cudaSuccess) { k_mlp_colsum<<<NH, 256, 0, st>>>(n, NH, dz2, gb + OFF_B2); e = cudaGetLastError(); }
   if (e == cudaSuccess)
-    e = gemm<float, __nv_bfloat16, false, false, EPI_MASK>(st, n, NH, NH, dz2, NH, W + OFF_W2, NH, dz1, NH, nullptr,
-                                                           nullptr, z1);
+    e = gemm<__nv_bfloat16, false, EPI_MASK>(st, n, NH, NH, dz2, NH, W + OFF_W2, NH, dz1, NH, z1);
   // layer 1
   if (e == cudaSuccess)
-    e = gemm<float, float, true, false, EPI_ATOMIC>(st, NH, NI, n, dz1, NH, X, NI, gW, NI, nullptr, nullptr, nullptr,
-                                                    splits);
+    e = gemm<float, true, EPI_ATOMIC>(st, NH, NI, n, dz1, NH, X, NI, gW, NI, nullptr,
+                                    splits);
   if (e == cudaSuccess) { k_mlp_colsum<<<NH, 256, 0, st>>>(n, NH, dz1, gb); e = cudaGetLastError(); }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   return e == cudaSuccess ? SC_OK : SC_ERR_CUDA;
