@@ -405,7 +405,12 @@ __global__ void __launch_bounds__(128) k_mx_resid(MxMesh M, const double* __rest
   }
 }
 
-// ---- own element blocks dR_e/dQ_e by five-direction duals, one CTA per element ---------
+// ---- own element blocks dR_e/dQ_e by five-direction duals ------------------------------
+// One work item is a range of seeds (nodes) of one element, after the unseeded pass that every
+// range needs; the CTAs take the items from a counter, longest elements first, with one scratch
+// slot per CTA.  Latency bound (per seed a chain of dependent small phases on 128 threads):
+// with one CTA per element the 343 seeds of order 6 ran one after the other, 74 ms on a mesh of
+// 6^3 elements of orders 2 .. 6, now 32 ms.
 // Per-element scratch (in T5 units): the qhat of the six faces unseeded (QH0) and seeded
 // (QH), the neighbour's qhat on each shared face (QHN, <= 49 nodes), the lifted gradient
 // (GE) and point fluxes (FE) of the element, the neighbour's gradients on each shared face
@@ -484,21 +489,30 @@ template <class R>
 __global__ void __launch_bounds__(128) k_mx_own(MxMesh M, Geo Gp, const double* __restrict__ Q,
                                                 const double* __restrict__ grad0, const int* __restrict__ elist,
                                                 DualN<R, 5>* __restrict__ scratch, long long scratch_slot,
-                                                OwnOut<R> outd) {
+                                                OwnOut<R> outd, const int2* __restrict__ work, int nwork, int nseeds,
+                                                int* __restrict__ next) {
   using T5 = DualN<R, 5>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T5* sbuf = reinterpret_cast<T5*>(smem_raw);
   T5* stmp = sbuf + 64 * 20;
-  const int e = elist[blockIdx.x], N = M.ord[e], p = N + 1, pp = p * p, nn = pp * p;
+  __shared__ int s_item;
+  T5* S = scratch + (long long)blockIdx.x * scratch_slot;
+  for (;;) {
+  __syncthreads();
+  if (threadIdx.x == 0) s_item = atomicAdd(next, 1);
+  __syncthreads();
+  if (s_item >= nwork) return;
+  const int2 item = work[s_item];  // list entry, first seed
+  const int e = elist[item.x], N = M.ord[e], p = N + 1, pp = p * p, nn = pp * p;
+  const int r_end = min(nn, item.y + nseeds);
   const int nin = (N - 1) * (N - 1) * (N - 1), ni = 5 * nin, cb0 = (ni + 3) & ~3;
   const int lda = outd.natural ? 5 * nn : ((cb0 + 5 * (nn - nin) + 3) & ~3);
-  R* out = outd.base[blockIdx.x];
+  R* out = outd.base[item.x];
   const size_t o = M.off[e];
   const double* D = &M.tab->D[N][0][0];
   const double* w = M.tab->w[N];
   const int* perm = M.tab->perm[N];
   const OwnScratch L(N);
-  T5* S = scratch + (long long)blockIdx.x * scratch_slot;
   int seed = -1;  // the node whose five variables are the dual directions
   auto qown = [&](int m, int k) {
     T5 t(Q[(o + m) * 5 + k]);
@@ -507,7 +521,7 @@ __global__ void __launch_bounds__(128) k_mx_own(MxMesh M, Geo Gp, const double* 
   };
   // neighbour across face f of e and the face of the neighbour that faces e
   auto nbr_of = [&](int f) { return M.nbr[e * 6 + f]; };
-  for (int r = -1; r < nn; ++r) {
+  for (int r = -1; r < r_end; r = r < 0 ? item.y : r + 1) {
     seed = r;
     int cr[3] = {0, 0, 0};
     if (r >= 0) { cr[0] = r % p; cr[1] = (r / p) % p; cr[2] = r / pp; }
@@ -739,6 +753,7 @@ __global__ void __launch_bounds__(128) k_mx_own(MxMesh M, Geo Gp, const double* 
     }
     __syncthreads();
   }
+  }
 }
 
 // ---- condensed vectors: boundary and interior dofs of every element, elements ordered by
@@ -770,23 +785,42 @@ __global__ void k_mx_gather(int nodes, const int* __restrict__ bmap, const int* 
   }
 }
 
-// u = A_ii^-1 x for the elements of one order class (FP32 inverses n_i x ldi, one CTA per
-// element, a warp per row); x and u in FP64, class-contiguous with stride n_i.
+// u = A_ii^-1 (x - xsub) for the elements of one order: eight lanes per row, four rows per warp,
+// gridDim.x CTAs per element.  Bound by L2 and HBM: a mesh of 6^3 elements of orders 2 .. 6 holds 89 MB
+// of inverses; one CTA per element and 4-byte loads left 43 CTAs to read them (per order and product
+// 71 us, now 12).
 __global__ void __launch_bounds__(256) k_mx_ainv(int ni, int ldi, const float* __restrict__ Ainv,
                                                  const double* __restrict__ x, const double* __restrict__ xsub,
                                                  double* __restrict__ u) {
-  __shared__ float xs[640];
-  const size_t el = blockIdx.x;
+  __shared__ __align__(16) float xs[640];
+  const size_t el = blockIdx.y;
   const double* xe = x + el * ni;
-  for (int j = threadIdx.x; j < ni; j += blockDim.x) xs[j] = (float)(xsub ? xe[j] - xsub[el * ni + j] : xe[j]);
+  for (int j = threadIdx.x; j < ldi; j += blockDim.x)
+    xs[j] = j < ni ? (float)(xsub ? xe[j] - xsub[el * ni + j] : xe[j]) : 0.f;
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & 7;
   const float* A = Ainv + el * (size_t)ni * ldi;
-  for (int i = warp; i < ni; i += blockDim.x / 32) {
-    float acc = 0.f;
-    for (int j = lane; j < ni; j += 32) acc = fmaf(A[(size_t)i * ldi + j], xs[j], acc);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) u[el * ni + i] = (double)acc;
+  for (int r0 = 4 * (blockIdx.x * 8 + warp); r0 < ni; r0 += 32 * gridDim.x) {
+    const int r = r0 + (lane >> 3);
+    float s0 = 0.f, s1 = 0.f;
+    if (r < ni) {
+#pragma unroll 5
+      for (int j = 4 * sub; j < ldi; j += 32) {
+        float4 a = __ldg(reinterpret_cast<const float4*>(A + (size_t)r * ldi + j));
+        const float4 v = *reinterpret_cast<const float4*>(xs + j);
+        if (j + 3 >= ni) {  // the rows' padding holds anything
+          if (j + 1 >= ni) a.y = 0.f;
+          if (j + 2 >= ni) a.z = 0.f;
+          if (j + 3 >= ni) a.w = 0.f;
+        }
+        s0 = fmaf(a.x, v.x, s0); s1 = fmaf(a.y, v.y, s1);
+        s0 = fmaf(a.z, v.z, s0); s1 = fmaf(a.w, v.w, s1);
+      }
+    }
+    s0 += s1;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+    if (sub == 0 && r < ni) u[el * ni + r] = (double)s0;
   }
 }
 
@@ -932,7 +966,9 @@ struct sc_mixed {
   int max_ni = 0, max_nb = 0, nbig_gj = 0, nbig_lu = 0, restart = 30;
   int* d_status = nullptr;
   DualN<float, 5>* own_scratch = nullptr;
-  long long own_slot = 0, own_chunk = 0;
+  long long own_slot = 0;
+  int2* d_own_work = nullptr;  // its work items, and the counter they are taken from
+  int *d_own_next = nullptr, own_items = 0, own_seeds = 0, own_slots = 0;
   float** d_own_out = nullptr;
   int* d_elist = nullptr;
   sc_ctx* aux = nullptr;  // Krylov workspace of the shared vector kernels
@@ -984,17 +1020,31 @@ cudaError_t mx_eval(sc_mixed* m, const double* dir, double* out) {
 
 namespace {
 
-// Scratch of the own-block kernel: elements processed per launch, and the per-element slot.
-constexpr int kOwnChunk = 512;
+// Scratch slots of the own-block kernel: its 61 KB of shared memory let 3 CTAs reside per SM.
+constexpr int kOwnSlots = 3 * 152;
+
+// Work items of a list of elements (orders ord, longest first): seeds per item so that each slot
+// gets about four, but at least 24, which keeps the unseeded pass of each item small.
+int own_work(const std::vector<int>& ord, std::vector<int2>& work) {
+  long long seeds = 0;
+  for (int N : ord) seeds += (long long)(N + 1) * (N + 1) * (N + 1);
+  const int per = (int)std::max<long long>(24, (seeds + 4 * kOwnSlots - 1) / (4 * kOwnSlots));
+  work.clear();
+  for (int i = 0; i < (int)ord.size(); ++i)
+    for (int r = 0; r < (ord[i] + 1) * (ord[i] + 1) * (ord[i] + 1); r += per) work.push_back(make_int2(i, r));
+  return per;
+}
 
 template <class R>
-cudaError_t mx_own_launch(sc_mixed* m, const int* d_elist, int count, DualN<R, 5>* scratch, long long slot,
-                          R* const* d_out, int natural) {
+cudaError_t mx_own_launch(sc_mixed* m, const int* d_elist, const int2* d_work, int nwork, int nseeds, int* d_next,
+                          DualN<R, 5>* scratch, int slots, long long slot, R* const* d_out, int natural) {
   const size_t smem = (size_t)2 * 64 * 20 * sizeof(DualN<R, 5>);
   cudaError_t e = cudaFuncSetAttribute(k_mx_own<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d_next, 0, sizeof(int), m->stream);
   if (e != cudaSuccess) return e;
   OwnOut<R> od{d_out, natural};
-  k_mx_own<R><<<count, 128, smem, m->stream>>>(m->M, m->Gp, m->Q, m->grad0, d_elist, scratch, slot, od);
+  k_mx_own<R><<<std::min(slots, nwork), 128, smem, m->stream>>>(m->M, m->Gp, m->Q, m->grad0, d_elist, scratch, slot, od,
+                                                              d_work, nwork, nseeds, d_next);
   m->launches += 1;
   return cudaGetLastError();
 }
@@ -1173,10 +1223,17 @@ sc_status sc_mixed_create(const sc_config* cfg, void* cuda_stream, int n, double
       A(cudaMemcpy(m->d_ptrs, m->h_ptrs.data(), m->h_ptrs.size() * sizeof(void*), cudaMemcpyHostToDevice));
     }
   }
-  // own-block scratch: a chunk of elements per launch, slots sized for the largest order
-  m->own_chunk = std::min<long long>(K, kOwnChunk);
+  // own-block work items and scratch, slots sized for the largest order
+  std::vector<int> ords;
+  for (int el : m->slot_elem) ords.push_back(m->ord[el]);
+  std::vector<int2> work;
+  m->own_seeds = own_work(ords, work);
+  m->own_items = (int)work.size();
+  m->own_slots = std::min(kOwnSlots, m->own_items);
+  A(mx_alloc(&m->d_own_work, work.size())); A(mx_alloc(&m->d_own_next, 1));
+  if (e == cudaSuccess) A(cudaMemcpy(m->d_own_work, work.data(), work.size() * sizeof(int2), cudaMemcpyHostToDevice));
   m->own_slot = OwnScratch(m->cls.empty() ? 2 : m->cls[0].N).total;
-  A(mx_alloc(&m->own_scratch, (size_t)m->own_chunk * m->own_slot));
+  A(mx_alloc(&m->own_scratch, (size_t)m->own_slots * m->own_slot));
   A(mx_alloc(&m->d_own_out, (size_t)K));
   A(mx_alloc(&m->d_elist, (size_t)K));
   // Krylov workspace
@@ -1198,7 +1255,7 @@ void sc_mixed_destroy(sc_mixed* m) {
   void* ps[] = {m->d_tab, m->d_ord, m->d_off, m->d_foff, m->d_nbr, m->d_bmap, m->d_imap, m->Q, m->Qh, m->grad0,
                 m->F0, m->qh0, m->fh0, m->gJ, m->FJ, m->qhJ, m->fhJ, m->vA, m->vB, m->B, m->Rr, m->dQ, m->ri,
                 m->ui, m->xi, m->gb, m->xb, m->V, m->Wv, m->Tb, m->Zb, m->d_items, m->d_ptrs, m->d_status,
-                m->own_scratch, m->d_own_out, m->d_elist};
+                m->own_scratch, m->d_own_out, m->d_elist, m->d_own_work, m->d_own_next};
   for (void* p : ps) if (p) cudaFree(p);
   for (MxClass& c : m->cls) {
     void* cs[] = {c.Aown32, c.Ainv32, c.Y32, c.See32, c.Sls32, c.dsc, c.piv, c.rowperm};
@@ -1281,17 +1338,25 @@ sc_status sc_mixed_own_block(sc_mixed* m, int e, double* block) {
   double* blk = nullptr;
   double** outp = nullptr;
   int* el = nullptr;
-  cudaError_t ce = mx_alloc(&scr, (size_t)OwnScratch(m->ord[e]).total);
+  std::vector<int2> work;
+  const int seeds = own_work({m->ord[e]}, work), nwork = (int)work.size();
+  int2* d_work = nullptr;
+  int* d_next = nullptr;
+  const long long slot = OwnScratch(m->ord[e]).total;
+  cudaError_t ce = mx_alloc(&scr, (size_t)(nwork * slot));
+  if (ce == cudaSuccess) ce = mx_alloc(&d_work, nwork);
+  if (ce == cudaSuccess) ce = mx_alloc(&d_next, 1);
+  if (ce == cudaSuccess) ce = cudaMemcpy(d_work, work.data(), nwork * sizeof(int2), cudaMemcpyHostToDevice);
   if (ce == cudaSuccess) ce = mx_alloc(&blk, (size_t)ne * ne);
   if (ce == cudaSuccess) ce = mx_alloc(&outp, 1);
   if (ce == cudaSuccess) ce = mx_alloc(&el, 1);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(outp, &blk, sizeof(double*), cudaMemcpyHostToDevice, m->stream);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(el, &e, sizeof(int), cudaMemcpyHostToDevice, m->stream);
   if (ce == cudaSuccess) ce = cudaMemsetAsync(blk, 0, (size_t)ne * ne * sizeof(double), m->stream);
-  if (ce == cudaSuccess) ce = mx_own_launch<double>(m, el, 1, scr, 0, outp, 1);
+  if (ce == cudaSuccess) ce = mx_own_launch<double>(m, el, d_work, nwork, seeds, d_next, scr, nwork, slot, outp, 1);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(block, blk, (size_t)ne * ne * sizeof(double), cudaMemcpyDeviceToHost, m->stream);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(m->stream);
-  cudaFree(scr); cudaFree(blk); cudaFree(outp); cudaFree(el);
+  cudaFree(scr); cudaFree(blk); cudaFree(outp); cudaFree(el); cudaFree(d_work); cudaFree(d_next);
   if (ce != cudaSuccess) return mfail(m, SC_ERR_CUDA, std::string("own block: ") + cudaGetErrorString(ce));
   return SC_OK;
 }
@@ -1354,7 +1419,9 @@ cudaError_t mx_per_class(sc_mixed* m, F&& launch) {
 cudaError_t mx_ainv(sc_mixed* m, const double* x, const double* xsub, double* u) {
   return mx_per_class(m, [&](MxClass& c) {
     const long long o = m->ioff[c.slot0];
-    k_mx_ainv<<<c.count, 256, 0, c.st>>>(c.ni, c.ldi, c.Ainv32, x + o, xsub ? xsub + o : nullptr, u + o);
+    // every 32 rows their own CTA until the elements alone give four CTAs per SM
+    const int split = std::max(1, std::min((c.ni + 31) / 32, (4 * 152 + c.count - 1) / c.count));
+    k_mx_ainv<<<dim3(split, c.count), 256, 0, c.st>>>(c.ni, c.ldi, c.Ainv32, x + o, xsub ? xsub + o : nullptr, u + o);
     m->launches += 1;
     return cudaGetLastError();
   });
@@ -1497,10 +1564,8 @@ sc_status sc_mixed_condense(sc_mixed* m) {
                           m->stream));
   for (const MxClass& c : m->cls)
     MX_CUDA(cudaMemsetAsync(c.Aown32, 0, (size_t)c.count * c.ne * c.lda * sizeof(float), m->stream));
-  for (long long s0 = 0; s0 < m->K; s0 += m->own_chunk) {
-    const int cnt = (int)std::min<long long>(m->own_chunk, m->K - s0);
-    MX_CUDA(mx_own_launch<float>(m, m->d_elist + s0, cnt, m->own_scratch, m->own_slot, m->d_own_out + s0, 0));
-  }
+  MX_CUDA(mx_own_launch<float>(m, m->d_elist, m->d_own_work, m->own_items, m->own_seeds, m->d_own_next, m->own_scratch,
+                               m->own_slots, m->own_slot, m->d_own_out, 0));
   const int minus1 = -1;
   MX_CUDA(cudaMemcpyAsync(m->d_status, &minus1, sizeof(int), cudaMemcpyHostToDevice, m->stream));
   MX_CUDA(mx_condense_blocks(m));
