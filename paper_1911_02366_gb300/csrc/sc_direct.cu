@@ -4,23 +4,25 @@
 // (Tables tab:Advantages and tab:Advantages2; it uses a sparse direct solver on the CPU).
 //
 // Forming the dense matrices: A from the own element blocks and the neighbour couplings
-// (scatter); S column by column through the condensed operator (S e_j), the system the
+// (scatter); S through the condensed operator (S e_j, 32 columns at a time), the system the
 // condensation forms.  LU with partial pivoting (the first row of largest |a| wins), right
 // looking in panels of 64 columns:
-//   per column j of a panel: pivot search (block partial maxima, then one block), the row
-//   interchange over the whole row, scaling of column j and the rank-1 update of the rest of
-//   the panel;
+//   per half panel of 32 columns: one thread-block cluster with the rows in shared memory, then its
+//   interchanges on the other columns (matrices with more rows than a cluster holds: column by
+//   column, pivot search, interchange, scaling and rank-1 update in four kernels);
 //   per panel: U12 = L11^-1 A12 (unit lower triangle in shared memory, 32-column tiles), then
 //   the trailing update A22 -= L21 U12 on the TF32 tensor cores (mixed arm, tensor_cores) or
 //   the CUDA cores (64 x 64 tiles; FP64 on the FP64 arm).
 // Solves: the row interchanges as one gather, then blocked forward and backward
-// substitution (64-row blocks: off-diagonal dot products by 32 warps, the 64 x 64 triangle
-// by one warp).  The mixed arm stores the factors in FP32 and refines in FP64 on the global
+// substitution, one launch per 64-row block (the triangle, then its update of all rows left).  The mixed arm stores the factors in FP32 and refines in FP64 on the global
 // residual B - A dQ until rel_tol.
 #include <algorithm>
 #include <cmath>
 #include <string>
+#include <type_traits>
 #include <vector>
+
+#include <cooperative_groups.h>
 
 #include "sc_internal.cuh"
 
@@ -34,6 +36,7 @@ namespace {
 
 constexpr int kPanel = 64;
 constexpr int kPivBlocks = 152;
+constexpr int kColumns = 32;  // columns of S formed at a time
 
 inline unsigned cdivu(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
@@ -69,18 +72,24 @@ __global__ void k_dense_cross(Geo G, const double* __restrict__ X, const int* __
   atomicAdd(&D[row * ldd + col], (T)X[(size_t)e * per + ((size_t)k * G.NP + p) * 5 + l]);
 }
 
-__global__ void k_unit_vec(double* x, long long on, long long off) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    if (off >= 0) x[off] = 0.0;
-    x[on] = 1.0;
-  }
+// Unit vectors e_j, j = j0 .. j0 + m - 1, one behind the other (n values each).
+template <class T>
+__global__ void k_unit_vecs(T* __restrict__ x, int n, int j0, int m) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t < (long long)n * m) x[t] = t % n == j0 + t / n ? T(1) : T(0);
 }
 
-// D[:, j] = col (n entries).
+// Columns j0 .. j0 + m - 1 of D from the vectors col[i] (n values each): 32 x 32 tiles.
 template <class T>
-__global__ void k_put_column(const double* __restrict__ col, int n, int j, T* __restrict__ D, long long ldd) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) D[(long long)i * ldd + j] = (T)col[i];
+__global__ void __launch_bounds__(256) k_put_columns(const double* __restrict__ col, int n, int j0, int m,
+                                                     T* __restrict__ D, long long ldd) {
+  __shared__ T tile[32][33];
+  const int r0 = 32 * blockIdx.x, lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i < m; i += 8)
+    if (r0 + lane < n) tile[i][lane] = (T)col[(long long)i * n + r0 + lane];
+  __syncthreads();
+  for (int r = threadIdx.x >> 5; r < 32 && r0 + r < n; r += 8)
+    if (lane < m) D[(long long)(r0 + r) * ldd + j0 + lane] = tile[lane][r];
 }
 
 // ---- LU with partial pivoting -------------------------------------------------------
@@ -155,6 +164,143 @@ __global__ void k_panel_col(T* __restrict__ D, long long ldd, int n, int j, int 
   }
 }
 
+// Panel of pw <= 32 columns from k0 on by one cluster: CTA i keeps the panel rows i rpc .. (relative
+// to k0) in shared memory.  Per column every CTA sends its best pivot candidate, with its row,
+// to all CTAs (and the first CTA row j, which gives way), so that one cluster barrier per column
+// suffices: afterwards all know the pivot row, the two owners exchange the rows, and every thread
+// updates its rows and looks for the next column's candidate on the way.  The interchanges of the
+// other columns follow in k_swap_cols.  Bound by the 16 SMs' FP64 rate and the barriers: about 0.1 ms for
+// 7560 rows in FP64 against 32 columns x 4 launches, 25 us each (the same operations, one kernel each).
+constexpr int kLuW = 32;
+template <class T>
+__global__ void __launch_bounds__(512) k_lu_panel_cluster(T* __restrict__ D, long long ldd, int n, int k0, int pw,
+                                                          int rpc, int* __restrict__ piv, int* __restrict__ status) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int LD = kLuW + 1;
+  T* a = reinterpret_cast<T*>(smem_raw);  // [rpc][LD]
+  __shared__ T pub[2][17][kLuW];          // candidates' rows by rank; 16: row j
+  __shared__ double cval[2][16];
+  __shared__ int crow[2][16];
+  __shared__ double wval[16];
+  __shared__ int wrow[16];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = (int)cl.block_rank(), ncta = (int)cl.num_blocks();
+  const int first = rank * rpc, mine = max(0, min(rpc, n - k0 - first));
+  for (int i = tid; i < mine * kLuW; i += 512) {
+    const int r = i / kLuW, c = i % kLuW;
+    a[r * LD + c] = c < pw ? D[(long long)(k0 + first + r) * ldd + k0 + c] : T(0);
+  }
+  __syncthreads();
+  double best = -1.0;
+  int brow = 1 << 30;
+  for (int r = tid; r < mine; r += 512) {
+    const double v = fabs((double)a[r * LD]);
+    if (v > best) { best = v; brow = first + r; }
+  }
+  for (int j = 0; j < pw; ++j) {
+    const int par = j & 1;
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int orow = __shfl_xor_sync(0xffffffffu, brow, o);
+      if (ov > best || (ov == best && orow < brow)) { best = ov; brow = orow; }
+    }
+    if (lane == 0) { wval[warp] = best; wrow[warp] = brow; }
+    __syncthreads();
+    best = wval[0];
+    brow = wrow[0];
+    for (int w = 1; w < 16; ++w)
+      if (wval[w] > best || (wval[w] == best && wrow[w] < brow)) { best = wval[w]; brow = wrow[w]; }
+    if (warp < ncta) {  // warp w writes to CTA w
+      if (best >= 0.0) *cl.map_shared_rank(&pub[par][rank][lane], warp) = a[(brow - first) * LD + lane];
+      if (lane == 0) {
+        *cl.map_shared_rank(&cval[par][rank], warp) = best;
+        *cl.map_shared_rank(&crow[par][rank], warp) = brow;
+      }
+      if (rank == 0) *cl.map_shared_rank(&pub[par][16][lane], warp) = a[j * LD + lane];
+    }
+    cl.sync();
+    double pv = -1.0;
+    int p = 1 << 30, q = 0;
+    for (int i = 0; i < ncta; ++i)
+      if (cval[par][i] > pv || (cval[par][i] == pv && crow[par][i] < p)) { pv = cval[par][i]; p = crow[par][i]; q = i; }
+    const bool none = !(pv > 0.0);  // zero (or NaN) column: record the first such column, keep the row
+    if (none) p = j;
+    if (rank == 0 && tid == 0) {
+      piv[k0 + j] = k0 + p;
+      if (none && status[0] < 0) status[0] = k0 + j;
+    }
+    const T* prow = p == j ? pub[par][16] : pub[par][q];
+    if (p != j) {
+      if (q == rank && tid < kLuW) a[(p - first) * LD + tid] = pub[par][16][tid];
+      if (rank == 0 && tid >= 32 && tid < 32 + kLuW) a[j * LD + tid - 32] = prow[tid - 32];
+    }
+    __syncthreads();
+    const T pivot = prow[j], inv = pivot == T(0) ? T(0) : T(1) / pivot;
+    best = -1.0;
+    brow = 1 << 30;
+    for (int r = tid; r < mine; r += 512) {
+      if (first + r <= j) continue;
+      T* row = a + r * LD;
+      if (pivot != T(0)) {
+        const T l = row[j] * inv;
+        row[j] = l;
+#pragma unroll 8
+        for (int c = j + 1; c < kLuW; ++c) row[c] -= l * prow[c];
+      }
+      if (j + 1 < pw) {
+        const double v = fabs((double)row[j + 1]);
+        if (v > best) { best = v; brow = first + r; }
+      }
+    }
+  }
+  cl.sync();  // nobody leaves while others may still write to it
+  for (int i = tid; i < mine * kLuW; i += 512) {
+    const int r = i / kLuW, c = i % kLuW;
+    if (c < pw) D[(long long)(k0 + first + r) * ldd + k0 + c] = a[r * LD + c];
+  }
+}
+
+// The interchanges k0 + j <-> piv[k0 + j], j < pw <= 32, on all columns outside the panel: one warp works out
+// where the at most 64 rows end up, then each CTA moves 32 columns through shared memory.
+template <class T>
+__global__ void __launch_bounds__(256) k_swap_cols(T* __restrict__ D, long long ldd, int n, int k0, int pw,
+                                                   const int* __restrict__ piv) {
+  __shared__ int row[64], from[64], cnt;
+  __shared__ T tile[64][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp == 0) {
+    int c = pw;
+    if (lane < pw) row[lane] = from[lane] = k0 + lane;
+    __syncwarp();
+    for (int j = 0; j < pw; ++j) {
+      const int p = __ldg(piv + k0 + j);
+      int at = p - k0;  // position of row p in the list
+      if (at >= pw) {
+        const unsigned hit = __ballot_sync(0xffffffffu, pw + lane < c && row[pw + lane] == p);
+        at = hit ? pw + __ffs(hit) - 1 : c;
+        if (!hit) {
+          if (lane == 0) row[c] = from[c] = p;
+          ++c;
+        }
+      }
+      __syncwarp();
+      if (lane == 0) { const int t = from[j]; from[j] = from[at]; from[at] = t; }
+      __syncwarp();
+    }
+    if (lane == 0) cnt = c;
+  }
+  __syncthreads();
+  const int c0 = 32 * blockIdx.x + lane, m = cnt;
+  const bool live = c0 < n && (c0 < k0 || c0 >= k0 + pw);
+  if (live)
+    for (int i = warp; i < m; i += 8) tile[i][lane] = D[(long long)from[i] * ldd + c0];
+  __syncthreads();
+  if (live)
+    for (int i = warp; i < m; i += 8) D[(long long)row[i] * ldd + c0] = tile[i][lane];
+}
+
 // U12 = L11^-1 A12 for columns >= k0 + kb: one CTA per 32-column tile, L11 (unit lower,
 // kb <= 64) and the tile in shared memory, one barrier per eliminated row.
 constexpr int kLdL = kPanel + 1, kLdT = 33;
@@ -203,56 +349,131 @@ __global__ void k_to_double(int n, const T* __restrict__ y, double* __restrict__
   if (i < n) x[i] = (double)y[i];
 }
 
-// One 64-row block of a substitution in place on y: LOWER (unit diagonal, columns left of
-// the block) or upper (diagonal of U, columns right of it).  32 warps form the off-diagonal
-// dot products of the block's rows, then warp 0 solves the 64 x 64 triangle.
+// One 64-row block of a substitution: every CTA solves the triangle (LOWER: unit diagonal; else the
+// diagonal of U) for the block's part of y in its first warp, the first CTA writes the result to
+// x, and the warps subtract the block's columns from the rows of y still to come (below or above; n <=
+// all of them).  A single CTA forming each block's dot products over the whole row took 0.1 ms per
+// block of a matrix of 7560 rows.
 template <class T, bool LOWER>
-__global__ void __launch_bounds__(1024) k_trsv_block(const T* __restrict__ D, long long ldd, int n, int b0, int bs,
-                                                     T* __restrict__ y) {
-  __shared__ T s[kPanel];
+__global__ void __launch_bounds__(256) k_trsv_block(const T* __restrict__ D, long long ldd, int n, int b0, int bs,
+                                                    T* __restrict__ y, T* __restrict__ x) {
+  __shared__ T tri[kPanel][kPanel + 1];
+  __shared__ T xs[kPanel];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c_lo = LOWER ? 0 : b0 + bs, c_hi = LOWER ? b0 : n;
-  for (int r = warp; r < bs; r += 32) {
-    const T* row = D + (long long)(b0 + r) * ldd;
-    T acc = T(0);
-    for (int cc = c_lo + lane; cc < c_hi; cc += 32) acc += row[cc] * y[cc];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) s[r] = y[b0 + r] - acc;
+  for (int i = threadIdx.x; i < bs * bs; i += 256) tri[i / bs][i % bs] = D[(long long)(b0 + i / bs) * ldd + b0 + i % bs];
+  __syncthreads();
+  if (warp == 0) {  // lanes own rows lane and lane + 32 of the block
+    T v0 = lane < bs ? y[b0 + lane] : T(0), v1 = lane + 32 < bs ? y[b0 + lane + 32] : T(0);
+    if (LOWER) {
+      for (int i = 0; i < bs; ++i) {
+        const T xi = __shfl_sync(0xffffffffu, i < 32 ? v0 : v1, i & 31);
+        if (lane > i && lane < bs) v0 -= tri[lane][i] * xi;
+        if (lane + 32 > i && lane + 32 < bs) v1 -= tri[lane + 32][i] * xi;
+      }
+    } else {
+      for (int i = bs - 1; i >= 0; --i) {
+        T xi = __shfl_sync(0xffffffffu, i < 32 ? v0 : v1, i & 31);
+        xi = xi / tri[i][i];
+        if (lane == (i & 31)) { if (i < 32) v0 = xi; else v1 = xi; }
+        if (lane < i) v0 -= tri[lane][i] * xi;
+        if (lane + 32 < i) v1 -= tri[lane + 32][i] * xi;
+      }
+    }
+    xs[lane] = v0;
+    xs[lane + 32] = v1;
+    if (blockIdx.x == 0) {
+      if (lane < bs) x[b0 + lane] = v0;
+      if (lane + 32 < bs) x[b0 + lane + 32] = v1;
+    }
   }
   __syncthreads();
-  if (warp != 0) return;
-  // the triangle: lanes own rows lane and lane + 32 of the block
-  T v0 = lane < bs ? s[lane] : T(0), v1 = lane + 32 < bs ? s[lane + 32] : T(0);
-  if (LOWER) {
-    for (int i = 0; i < bs; ++i) {
-      const T xi = __shfl_sync(0xffffffffu, i < 32 ? v0 : v1, i & 31);
-      const int r0 = lane, r1 = lane + 32;
-      if (r0 > i && r0 < bs) v0 -= D[(long long)(b0 + r0) * ldd + b0 + i] * xi;
-      if (r1 > i && r1 < bs) v1 -= D[(long long)(b0 + r1) * ldd + b0 + i] * xi;
-    }
-  } else {
-    for (int i = bs - 1; i >= 0; --i) {
-      T xi = __shfl_sync(0xffffffffu, i < 32 ? v0 : v1, i & 31);
-      xi = xi / D[(long long)(b0 + i) * ldd + b0 + i];
-      if (lane == (i & 31)) { if (i < 32) v0 = xi; else v1 = xi; }
-      const int r0 = lane, r1 = lane + 32;
-      if (r0 < i) v0 -= D[(long long)(b0 + r0) * ldd + b0 + i] * xi;
-      if (r1 < i) v1 -= D[(long long)(b0 + r1) * ldd + b0 + i] * xi;
-    }
+  const int r0 = LOWER ? b0 + bs : 0, r1 = LOWER ? n : b0;
+  const T x0 = lane < bs ? xs[lane] : T(0), x1 = lane + 32 < bs ? xs[lane + 32] : T(0);
+  for (int r = r0 + blockIdx.x * 8 + warp; r < r1; r += gridDim.x * 8) {
+    const T* row = D + (long long)r * ldd + b0;
+    T acc = T(0);
+    if (lane < bs) acc = row[lane] * x0;
+    if (lane + 32 < bs) acc += row[lane + 32] * x1;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) y[r] -= acc;
   }
-  if (lane < bs) y[b0 + lane] = v0;
-  if (lane + 32 < bs) y[b0 + lane + 32] = v1;
+}
+
+// Cluster size and rows per CTA of the panel kernel for `rows` panel rows; 0: does not fit.  The
+// largest cluster the device can run: 16 where a GPC has room for it, else 8.
+template <class T>
+int panel_cluster(int rows, int* rpc) {
+  constexpr size_t row_bytes = (kLuW + 1) * sizeof(T), cap = 200 * 1024;
+  for (int nc : {16, 8}) {
+    const int need = std::max(kLuW, (rows + nc - 1) / nc);
+    if (need * row_bytes > cap) continue;
+    if (cudaFuncSetAttribute(k_lu_panel_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess ||
+        cudaFuncSetAttribute(k_lu_panel_cluster<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return 0;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nc);
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = need * row_bytes;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = nc;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int active = 0;
+    if (cudaOccupancyMaxActiveClusters(&active, k_lu_panel_cluster<T>, &cfg) == cudaSuccess && active > 0) {
+      *rpc = need;
+      return nc;
+    }
+    (void)cudaGetLastError();
+  }
+  return 0;
 }
 
 template <class T>
 cudaError_t lu_factor(sc_ctx* c, T* D, long long ldd, int n, int* piv, bool tc) {
   double* pval = nullptr;
   int* prow = nullptr;
+  int nc = 0, rpc = 0;  // cluster of the panel kernel, once the rows left fit one
   cudaError_t e = cudaMalloc(&pval, kPivBlocks * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&prow, kPivBlocks * sizeof(int));
   for (int k0 = 0; k0 < n && e == cudaSuccess; k0 += kPanel) {
     const int kb = std::min(kPanel, n - k0), jend = k0 + kb;
-    for (int j = k0; j < jend && e == cudaSuccess; ++j) {
+    if (nc == 0) nc = panel_cluster<T>(n - k0, &rpc);
+    for (int ks = k0; nc > 0 && ks < jend && e == cudaSuccess; ks += kLuW) {
+      const int pw = std::min(kLuW, jend - ks), rest = n - ks - pw, cols = jend - ks - pw;
+      const int per = std::max(kLuW, (int)cdivu(n - ks, nc));  // at most rpc
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(nc);
+      cfg.blockDim = dim3(512);
+      cfg.dynamicSmemBytes = (size_t)per * (kLuW + 1) * sizeof(T);
+      cfg.stream = c->stream;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = nc;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      count_launch(c, 2);
+      e = cudaLaunchKernelEx(&cfg, k_lu_panel_cluster<T>, D, ldd, n, ks, pw, per, piv, c->d_status);
+      if (e != cudaSuccess) break;
+      k_swap_cols<T><<<cdivu(n, 32), 256, 0, c->stream>>>(D, ldd, n, ks, pw, piv);
+      e = cudaGetLastError();
+      if (e == cudaSuccess && cols > 0) {  // the panel's second half
+        count_launch(c);
+        e = cudaFuncSetAttribute(k_trsm_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsm_smem<T>());
+        if (e != cudaSuccess) break;
+        k_trsm_panel<T><<<cdivu(cols, 32), 256, trsm_smem<T>(), c->stream>>>(D, ldd, jend, ks, pw);
+        e = cudaGetLastError();
+        if (e == cudaSuccess && rest > 0)
+          e = sc::gemm_update<T>(c, rest, cols, pw, D + (long long)(ks + pw) * ldd + ks, (int)ldd,
+                                 D + (long long)ks * ldd + ks + pw, (int)ldd, D + (long long)(ks + pw) * ldd + ks + pw,
+                                 (int)ldd);
+      }
+    }
+    for (int j = k0; nc == 0 && j < jend && e == cudaSuccess; ++j) {
       const int rows = n - j;
       const int pb = std::min<int>(kPivBlocks, (int)cdivu(rows, 256));
       count_launch(c, 4);
@@ -288,20 +509,23 @@ cudaError_t lu_factor(sc_ctx* c, T* D, long long ldd, int n, int* piv, bool tc) 
   return e;
 }
 
-// x = A^-1 b with the factors (row interchanges piv applied through perm); y: n scratch.
+// x = A^-1 b with the factors (row interchanges piv applied through perm); y: 2 n scratch.
 template <class T>
 cudaError_t lu_solve_dense(sc_ctx* c, const T* D, long long ldd, int n, const int* perm, const double* b, T* y,
                            double* x) {
   count_launch(c);
   k_permute_in<T><<<cdivu(n, 256), 256, 0, c->stream>>>(n, perm, b, y);
+  T* z = y + n;
+  auto ctas = [](int rows) { return std::max(1, std::min((rows + 7) / 8, 4 * 152)); };
   for (int b0 = 0; b0 < n; b0 += kPanel) {
+    const int bs = std::min(kPanel, n - b0);
     count_launch(c);
-    k_trsv_block<T, true><<<1, 1024, 0, c->stream>>>(D, ldd, n, b0, std::min(kPanel, n - b0), y);
+    k_trsv_block<T, true><<<ctas(n - b0 - bs), 256, 0, c->stream>>>(D, ldd, n, b0, bs, y, z);
   }
   const int last = ((n - 1) / kPanel) * kPanel;
   for (int b0 = last; b0 >= 0; b0 -= kPanel) {
     count_launch(c);
-    k_trsv_block<T, false><<<1, 1024, 0, c->stream>>>(D, ldd, n, b0, std::min(kPanel, n - b0), y);
+    k_trsv_block<T, false><<<ctas(b0), 256, 0, c->stream>>>(D, ldd, n, b0, std::min(kPanel, n - b0), z, y);
   }
   count_launch(c);
   k_to_double<T><<<cdivu(n, 256), 256, 0, c->stream>>>(n, y, x);
@@ -350,22 +574,25 @@ sc_status direct_factor_t(sc_ctx* c, int which, double* ms_form, double* ms_fact
     DC_CUDA(cudaGetLastError());
   } else {
     // S e_j through the condensed operator, the system the condensation forms
-    double* xb = c->Xfull;  // K ne >= n doubles of scratch
-    double* col = c->Rfull;
-    DC_CUDA(cudaMemsetAsync(xb, 0, (size_t)n * sizeof(double), c->stream));
-    for (int j = 0; j < n; ++j) {
-      count_launch(c);
-      k_unit_vec<<<1, 32, 0, c->stream>>>(xb, j, j - 1);
-      if (c->cfg.precision == SC_PREC_MIXED) {
-        DC_CUDA(sc::vec_to_float(c, c->Xbf, xb, (size_t)n));
-        DC_CUDA(sc::cond_interior32(c, c->Xbf, 1.0, nullptr, 0.0, c->Uf));
-        DC_CUDA(sc::cond_boundary32(c, c->Xbf, 1.0, nullptr, 0.0, c->Uf, col));
-      } else {
-        DC_CUDA(sc::cond_interior(c, xb, 1.0, nullptr, 0.0, c->Ui));
-        DC_CUDA(sc::cond_boundary(c, xb, 1.0, nullptr, 0.0, c->Ui, col));
-      }
-      count_launch(c);
-      k_put_column<T><<<cdivu(n, 256), 256, 0, c->stream>>>(col, n, j, D, ldd);
+    const size_t m = (size_t)std::min(kColumns, n), kt = m * G.K;
+    T *xb = nullptr, *tu = nullptr;
+    double* col = nullptr;
+    struct Tmp { void* p[3]; ~Tmp() { for (void* q : p) cudaFree(q); } } tmp{};
+    DC_CUDA(cudaMalloc(&xb, m * n * sizeof(T)));
+    tmp.p[0] = xb;
+    DC_CUDA(cudaMalloc(&tu, std::max<size_t>(1, kt * (G.ldi + G.ni)) * sizeof(T)));
+    tmp.p[1] = tu;
+    DC_CUDA(cudaMalloc(&col, m * n * sizeof(double)));
+    tmp.p[2] = col;
+    const T *Apk, *Ainv;
+    if constexpr (std::is_same<T, float>::value) { Apk = c->Apk32; Ainv = c->Ainv32; }
+    else { Apk = c->Apk; Ainv = c->Ainv; }
+    for (int j = 0; j < n; j += (int)m) {
+      const int mj = std::min((int)m, n - j);
+      count_launch(c, 2);
+      k_unit_vecs<T><<<cdivu((long long)n * mj, 256), 256, 0, c->stream>>>(xb, n, j, mj);
+      DC_CUDA(sc::cond_columns_pk<T>(c, Apk, Ainv, xb, tu, tu + kt * G.ldi, col, mj));
+      k_put_columns<T><<<cdivu(n, 32), 256, 0, c->stream>>>(col, n, j, mj, D, ldd);
     }
     DC_CUDA(cudaGetLastError());
   }
@@ -403,7 +630,7 @@ sc_status direct_apply_t(sc_ctx* c, const double* r, double* d, float* ms_lu, fl
   const T* D = static_cast<const T*>(c->Dlu);
   const bool mixed = c->cfg.precision == SC_PREC_MIXED;
   T* y = nullptr;
-  DC_CUDA(cudaMalloc(&y, (size_t)n * sizeof(T)));
+  DC_CUDA(cudaMalloc(&y, 2 * (size_t)n * sizeof(T)));
   struct Free { void* p; ~Free() { cudaFree(p); } } fy{y};
   cudaEvent_t ev[4];
   for (auto& x : ev) DC_CUDA(cudaEventCreate(&x));

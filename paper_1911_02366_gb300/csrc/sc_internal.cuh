@@ -572,6 +572,8 @@ cudaError_t cond_interior_pk(sc_ctx* c, const T* Apk, const T* Ainv, const T* xb
 cudaError_t cond_interior_sweep(sc_ctx* c, const double* xb, double* u);
 cudaError_t cond_interior_sweep32(sc_ctx* c, const float* xb, float* u);
 template <class T>
+cudaError_t cond_columns_pk(sc_ctx* c, const T* Apk, const T* Ainv, const T* xb, T* t, T* u, double* y, int m);
+template <class T>
 cudaError_t cond_boundary_pk(sc_ctx* c, const T* Apk, const T* xb, double delta, const double* Bfull, double gamma_,
                              const T* u, double* y);
 cudaError_t vec_axpby(sc_ctx* c, double* y, double a, const double* x, double b, size_t n);

@@ -287,14 +287,17 @@ __global__ void __launch_bounds__(256, PkOcc<T>::v) k_cond_interior_pk(Geo G, co
 }
 
 // The two steps of the interior pass spread over gridDim.x CTAs per element, t through memory
-// (K x ldi).
+// (K x ldi).  gridDim.z vectors at once (the columns of a dense S): vector z is zx, zt, zu, zy
+// entries behind the first.
 template <class T>
 __global__ void __launch_bounds__(256, PkOcc<T>::v) k_interior_rows(Geo G, const T* __restrict__ Apk, long long pstride,
     const int* __restrict__ node_tab, const int* __restrict__ own_code, const int2* __restrict__ cross_code,
     const int* __restrict__ nbr, const int* __restrict__ iperm, const T* __restrict__ xb, double beta,
-    const double* __restrict__ Bfull, double alpha, T* __restrict__ t, int black_zero) {
+    const double* __restrict__ Bfull, double alpha, T* __restrict__ t, int black_zero, long long zx, long long zt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int e = blockIdx.y, nb = G.nb;
+  if (xb) xb += blockIdx.z * zx;
+  t += blockIdx.z * zt;
   T* v = reinterpret_cast<T*>(smem_raw);
   __shared__ int nbr_s[18];
   const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, nw = blockDim.x / 32;
@@ -308,8 +311,11 @@ __global__ void __launch_bounds__(256, PkOcc<T>::v) k_interior_rows(Geo G, const
 
 template <class T>
 __global__ void __launch_bounds__(256, PkOcc<T>::v) k_interior_apply(Geo G, const T* __restrict__ Ainv,
-                                                                     const T* __restrict__ t, T* __restrict__ u) {
+                                                                     const T* __restrict__ t, T* __restrict__ u,
+                                                                     long long zt, long long zu) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  t += blockIdx.z * zt;
+  u += blockIdx.z * zu;
   T* ts = reinterpret_cast<T*>(smem_raw);
   const int e = blockIdx.y, lane = threadIdx.x % 32, warp = threadIdx.x / 32, nw = blockDim.x / 32;
   for (int i = threadIdx.x; i < G.ldi; i += blockDim.x) ts[i] = i < G.ni ? t[(size_t)e * G.ldi + i] : T(0);
@@ -328,8 +334,11 @@ __global__ void __launch_bounds__(256, PkOcc<T>::v) k_cond_boundary_pk(Geo G, co
     long long pstride, const int* __restrict__ node_tab, const int* __restrict__ own_code,
     const int2* __restrict__ cross_code, const int* __restrict__ nbr, const int* __restrict__ iperm,
     const T* __restrict__ xb, double delta, const double* __restrict__ Bfull, double gamma_, const T* __restrict__ u,
-    double* __restrict__ y, const int* __restrict__ elist, int own_zero) {
+    double* __restrict__ y, const int* __restrict__ elist, int own_zero, long long zx, long long zu, long long zy) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (xb) xb += blockIdx.z * zx;
+  if (u) u += blockIdx.z * zu;
+  y += blockIdx.z * zy;
   // CTA row i serves element elist[i] (one colour of the red-black sweep), or element i
   const int e = elist ? __ldg(elist + blockIdx.y) : blockIdx.y, ni = G.ni, nb = G.nb, lda = G.lda, cb0 = G.cb0;
   T* v = reinterpret_cast<T*>(smem_raw);  // lda + 4: [-u_e | 0 | delta x_e | 0]
@@ -478,8 +487,8 @@ cudaError_t cond_interior_pk(sc_ctx* c, const T* Apk, const T* Ainv, const T* xb
   count_launch(c);  // the profiled span counts one
   k_interior_rows<T><<<dim3(s1, G.K), 256, (size_t)(G.lda + 4) * sizeof(T), c->stream>>>(
       G, Apk, c->pk_stride, c->d_pk_node, c->d_pk_own_code, cc, c->d_nbr, c->d_iperm, xb, beta, Bfull, alpha, t,
-      black_zero);
-  k_interior_apply<T><<<dim3(s2, G.K), 256, (size_t)G.ldi * sizeof(T), c->stream>>>(G, Ainv, t, u);
+      black_zero, 0, 0);
+  k_interior_apply<T><<<dim3(s2, G.K), 256, (size_t)G.ldi * sizeof(T), c->stream>>>(G, Ainv, t, u, 0, 0);
   return cudaGetLastError();
 }
 
@@ -489,7 +498,7 @@ static cudaError_t boundary_launch(sc_ctx* c, const T* Apk, const T* xb, double 
   const Geo& G = c->G;
   k_cond_boundary_pk<T><<<dim3(pk_splits(count, G.nbn), count), 256, (size_t)(G.lda + 4) * sizeof(T), c->stream>>>(
       G, Apk, c->pk_stride, c->d_pk_node, c->d_pk_own_code, reinterpret_cast<const int2*>(c->d_pk_cross_code), c->d_nbr,
-      c->d_iperm, xb, delta, Bfull, gamma_, u, y, elist, own_zero);
+      c->d_iperm, xb, delta, Bfull, gamma_, u, y, elist, own_zero, 0, 0, 0);
   return cudaGetLastError();
 }
 
@@ -498,6 +507,32 @@ cudaError_t cond_boundary_pk(sc_ctx* c, const T* Apk, const T* xb, double delta,
                              const T* u, double* y) {
   return boundary_launch<T>(c, Apk, xb, delta, Bfull, gamma_, c->G.ni ? u : nullptr, y, nullptr, c->G.K, 0);
 }
+
+// y_z = S x_z for m vectors at once (each K nb long, one behind the other; t: m K ldi, u: m K ni values
+// of scratch): a single vector's passes leave the chip mostly idle on the small meshes whose S is
+// formed densely (27 elements of order 3: 26 us and five launches per column, one vector at a time).
+template <class T>
+cudaError_t cond_columns_pk(sc_ctx* c, const T* Apk, const T* Ainv, const T* xb, T* t, T* u, double* y, int m) {
+  const Geo& G = c->G;
+  const int2* cc = reinterpret_cast<const int2*>(c->d_pk_cross_code);
+  const long long zx = (long long)G.K * G.nb, zt = (long long)G.K * G.ldi, zu = (long long)G.K * G.ni;
+  const int work = m * G.K;
+  if (G.ni > 0) {
+    count_launch(c, 2);
+    k_interior_rows<T><<<dim3(pk_splits(work, G.nin), G.K, m), 256, (size_t)(G.lda + 4) * sizeof(T), c->stream>>>(
+        G, Apk, c->pk_stride, c->d_pk_node, c->d_pk_own_code, cc, c->d_nbr, c->d_iperm, xb, 1.0, nullptr, 0.0, t, 0, zx, zt);
+    k_interior_apply<T><<<dim3(pk_splits(work, (G.ni + 3) / 4), G.K, m), 256, (size_t)G.ldi * sizeof(T), c->stream>>>(
+        G, Ainv, t, u, zt, zu);
+  }
+  count_launch(c);
+  k_cond_boundary_pk<T><<<dim3(pk_splits(work, G.nbn), G.K, m), 256, (size_t)(G.lda + 4) * sizeof(T), c->stream>>>(
+      G, Apk, c->pk_stride, c->d_pk_node, c->d_pk_own_code, cc, c->d_nbr, c->d_iperm, xb, 1.0, nullptr, 0.0,
+      G.ni ? u : nullptr, y, nullptr, 0, zx, zu, zx);
+  return cudaGetLastError();
+}
+template cudaError_t cond_columns_pk<float>(sc_ctx*, const float*, const float*, const float*, float*, float*, double*, int);
+template cudaError_t cond_columns_pk<double>(sc_ctx*, const double*, const double*, const double*, double*, double*,
+                                             double*, int);
 
 // y_e = (A_bb x_b)_e - (A_bi u)_e for the elements of a list only (rows of one colour), whose
 // own boundary values in x_b are zero (the black elements in the red-black sweep): their packed
