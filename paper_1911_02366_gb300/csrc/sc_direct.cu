@@ -169,9 +169,20 @@ __global__ void k_panel_col(T* __restrict__ D, long long ldd, int n, int j, int 
 // to all CTAs (and the first CTA row j, which gives way), so that one cluster barrier per column
 // suffices: afterwards all know the pivot row, the two owners exchange the rows, and every thread
 // updates its rows and looks for the next column's candidate on the way.  The interchanges of the
-// other columns follow in k_swap_cols.  Bound by the 16 SMs' FP64 rate and the barriers: about 0.1 ms for
-// 7560 rows in FP64 against 32 columns x 4 launches, 25 us each (the same operations, one kernel each).
-constexpr int kLuW = 32;
+// other columns follow in k_swap_cols.  Bound by the 16 SMs' FP64 rate and the barriers: 0.13 ms on average
+// over the panels of 7560 rows in FP64 (0.44 ms with FP64 comparisons in the searches), against 32
+// columns x 4 launches, 21 us together, 0.7 ms.
+// |a| as an integer of the same order, 0 for zero and NaN: the searches run beside the FP64 pipe, which
+// a search with FP64 comparisons kept busy three times as long as the eliminations.
+__device__ __forceinline__ unsigned long long pivot_key(double a) {
+  const unsigned long long k = (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
+  return k > 0x7ff0000000000000ull ? 0ull : k;
+}
+__device__ __forceinline__ unsigned long long pivot_key(float a) {
+  const unsigned k = __float_as_uint(a) & 0x7fffffffu;
+  return k > 0x7f800000u ? 0u : k;
+}
+constexpr int kLuW = 32, kNoRow = 1 << 30;
 template <class T>
 __global__ void __launch_bounds__(512) k_lu_panel_cluster(T* __restrict__ D, long long ldd, int n, int k0, int pw,
                                                           int rpc, int* __restrict__ piv, int* __restrict__ status) {
@@ -181,10 +192,8 @@ __global__ void __launch_bounds__(512) k_lu_panel_cluster(T* __restrict__ D, lon
   constexpr int LD = kLuW + 1;
   T* a = reinterpret_cast<T*>(smem_raw);  // [rpc][LD]
   __shared__ T pub[2][17][kLuW];          // candidates' rows by rank; 16: row j
-  __shared__ double cval[2][16];
-  __shared__ int crow[2][16];
-  __shared__ double wval[16];
-  __shared__ int wrow[16];
+  __shared__ unsigned long long cval[2][16], wval[16];
+  __shared__ int crow[2][16], wrow[16];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = (int)cl.block_rank(), ncta = (int)cl.num_blocks();
   const int first = rank * rpc, mine = max(0, min(rpc, n - k0 - first));
@@ -193,27 +202,30 @@ __global__ void __launch_bounds__(512) k_lu_panel_cluster(T* __restrict__ D, lon
     a[r * LD + c] = c < pw ? D[(long long)(k0 + first + r) * ldd + k0 + c] : T(0);
   }
   __syncthreads();
-  double best = -1.0;
-  int brow = 1 << 30;
+  unsigned long long best = 0;
+  int brow = kNoRow;
   for (int r = tid; r < mine; r += 512) {
-    const double v = fabs((double)a[r * LD]);
+    const unsigned long long v = pivot_key(a[r * LD]);
     if (v > best) { best = v; brow = first + r; }
   }
   for (int j = 0; j < pw; ++j) {
     const int par = j & 1;
     for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const unsigned long long ov = __shfl_xor_sync(0xffffffffu, best, o);
       const int orow = __shfl_xor_sync(0xffffffffu, brow, o);
       if (ov > best || (ov == best && orow < brow)) { best = ov; brow = orow; }
     }
     if (lane == 0) { wval[warp] = best; wrow[warp] = brow; }
     __syncthreads();
-    best = wval[0];
-    brow = wrow[0];
-    for (int w = 1; w < 16; ++w)
-      if (wval[w] > best || (wval[w] == best && wrow[w] < brow)) { best = wval[w]; brow = wrow[w]; }
+    best = wval[lane & 15];
+    brow = wrow[lane & 15];
+    for (int o = 8; o > 0; o >>= 1) {
+      const unsigned long long ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int orow = __shfl_xor_sync(0xffffffffu, brow, o);
+      if (ov > best || (ov == best && orow < brow)) { best = ov; brow = orow; }
+    }
     if (warp < ncta) {  // warp w writes to CTA w
-      if (best >= 0.0) *cl.map_shared_rank(&pub[par][rank][lane], warp) = a[(brow - first) * LD + lane];
+      if (brow != kNoRow) *cl.map_shared_rank(&pub[par][rank][lane], warp) = a[(brow - first) * LD + lane];
       if (lane == 0) {
         *cl.map_shared_rank(&cval[par][rank], warp) = best;
         *cl.map_shared_rank(&crow[par][rank], warp) = brow;
@@ -221,11 +233,17 @@ __global__ void __launch_bounds__(512) k_lu_panel_cluster(T* __restrict__ D, lon
       if (rank == 0) *cl.map_shared_rank(&pub[par][16][lane], warp) = a[j * LD + lane];
     }
     cl.sync();
-    double pv = -1.0;
-    int p = 1 << 30, q = 0;
-    for (int i = 0; i < ncta; ++i)
-      if (cval[par][i] > pv || (cval[par][i] == pv && crow[par][i] < p)) { pv = cval[par][i]; p = crow[par][i]; q = i; }
-    const bool none = !(pv > 0.0);  // zero (or NaN) column: record the first such column, keep the row
+    unsigned long long pv = lane < ncta ? cval[par][lane] : 0ull;
+    int p = lane < ncta ? crow[par][lane] : kNoRow;
+    for (int o = 8; o > 0; o >>= 1) {
+      const unsigned long long ov = __shfl_xor_sync(0xffffffffu, pv, o);
+      const int orow = __shfl_xor_sync(0xffffffffu, p, o);
+      if (ov > pv || (ov == pv && orow < p)) { pv = ov; p = orow; }
+    }
+    pv = __shfl_sync(0xffffffffu, pv, 0);  // lanes 0 .. 15 hold the winner
+    p = __shfl_sync(0xffffffffu, p, 0);
+    const int q = p / rpc;
+    const bool none = pv == 0;  // zero (or NaN) column: record the first such column, keep the row
     if (none) p = j;
     if (rank == 0 && tid == 0) {
       piv[k0 + j] = k0 + p;
@@ -238,19 +256,25 @@ __global__ void __launch_bounds__(512) k_lu_panel_cluster(T* __restrict__ D, lon
     }
     __syncthreads();
     const T pivot = prow[j], inv = pivot == T(0) ? T(0) : T(1) / pivot;
-    best = -1.0;
-    brow = 1 << 30;
+    best = 0;
+    brow = kNoRow;
     for (int r = tid; r < mine; r += 512) {
       if (first + r <= j) continue;
       T* row = a + r * LD;
       if (pivot != T(0)) {
         const T l = row[j] * inv;
         row[j] = l;
-#pragma unroll 8
-        for (int c = j + 1; c < kLuW; ++c) row[c] -= l * prow[c];
+        for (int c0 = (j + 1) & ~7; c0 < kLuW; c0 += 8) {
+          T v[8], u[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) { v[i] = row[c0 + i]; u[i] = prow[c0 + i]; }
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (c0 + i > j) row[c0 + i] = v[i] - l * u[i];
+        }
       }
       if (j + 1 < pw) {
-        const double v = fabs((double)row[j + 1]);
+        const unsigned long long v = pivot_key(row[j + 1]);
         if (v > best) { best = v; brow = first + r; }
       }
     }
