@@ -302,28 +302,35 @@ __global__ void __launch_bounds__(64) k_mx_face(MxMesh M, Geo Gp, const double* 
 }
 
 // Lifted gradient g_a(m) = (2/h) [ sum_b D[m_a][b] q_b + s (qhat - q_m) / w_{m_a} on a face ]
-// (the weak form of eq. DGSEMsystem:2 after summation by parts on Gauss-Lobatto nodes).
+// (the weak form of eq. DGSEMsystem:2 after summation by parts on Gauss-Lobatto nodes).  One CTA per
+// element, one thread per node (up to order 6), the element's values in shared memory.  Latency bound:
+// 216 elements of orders 2 .. 6 take 21 us (56 us with 128 threads and global loads per term).
+constexpr int kMxNodeThreads = 352;
 template <class T>
-__global__ void __launch_bounds__(128) k_mx_lift(MxMesh M, const double* __restrict__ Q,
+__global__ void __launch_bounds__(kMxNodeThreads) k_mx_lift(MxMesh M, const double* __restrict__ Q,
                                                  const double* __restrict__ dir, const T* __restrict__ qhat,
                                                  T* __restrict__ grad) {
   const int e = blockIdx.x, N = M.ord[e], p = N + 1, nn = p * p * p;
   const size_t o = M.off[e];
   const double* D = &M.tab->D[N][0][0];
   const double* w = M.tab->w[N];
+  __shared__ __align__(16) unsigned char raw[343 * 5 * sizeof(T)];  // no constructors in shared memory
+  T* qs = reinterpret_cast<T*>(raw);
+  for (int i = threadIdx.x; i < nn * 5; i += blockDim.x) qs[i] = Val<T>::make(Q[o * 5 + i], dir ? dir[o * 5 + i] : 0.0);
+  __syncthreads();
   for (int m = threadIdx.x; m < nn; m += blockDim.x) {
     const int c[3] = {m % p, (m / p) % p, m / (p * p)};
     T qm[5];
-    for (int k = 0; k < 5; ++k) qm[k] = Val<T>::make(Q[(o + m) * 5 + k], dir ? dir[(o + m) * 5 + k] : 0.0);
+    for (int k = 0; k < 5; ++k) qm[k] = qs[m * 5 + k];
     for (int a = 0; a < 3; ++a) {
       T acc[5];
       for (int k = 0; k < 5; ++k) acc[k] = T(0.0);
       int cc[3] = {c[0], c[1], c[2]};
       for (int b = 0; b < p; ++b) {
         cc[a] = b;
-        const size_t nd = o + mx_node(cc, p);
+        const int nd = mx_node(cc, p);
         const double Dab = D[c[a] * 8 + b];
-        for (int k = 0; k < 5; ++k) acc[k] = acc[k] + Dab * Val<T>::make(Q[nd * 5 + k], dir ? dir[nd * 5 + k] : 0.0);
+        for (int k = 0; k < 5; ++k) acc[k] = acc[k] + Dab * qs[nd * 5 + k];
       }
       if (c[a] == 0 || c[a] == N) {
         const int s = c[a] == N ? 1 : -1, f = 2 * a + (s > 0);
@@ -362,8 +369,9 @@ __global__ void __launch_bounds__(128) k_mx_flux(MxMesh M, Geo Gp, const double*
 //   R_j = c0 J W_j (q_j - qh_j) / dt + Jf W_j sum_d sum_b D[j_d][b] F_d(b)
 //         + sum_{faces of j} Jf W_j / w_{j_d} (fhat_j - s F_d(j)).
 // out: the value (T = double) or the derivative part (dual T).
+// One thread per node of the CTA's element, as in k_mx_lift.
 template <class T>
-__global__ void __launch_bounds__(128) k_mx_resid(MxMesh M, const double* __restrict__ Q,
+__global__ void __launch_bounds__(kMxNodeThreads) k_mx_resid(MxMesh M, const double* __restrict__ Q,
                                                   const double* __restrict__ dir, const double* __restrict__ Qh,
                                                   const T* __restrict__ F, const T* __restrict__ fhat,
                                                   double* __restrict__ out) {
@@ -410,7 +418,7 @@ __global__ void __launch_bounds__(128) k_mx_resid(MxMesh M, const double* __rest
 // range needs; the CTAs take the items from a counter, longest elements first, with one scratch
 // slot per CTA.  Latency bound (per seed a chain of dependent small phases on 128 threads):
 // with one CTA per element the 343 seeds of order 6 ran one after the other, 74 ms on a mesh of
-// 6^3 elements of orders 2 .. 6, now 32 ms.
+// 6^3 elements of orders 2 .. 6, now 28 ms.
 // Per-element scratch (in T5 units): the qhat of the six faces unseeded (QH0) and seeded
 // (QH), the neighbour's qhat on each shared face (QHN, <= 49 nodes), the lifted gradient
 // (GE) and point fluxes (FE) of the element, the neighbour's gradients on each shared face
@@ -427,33 +435,43 @@ struct OwnScratch {
   }
 };
 
-// Point function of the unseeded pass: the face-flux Jacobians at every point (seven passes of
-// five directions: the own 20 inputs, then the neighbour's 15 gradient inputs); no output.
+// Point function of the unseeded pass: the values of both sides' inputs at every point, for
+// face_jacobian; no output.
+constexpr int kFaceVals = 40;
 template <class R>
-struct PfJac {
-  Geo Gp; R* J;  // J[point][175] of one face
+struct PfVals {
+  R* V;  // V[point][40] of one face
   template <class T>
-  __device__ void operator()(int t, const T* a, const T* b, int d, int s, T* out) const {
-    R* Jt = J + t * kFaceJac;
-    for (int pass = 0; pass < 7; ++pass) {
-      T qa[20], qb[20], o[5];
-      for (int c = 0; c < 20; ++c) { qa[c] = T((double)a[c].v); qb[c] = T((double)b[c].v); }
-      for (int i = 0; i < 5; ++i) {
-        const int dir = pass * 5 + i;
-        if (dir < 20) qa[dir].d[i] = R(1);
-        else qb[5 + dir - 20].d[i] = R(1);
-      }
-      PfFhat{Gp}(t, qa, qb, d, s, o);
-      for (int k = 0; k < 5; ++k)
-        for (int i = 0; i < 5; ++i) {
-          const int dir = pass * 5 + i;
-          if (dir < 20) Jt[k * 20 + dir] = o[k].d[i];
-          else Jt[100 + k * 15 + dir - 20] = o[k].d[i];
-        }
-    }
+  __device__ void operator()(int t, const T* a, const T* b, int, int, T* out) const {
+    for (int c = 0; c < 20; ++c) { V[t * kFaceVals + c] = a[c].v; V[t * kFaceVals + 20 + c] = b[c].v; }
     for (int k = 0; k < 5; ++k) out[k] = T(0.0);
   }
 };
+
+// Face-flux Jacobians at the npt points of a face, J[point][175]: seven passes of five directions
+// (the own 20 inputs, then the neighbour's 15 gradient inputs), spread over the CTA's threads.
+template <class R>
+__device__ void face_jacobian(const Geo& Gp, int npt, int d, int s, const R* V, R* J) {
+  using T = DualN<R, 5>;
+  for (int u = threadIdx.x; u < 7 * npt; u += blockDim.x) {
+    const int pass = u / npt, t = u % npt;
+    R* Jt = J + t * kFaceJac;
+    T qa[20], qb[20], o[5];
+    for (int c = 0; c < 20; ++c) { qa[c] = T((double)V[t * kFaceVals + c]); qb[c] = T((double)V[t * kFaceVals + 20 + c]); }
+    for (int i = 0; i < 5; ++i) {
+      const int dir = pass * 5 + i;
+      if (dir < 20) qa[dir].d[i] = R(1);
+      else qb[5 + dir - 20].d[i] = R(1);
+    }
+    PfFhat{Gp}(t, qa, qb, d, s, o);
+    for (int k = 0; k < 5; ++k)
+      for (int i = 0; i < 5; ++i) {
+        const int dir = pass * 5 + i;
+        if (dir < 20) Jt[k * 20 + dir] = o[k].d[i];
+        else Jt[100 + k * 15 + dir - 20] = o[k].d[i];
+      }
+  }
+}
 
 // Point function of a seed: the dual parts of fhat from those of the inputs through the
 // Jacobians of the unseeded pass (values are not needed: the rows take dual parts only).
@@ -692,8 +710,15 @@ __global__ void __launch_bounds__(128) k_mx_own(MxMesh M, Geo Gp, const double* 
         }
         return S[L.gn + (f * 49 + x) * 15 + (k - 5)];
       };
-      if (r < 0) face_eval<T5, 20>(M, e, f, ld, PfJac<R>{Gp, Jf + f * 49 * kFaceJac}, sbuf, stmp, S + L.fh + f * pp * 5);
-      else face_eval<T5, 20>(M, e, f, ld, PfLin<R>{Jf + f * 49 * kFaceJac}, sbuf, stmp, S + L.fh + f * pp * 5);
+      if (r < 0) {
+        R* V = reinterpret_cast<R*>(S + L.qh);  // qh and qhn belong to the seeds
+        face_eval<T5, 20>(M, e, f, ld, PfVals<R>{V}, sbuf, stmp, S + L.fh + f * pp * 5);
+        const int Mo = max(N, M.ord[nb]);
+        face_jacobian<R>(Gp, N != M.ord[nb] || M.force_mortar ? (Mo + 1) * (Mo + 1) : pp, d, s, V, Jf + f * 49 * kFaceJac);
+        __syncthreads();  // V serves the next face
+        continue;
+      }
+      face_eval<T5, 20>(M, e, f, ld, PfLin<R>{Jf + f * 49 * kFaceJac}, sbuf, stmp, S + L.fh + f * pp * 5);
     }
     if (r < 0) continue;  // unseeded gradients, fluxes and face Jacobians are in place
     // rows of e: the column block of the seed.  Only moved nodes carry a flux derivative, so
@@ -1008,10 +1033,10 @@ cudaError_t mx_eval(sc_mixed* m, const double* dir, double* out) {
   T* F = std::is_same<T, double>::value ? reinterpret_cast<T*>(m->F0) : reinterpret_cast<T*>(m->FJ);
   const cudaStream_t st = m->stream;
   k_mx_face<T, false><<<M.K * 6, 64, 0, st>>>(M, m->Gp, m->Q, dir, nullptr, qh);
-  k_mx_lift<T><<<M.K, 128, 0, st>>>(M, m->Q, dir, qh, g);
+  k_mx_lift<T><<<M.K, kMxNodeThreads, 0, st>>>(M, m->Q, dir, qh, g);
   k_mx_face<T, true><<<M.K * 6, 64, 0, st>>>(M, m->Gp, m->Q, dir, g, fh);
   k_mx_flux<T><<<mx_blocks(m->nodes, 128), 128, 0, st>>>(M, m->Gp, m->Q, dir, g, F, (int)m->nodes);
-  k_mx_resid<T><<<M.K, 128, 0, st>>>(M, m->Q, dir, m->Qh, F, fh, out);
+  k_mx_resid<T><<<M.K, kMxNodeThreads, 0, st>>>(M, m->Q, dir, m->Qh, F, fh, out);
   m->launches += 5;
   return cudaGetLastError();
 }
