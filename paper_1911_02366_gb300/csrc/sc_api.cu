@@ -93,7 +93,7 @@ void free_all(sc_ctx* c) {
   double** dps[] = {&c->Q, &c->Qh, &c->grad, &c->F, &c->B, &c->NJ, &c->RJ, &c->Aown, &c->X, &c->Ainv,
                     &c->Ytmp, &c->See, &c->V, &c->Wv, &c->Zv, &c->Xb, &c->Gb, &c->Rb, &c->Ui, &c->Tb,
                     &c->Hd, &c->partial, &c->Xfull, &c->Rfull, &c->Apk, &c->Sls, &c->dQn,
-                    &c->OV, &c->OZ, &c->gloc, &c->NJL, &c->Floc};
+                    &c->OV, &c->OZ, &c->gloc, &c->NJL, &c->Floc, &c->diss};
   for (auto p : dps) { if (*p) cudaFree(*p); *p = nullptr; }
   float** fps[] = {&c->Aown32, &c->Ainv32, &c->Y32, &c->See32, &c->Zf, &c->Xbf, &c->Uf,
                    &c->Apk32, &c->Sls32, &c->Sdiag, &c->Cpl, &c->Feat, &c->Snorm, &c->Ynet,
@@ -346,6 +346,7 @@ sc_status sc_set_mesh(sc_ctx* c, int n, double L, int N) {
   A(dalloc(&c->Xfull, dofs)); A(dalloc(&c->Rfull, dofs)); A(dalloc(&c->dQn, dofs));
   A(dalloc(&c->grad, nodes * 15)); A(dalloc(&c->F, nodes * 15));
   A(dalloc(&c->NJ, nodes * 375)); A(dalloc(&c->RJ, (size_t)G.K * 6 * 50 * G.p * G.p));
+  A(dalloc(&c->diss, (size_t)G.K * 3 * G.p * G.p * 5));
   if (G.visc_flux == SC_VISC_SIPG) { A(dalloc(&c->gloc, nodes * 15)); A(dalloc(&c->Floc, nodes * 15)); A(dalloc(&c->NJL, nodes * 375)); }
   A(dalloc(&c->Aown, (size_t)G.K * own_stride(G))); A(dalloc(&c->X, (size_t)G.K * G.NP * 25));
   if (c->cfg.precision == SC_PREC_MIXED) {

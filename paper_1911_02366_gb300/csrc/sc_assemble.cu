@@ -46,15 +46,17 @@ __global__ void k_history(Geo G, const double* __restrict__ Qs, const double* __
 // ---- residual ---------------------------------------------------------------------------
 // Two kernels, one thread per node, CTAs of whole elements (four of order 2, two of order 3, else
 // one) whose values sit in shared memory:
-//   k_point  lifted gradients and point fluxes F_d = f^a_d - f^nu_d
+//   k_point  lifted gradients and point fluxes F_d = f^a_d - f^nu_d, and the dissipation of the
+//            numerical flux on the element's three faces in positive direction
 //   k_rows   rows of the residual: divergence lines, face terms, and what becomes of them
 // Face terms: with the central part of the numerical flux s (f^a(+) + f^a(-)) / 2 and the viscous
 // average s (f^nu(+) + f^nu(-)) / 2, fhat = s (F(+) + F(-)) / 2 - diss / 2 with the point fluxes
-// that are there already, so a face node costs one dissipation and no viscous flux.  Face
-// nodes are their own work items (6 (N+1)^2 per element, equal work), summed by their nodes
-// afterwards.  FP64-pipe bound: 46 + 54 us per Runge-Kutta stage at 8^3, N = 4 (the stage's update
-// included) against 22 + 22 + 215 + 16 us in five kernels with one thread per node doing its up to
-// three faces (Roe and two viscous fluxes each, 16 % of the warps resident).
+// that are there already, and diss changes its sign with the side: a pair of face nodes costs one
+// dissipation and no viscous flux.  Face nodes are their own work items, summed by their nodes
+// afterwards.  FP64-pipe bound: 61 + 30 us per Runge-Kutta stage at 8^3, N = 4 (the
+// stage's update included; 46 + 54 us with a dissipation per side, evaluated in k_rows) against 22 + 22 +
+// 215 + 16 us in five kernels with one thread per node doing its up to three faces (Roe and two
+// viscous fluxes each, 16 % of the warps resident).
 inline int group_elems(const Geo& G) { return G.nn <= 32 ? 4 : G.nn <= 64 ? 2 : 1; }
 inline int group_threads(const Geo& G) { return (group_elems(G) * G.nn + 31) / 32 * 32; }
 
@@ -96,13 +98,22 @@ __device__ __forceinline__ void store_nodes(const double (&v)[n], double* buf, d
   for (int i = threadIdx.x; i < nodes * n; i += blockDim.x) out[first * n + i] = buf[i];
 }
 
+// Face node ia = a + p b of the faces normal to d: node m at the lower end, sd from one layer to the next.
+struct FaceNode {
+  int m, sd;
+  __device__ __forceinline__ FaceNode(int p, int d, int ia) {
+    sd = d == 0 ? 1 : d == 1 ? p : p * p;
+    m = ia % p * (d == 0 ? p : 1) + ia / p * (d == 2 ? p : p * p);
+  }
+};
+
 // spd (or null): the largest signal speed |v| + c and the largest diffusivity
 // max(4/3, gamma/Pr) mu / (rho Re) of all nodes, folded in as bit patterns.
 template <bool IP>
 __global__ void __launch_bounds__(352) k_point(Geo G, int ge, const double* __restrict__ Q, const int* __restrict__ nbr,
                                                double* __restrict__ F, double* __restrict__ grad,
                                                double* __restrict__ Floc, double* __restrict__ gloc,
-                                               unsigned long long* __restrict__ spd) {
+                                               double* __restrict__ diss, unsigned long long* __restrict__ spd) {
   extern __shared__ __align__(16) double sm[];
   const int p = G.p, N = G.N, nn = G.nn, e0 = blockIdx.x * ge, ne = min(ge, G.K - e0), nodes = ne * nn;
   double* Ds = sm;               // p x p
@@ -112,6 +123,19 @@ __global__ void __launch_bounds__(352) k_point(Geo G, int ge, const double* __re
   for (int i = threadIdx.x; i < p * p; i += blockDim.x) Ds[i] = G.D[i / p][i % p];
   for (int i = threadIdx.x; i < nodes * 5; i += blockDim.x) qs[i] = Q[first * 5 + i];
   __syncthreads();
+  for (int i = threadIdx.x; i < ne * 3 * p * p; i += blockDim.x) {  // diss[e][d][face node]
+    const int el = i / (3 * p * p), d = i / (p * p) % 3, ia = i % (p * p);
+    const FaceNode fn(p, d, ia);
+    const int m = fn.m + N * fn.sd;
+    const size_t tn = (size_t)__ldg(nbr + (e0 + el) * 18 + 2 * d + 1) * nn + fn.m;
+    const int kk[5] = {0, 1 + d, d == 0 ? 2 : 1, d == 2 ? 2 : 3, 4};  // normal momentum first
+    double ra[5], rb[5], o[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) { ra[k] = qs[(el * nn + m) * 5 + kk[k]]; rb[k] = __ldg(Q + tn * 5 + kk[k]); }
+    adv_dissipation_x(G, ra, rb, 1.0, o);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) diss[(((size_t)e0 * 3) * p * p + i) * 5 + kk[k]] = o[k];
+  }
   const bool live = threadIdx.x < nodes;
   const int t = live ? threadIdx.x : 0, el = t / nn, m = t - el * nn, e = e0 + el;
   const double* qe = qs + el * nn * 5;
@@ -171,7 +195,8 @@ __global__ void __launch_bounds__(352) k_point(Geo G, int ge, const double* __re
 template <bool IP, bool RK>
 __global__ void __launch_bounds__(352) k_rows(Geo G, int ge, const double* __restrict__ Q, const double* __restrict__ Qh,
                                               const double* __restrict__ F, const double* __restrict__ Floc,
-                                              const int* __restrict__ nbr, double* __restrict__ out, sc::RkStage st) {
+                                              const double* __restrict__ diss, const int* __restrict__ nbr,
+                                              double* __restrict__ out, sc::RkStage st) {
   extern __shared__ __align__(16) double sm[];
   const int p = G.p, N = G.N, nn = G.nn, pp = p * p, e0 = blockIdx.x * ge, ne = min(ge, G.K - e0), nodes = ne * nn;
   double* Ds = sm;                   // p x p
@@ -185,35 +210,25 @@ __global__ void __launch_bounds__(352) k_rows(Geo G, int ge, const double* __res
   __syncthreads();
   for (int i = threadIdx.x; i < ne * 6 * pp; i += blockDim.x) {
     const int el = i / (6 * pp), f = i / pp % 6, ia = i % pp, d = f >> 1, s = (f & 1) ? 1 : -1;
-    const int a = ia % p, b = ia / p, end = s > 0 ? N : 0;
-    const int sd = d == 0 ? 1 : d == 1 ? p : pp, s1 = d == 0 ? p : 1, s2 = d == 2 ? p : pp;  // in-face strides
-    const int m = end * sd + a * s1 + b * s2;
-    const size_t tn = (size_t)__ldg(nbr + (e0 + el) * 18 + f) * nn + m + (N - 2 * end) * sd;
-    const int k1 = 1 + d, k2 = d == 0 ? 2 : 1, k3 = d == 2 ? 2 : 3;  // momenta, normal one first
-    const double* qa = qs + (el * nn + m) * 5;
-    const double* qb = Q + tn * 5;
-    const double ra[5] = {qa[0], qa[k1], qa[k2], qa[k3], qa[4]};
-    const double rb[5] = {__ldg(qb), __ldg(qb + k1), __ldg(qb + k2), __ldg(qb + k3), __ldg(qb + 4)};
+    const FaceNode fn(p, d, ia);
+    const int m = fn.m + (s > 0 ? N : 0) * fn.sd, nb = __ldg(nbr + (e0 + el) * 18 + f);
+    const size_t tn = (size_t)nb * nn + fn.m + (s > 0 ? 0 : N) * fn.sd;
     const double* Fa = Fs + (el * nn + m) * 15 + d * 5;
     const double* Fb = (IP ? Floc : F) + tn * 15 + d * 5;
-    double fb[5], diss[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) fb[k] = __ldg(Fb + k);
-    adv_dissipation_x(G, ra, rb, (double)s, diss);
+    const double* ds = diss + (((size_t)(s > 0 ? e0 + el : nb) * 3 + d) * pp + ia) * 5;
     double* o = fs + (size_t)i * 5;
-    const int kk[5] = {0, k1, k2, k3, 4};
+    double fb[5], dk[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) { fb[k] = __ldg(Fb + k); dk[k] = __ldg(ds + k); }
     if (IP) {
       const double* Fl = Floc + (first + el * nn + m) * 15 + d * 5;
+      const double* qa = qs + (el * nn + m) * 5;
 #pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        const int v = kk[k];
-        o[v] = 0.5 * s * (__ldg(Fl + v) + __ldg(Fb + v)) - 0.5 * diss[k] + G.sigma * (ra[k] - rb[k]) - s * Fa[v];
-      }
+      for (int k = 0; k < 5; ++k)
+        o[k] = 0.5 * s * (__ldg(Fl + k) + fb[k] - dk[k]) + G.sigma * (qa[k] - __ldg(Q + tn * 5 + k)) - s * Fa[k];
     } else {
 #pragma unroll
-      for (int k = 0; k < 5; ++k) o[k] = 0.5 * s * (fb[k] - Fa[k]);
-#pragma unroll
-      for (int k = 0; k < 5; ++k) o[kk[k]] -= 0.5 * diss[k];
+      for (int k = 0; k < 5; ++k) o[k] = 0.5 * s * (fb[k] - Fa[k] - dk[k]);
     }
   }
   __syncthreads();
@@ -649,7 +664,7 @@ static cudaError_t launch_point(sc_ctx* c, const Geo& G, const double* Q, bool s
   if (e != cudaSuccess) return e;
   count_launch(c);
   k_point<IP><<<(G.K + ge - 1) / ge, group_threads(G), point_smem(G), c->stream>>>(
-      G, ge, Q, c->d_nbr, c->F, store_grad ? c->grad : nullptr, c->Floc, c->gloc, spd);
+      G, ge, Q, c->d_nbr, c->F, store_grad ? c->grad : nullptr, c->Floc, c->gloc, c->diss, spd);
   return cudaGetLastError();
 }
 
@@ -659,7 +674,7 @@ static cudaError_t launch_rows(sc_ctx* c, const Geo& G, const double* Q, const d
   cudaError_t e = cudaFuncSetAttribute(k_rows<IP, RK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem(G));
   if (e != cudaSuccess) return e;
   count_launch(c);
-  k_rows<IP, RK><<<(G.K + ge - 1) / ge, group_threads(G), rows_smem(G), c->stream>>>(G, ge, Q, Qh, c->F, c->Floc, c->d_nbr,
+  k_rows<IP, RK><<<(G.K + ge - 1) / ge, group_threads(G), rows_smem(G), c->stream>>>(G, ge, Q, Qh, c->F, c->Floc, c->diss, c->d_nbr,
                                                                                      out, st);
   return cudaGetLastError();
 }

@@ -327,6 +327,7 @@ struct sc_ctx {
   // interior penalty only: the elements' own (unlifted) gradients and the point-flux
   // Jacobians at them, same layouts as grad and NJ
   double *gloc = nullptr, *NJL = nullptr, *Floc = nullptr;
+  double* diss = nullptr;  // [K][3][p^2][5] dissipation of the numerical flux on the positive faces
   int *d_nbr = nullptr, *d_perm = nullptr, *d_iperm = nullptr, *d_own_pairs = nullptr;
   double* gj_scale = nullptr;      // [K][n_i] row scaling of the blocked Gauss-Jordan (T-typed)
   double *OV = nullptr, *OZ = nullptr;  // outer FGMRES: Arnoldi basis (m+1 global vectors), preconditioned (m)
