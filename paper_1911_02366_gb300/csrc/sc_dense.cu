@@ -6,7 +6,7 @@
 //               per CTA held in shared memory.
 //   k_gemm      C = alpha A B + beta C for a batch of row-major blocks (SIMT, 64x64
 //               tiles, 4x4 register micro-tiles).
-//   k_lu        right-looking blocked LU with partial pivoting of a batch of blocks
+//   k_lu_panel  one 32-column panel of the right-looking LU with partial pivoting of a batch of blocks
 //               in global memory (32-column panels factorised in shared memory).
 //   k_solve_prep  partitioned inverses of the LU factors in the solve layout (below).
 //   k_lu_solve    z = (P^T L U)^-1 v for every element, one warp per element, one lane
@@ -390,52 +390,6 @@ __device__ void lu_panel(int n, int k0, T* __restrict__ Mx, int lda, int* __rest
     }
   }
   __syncthreads();
-}
-
-// Whole LU of one element block per CTA: panel steps with the trailing update
-// A22 -= L21 U12 done by the same CTA in 4 x 4 register tiles.
-template <class T>
-__global__ void __launch_bounds__(256) k_lu(int n, T* __restrict__ A, long long stride, int lda,
-                                            int* __restrict__ piv_all, int* __restrict__ status) {
-  extern __shared__ unsigned char smem_raw[];
-  T* P = reinterpret_cast<T*>(smem_raw);  // panel [n][PW+1]
-  constexpr int pld = PW + 1;
-  __shared__ int s_p;
-  __shared__ int s_bad;
-  const int e = blockIdx.x;
-  T* Mx = A + (long long)e * stride;
-  int* piv = piv_all + (long long)e * n;
-  if (threadIdx.x == 0) s_bad = 0;
-  __syncthreads();
-  for (int k0 = 0; k0 < n; k0 += PW) {
-    lu_panel<T>(n, k0, Mx, lda, piv, P, &s_p, &s_bad);
-    const int bw = min(PW, n - k0), rest = n - k0 - bw;
-    if (rest > 0) {
-      // A22 -= L21 U12, 4x4 register tiles
-      const int tr = (rest + 3) / 4, tcn = (rest + 3) / 4;
-      for (int t = threadIdx.x; t < tr * tcn; t += blockDim.x) {
-        const int bi = (t / tcn) * 4, bj = (t % tcn) * 4;
-        T acc[4][4];
-        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-        for (int c = 0; c < bw; ++c) {
-          T l[4], u[4];
-          for (int a = 0; a < 4; ++a) l[a] = (bi + a < rest) ? P[(bw + bi + a) * pld + c] : T(0);
-          for (int b = 0; b < 4; ++b)
-            u[b] = (bj + b < rest) ? Mx[(long long)(k0 + c) * lda + k0 + bw + bj + b] : T(0);
-          for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) acc[a][b] = fma(l[a], u[b], acc[a][b]);
-        }
-        for (int a = 0; a < 4; ++a) {
-          if (bi + a >= rest) continue;
-          for (int b = 0; b < 4; ++b) {
-            if (bj + b >= rest) continue;
-            Mx[(long long)(k0 + bw + bi + a) * lda + k0 + bw + bj + b] -= acc[a][b];
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && s_bad) atomicCAS(status, -1, e);
 }
 
 // One panel step for every element (the trailing update is a separate batched GEMM).
@@ -1362,6 +1316,30 @@ namespace sc {
 
 // Blocked LU of the S_ee blocks with the trailing updates A22 -= L21 U12 as batched TF32
 // tensor-core GEMMs (mixed arm): per panel one k_lu_panel launch and one GEMM.
+// LU with partial pivoting of `batch` n x n blocks on the CUDA cores: per 32 columns one panel step per
+// block, then the trailing updates of all blocks as one batched product.  FP64-pipe bound (FP32 without
+// tensor cores: FMA bound); the panels are latency bound.  With the updates in the panel's CTA 64
+// blocks of n_b = 280 kept 64 SMs at FP64 rate and the others idle (3.2 ms; now 1.6 ms of panels and
+// the products on all SMs).
+template <class T>
+static cudaError_t lu_blocked_simt(sc_ctx* c, int n, T* A, long long stride, int lda, int batch, int* piv, int* status) {
+  const size_t smem = (size_t)n * (PW + 1) * sizeof(T);
+  cudaError_t err = cudaFuncSetAttribute(k_lu_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err != cudaSuccess) return err;
+  for (int k0 = 0; k0 < n; k0 += PW) {
+    const int bw = min(PW, n - k0), rest = n - k0 - bw;
+    if (k0 > 0) count_launch(c);
+    k_lu_panel<T><<<batch, 256, smem, c->stream>>>(n, k0, A, stride, lda, piv, status);
+    if (rest <= 0) continue;
+    count_launch(c);
+    T* A21 = A + (size_t)(k0 + bw) * lda + k0;
+    T* A12 = A + (size_t)k0 * lda + k0 + bw;
+    k_gemm<T><<<dim3(cdiv(rest, 64), cdiv(rest, 64), batch), 256, 0, c->stream>>>(
+        rest, rest, bw, T(-1), A21, stride, lda, A12, stride, lda, T(1), A21 + bw, stride, lda);
+  }
+  return cudaGetLastError();
+}
+
 // Blocked LU with partial pivoting of `batch` n_b x n_b blocks (row stride lds, block stride
 // n_b lds): panels of PW columns, TF32 tensor-core trailing updates; pivots in piv, the first
 // singular block's index in *status.
@@ -1527,11 +1505,9 @@ cudaError_t condense_t(sc_ctx* c, T* Aown, T* Ainv, T* Y, T* See, bool tc, bool 
       }
     }
     if (!done) {
-      const size_t smem = (size_t)nb * (PW + 1) * sizeof(T);
-      err = cudaFuncSetAttribute(k_lu<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (err != cudaSuccess) return err;
       ProfScope ps(c, SCK_LU);
-      k_lu<T><<<K, 256, smem, c->stream>>>(nb, See, (long long)nb * lds, lds, c->piv, c->d_status);
+      err = lu_blocked_simt<T>(c, nb, See, (long long)nb * lds, lds, K, c->piv, c->d_status);
+      if (err != cudaSuccess) return err;
     }
     count_launch(c, 2);
     k_piv_to_perm<<<K, 128, 2 * nb * sizeof(int), c->stream>>>(nb, c->piv, c->rowperm);
@@ -1767,11 +1743,9 @@ cudaError_t factor_batch32(sc_ctx* c, float* A, int n, int lda, long long stride
     if (err != cudaSuccess) return err;
     count_launch(c, 3);
   } else {
-    const size_t smem = (size_t)n * (PW + 1) * sizeof(float);
-    err = cudaFuncSetAttribute(k_lu<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    err = lu_blocked_simt<float>(c, n, A, stride, lda, batch, piv, status);
     if (err != cudaSuccess) return err;
     count_launch(c, 4);
-    k_lu<float><<<batch, 256, smem, c->stream>>>(n, A, stride, lda, piv, status);
   }
   k_piv_to_perm<<<batch, 128, 2 * n * sizeof(int), c->stream>>>(n, piv, rowperm);
   const size_t dsm = (size_t)8 * 2 * 32 * 33 * sizeof(float);
