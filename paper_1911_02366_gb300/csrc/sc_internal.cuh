@@ -336,6 +336,8 @@ struct sc_ctx {
   int *piv = nullptr, *rowperm = nullptr, *d_status = nullptr;
   // Krylov workspace (boundary space of size n1 = K*nb)
   double *V = nullptr, *Wv = nullptr, *Zv = nullptr, *Xb = nullptr, *Gb = nullptr, *Rb = nullptr;
+  double* h_gs = nullptr;          // pinned host copy of one iteration's Gram-Schmidt results
+  cudaEvent_t ev_gs = nullptr;     // recorded behind that copy
   double *Ui = nullptr, *Tb = nullptr, *Hd = nullptr, *partial = nullptr, *Xfull = nullptr, *Rfull = nullptr;
   int restart_alloc = 0;
   // mixed-precision arm: FP32 copies of the element blocks and FP32 condensation
@@ -507,6 +509,11 @@ cudaError_t vec_to_float(sc_ctx* c, float* y, const double* x, size_t n);
 cudaError_t global_apply(sc_ctx* c, const double* x, double* y);
 cudaError_t scatter_solution(sc_ctx* c, const double* xb, const double* xi, double* x);
 cudaError_t multidot(sc_ctx* c, const double* V, int nvec, size_t n, const double* w, double* out_dev);
+cudaError_t gram_schmidt(sc_ctx* c, const double* V, int nvec, size_t n, double* w, double* h1, double* h2, double* hn2);
+cudaError_t vec_normalize(sc_ctx* c, double* dst, const double* w, size_t n, const double* norm2_dev);
+cudaError_t alloc_gs(sc_ctx* c, int restart);
+void free_gs(sc_ctx* c);
+constexpr int kGsBlocks = 456;  // CTAs of a Gram-Schmidt sweep: 3 x 152 SMs
 cudaError_t vec_update(sc_ctx* c, double* w, const double* V, int nvec, size_t n, const double* coef_dev,
                        double sign);
 cudaError_t vec_scale_copy(sc_ctx* c, double* dst, const double* src, size_t n, const double* scal_dev,

@@ -83,59 +83,139 @@ __global__ void k_scatter(Geo G, const int* __restrict__ iperm, const double* __
   x[((size_t)e * G.nn + iperm[pos]) * 5 + k] = v;
 }
 
-// Partial dot products <V[i], w> over a slice of the vectors: grid (chunks, nvec);
-// partial[i * gridDim.x + chunk].
-// Partial dot products w . v_i over the chunk of block x, one vector per block row y.  With
-// vec2 (n even, both pointers 16-byte aligned) the loads are double2, two chains per thread.
-__global__ void __launch_bounds__(256) k_multidot_partial(const double* __restrict__ V, size_t n,
-                                                          const double* __restrict__ w,
-                                                          double* __restrict__ partial, int vec2) {
-  __shared__ double red[8];
-  const int i = blockIdx.y;
-  const double* v = V + (size_t)i * n;
-  double s = 0.0, s2 = 0.0;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  if (vec2) {
-    const double2* v2 = reinterpret_cast<const double2*>(v);
-    const double2* w2 = reinterpret_cast<const double2*>(w);
-    const size_t n2 = n / 2;
-    size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    for (; t + stride < n2; t += 2 * stride) {
-      const double2 a = __ldg(v2 + t), b = __ldg(w2 + t), c = __ldg(v2 + t + stride), d = __ldg(w2 + t + stride);
-      s = fma(a.x, b.x, s); s2 = fma(a.y, b.y, s2);
-      s = fma(c.x, d.x, s); s2 = fma(c.y, d.y, s2);
+// Gram-Schmidt sweeps over the basis vectors V[0 .. nvec), each n long, against w:
+//   GS_DOTS     out[i] = <V_i, w>
+//   GS_UPDATE   w -= sum_i coef[i] V_i, then out[i] = <V_i, w>
+//   GS_NORM     w -= sum_i coef[i] V_i, then out[0] = <w, w>
+// The CTAs take tiles of 512 entries; the updated tile of w sits in shared memory and the second use of
+// the vectors' tiles hits L1, so CGS2 reads the basis three times from memory, not four.  A warp
+// takes a vector (or a part of the tile, while there are fewer than eight vectors) and
+// keeps its lanes' sums in shared memory; the last CTA to finish adds up the CTAs' partial sums, in a
+// fixed order.  HBM and L2 bound on large systems (16^3 elements of order 4, 15 vectors of 16 MB on
+// average: 0.07 + 0.13 + 0.08 ms, as long as separate products and updates), launch bound on
+// small ones: three launches per iteration in place of eight.  Tried: half a tile per unit for an
+// even load of the warps (16^3: 0.29 ms in all), 2 CTAs per SM (0.32 ms).
+using sc::kGsBlocks;
+enum { GS_DOTS = 0, GS_UPDATE = 1, GS_NORM = 2 };
+constexpr int kGsTile = 512;
+__device__ __forceinline__ double2 gs_load(const double* __restrict__ v, size_t t, size_t n, bool vec2) {
+  if (vec2) return t < n ? *reinterpret_cast<const double2*>(v + t) : make_double2(0.0, 0.0);
+  return make_double2(t < n ? v[t] : 0.0, t + 1 < n ? v[t + 1] : 0.0);
+}
+// Parts of a tile that a vector's dot product is split into: 8, 4, 2 for 1, 2, 3 .. 4 vectors, else 1.
+__host__ __device__ __forceinline__ int gs_parts(int nvec) { return nvec == 1 ? 8 : nvec == 2 ? 4 : nvec <= 4 ? 2 : 1; }
+
+template <int MODE>
+__global__ void __launch_bounds__(256) k_gs(const double* __restrict__ V, int nvec, size_t n, double* w,
+                                            const double* __restrict__ coef, double* __restrict__ partial,
+                                            double* __restrict__ out, unsigned* __restrict__ ticket, int vec2) {
+  extern __shared__ __align__(16) double gsm[];
+  double* ws = gsm;             // [512] the tile of w
+  double* cs = ws + kGsTile;    // [nvec]
+  double* acc = cs + nvec;      // [units][32] the lanes' sums
+  __shared__ bool last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nout = MODE == GS_NORM ? 1 : nvec, parts = MODE == GS_NORM ? 8 : gs_parts(nvec);
+  const int units = nout * parts, span = 8 / parts;  // 64-entry pieces of a unit
+  if (MODE != GS_DOTS)
+    for (int i = tid; i < nvec; i += 256) cs[i] = coef[i];
+  for (int i = tid; i < units * 32; i += 256) acc[i] = 0.0;
+  for (size_t t0 = (size_t)blockIdx.x * kGsTile; t0 < n; t0 += (size_t)gridDim.x * kGsTile) {
+    __syncthreads();
+    {
+      const size_t t = t0 + 2 * tid;
+      double2 x = gs_load(w, t, n, vec2);
+      if (MODE != GS_DOTS) {
+        double2 s0 = make_double2(0.0, 0.0), s1 = s0;
+        int i = 0;
+        for (; i + 8 <= nvec; i += 8) {
+          double2 a[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) a[q] = gs_load(V + (size_t)(i + q) * n, t, n, vec2);
+#pragma unroll
+          for (int q = 0; q < 8; q += 2) {
+            s0.x = fma(cs[i + q], a[q].x, s0.x); s0.y = fma(cs[i + q], a[q].y, s0.y);
+            s1.x = fma(cs[i + q + 1], a[q + 1].x, s1.x); s1.y = fma(cs[i + q + 1], a[q + 1].y, s1.y);
+          }
+        }
+        for (; i + 2 <= nvec; i += 2) {
+          const double2 a = gs_load(V + (size_t)i * n, t, n, vec2), b = gs_load(V + (size_t)(i + 1) * n, t, n, vec2);
+          s0.x = fma(cs[i], a.x, s0.x); s0.y = fma(cs[i], a.y, s0.y);
+          s1.x = fma(cs[i + 1], b.x, s1.x); s1.y = fma(cs[i + 1], b.y, s1.y);
+        }
+        for (; i < nvec; ++i) {
+          const double2 a = gs_load(V + (size_t)i * n, t, n, vec2);
+          s0.x = fma(cs[i], a.x, s0.x); s0.y = fma(cs[i], a.y, s0.y);
+        }
+        x.x -= s0.x + s1.x;
+        x.y -= s0.y + s1.y;
+        if (t < n) w[t] = x.x;
+        if (t + 1 < n) w[t + 1] = x.y;
+      }
+      ws[2 * tid] = x.x;
+      ws[2 * tid + 1] = x.y;
     }
-    if (t < n2) {
-      const double2 a = __ldg(v2 + t), b = __ldg(w2 + t);
-      s = fma(a.x, b.x, s); s2 = fma(a.y, b.y, s2);
+    __syncthreads();
+    for (int u = warp; u < units; u += 8) {
+      const int i = u / parts, q = u % parts;
+      double s0 = 0.0, s1 = 0.0;
+      if (MODE != GS_NORM && parts == 1) {  // all eight pieces' loads in flight
+        double2 a[8];
+#pragma unroll
+        for (int p = 0; p < 8; ++p) a[p] = gs_load(V + (size_t)i * n, t0 + 64 * p + 2 * lane, n, vec2);
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          const double2 y = *reinterpret_cast<const double2*>(ws + 64 * p + 2 * lane);
+          s0 = fma(a[p].x, y.x, s0);
+          s1 = fma(a[p].y, y.y, s1);
+        }
+      } else {
+        for (int p = 0; p < span; ++p) {
+          const int l = 64 * (q * span + p) + 2 * lane;
+          const double2 y = *reinterpret_cast<const double2*>(ws + l);
+          const double2 a = MODE == GS_NORM ? y : gs_load(V + (size_t)i * n, t0 + l, n, vec2);
+          s0 = fma(a.x, y.x, s0);
+          s1 = fma(a.y, y.y, s1);
+        }
+      }
+      acc[u * 32 + lane] += s0 + s1;
     }
-  } else {
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += stride) s = fma(v[t], w[t], s);
   }
-  s = warp_sum(s + s2);
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int k = 0; k < (int)(blockDim.x / 32); ++k) r += red[k];
-    partial[(size_t)i * gridDim.x + blockIdx.x] = r;
+  for (int i = warp; i < nout; i += 8) {
+    double s = 0.0;
+    for (int q = 0; q < parts; ++q) s += acc[(i * parts + q) * 32 + lane];
+    s = warp_sum(s);
+    if (lane == 0) partial[(size_t)i * gridDim.x + blockIdx.x] = s;
   }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = warp; i < nout; i += 8) {
+    constexpr int kPer = (kGsBlocks + 31) / 32;
+    double v[kPer], s = 0.0;  // all loads in flight: a serial sum of them took most of a small sweep's time
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int b = lane + 32 * q;
+      v[q] = b < (int)gridDim.x ? __ldcg(partial + (size_t)i * gridDim.x + b) : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) s += v[q];
+    s = warp_sum(s);
+    if (lane == 0) out[i] = s;
+  }
+  if (tid == 0) *ticket = 0u;  // for the next launch on the stream
 }
 
-__global__ void k_multidot_final(const double* __restrict__ partial, int nchunks, int nvec, double* __restrict__ out) {
-  const int i = blockIdx.x;
-  if (i >= nvec) return;
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nchunks; b += blockDim.x) s += partial[(size_t)i * nchunks + b];
-  s = warp_sum(s);
-  __shared__ double red[8];
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int k = 0; k < (int)(blockDim.x / 32); ++k) r += red[k];
-    out[i] = r;
-  }
+// dst = w / sqrt(norm2)
+__global__ void k_normalize(double* __restrict__ dst, const double* __restrict__ w, size_t n,
+                            const double* __restrict__ norm2) {
+  const double a = 1.0 / sqrt(norm2[0]);
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
+    dst[t] = a * w[t];
 }
 
 // w -= or += sum_i coef[i] v_i (sign); with vec2 (n even, pointers 16-byte aligned) double2
@@ -201,7 +281,6 @@ __global__ void k_axpby(double* __restrict__ y, double a, const double* __restri
 }
 
 constexpr int kDotBlocks = 608;  // 4 x 152 SMs
-constexpr int kDotChunks = 152;
 
 }  // namespace
 
@@ -272,14 +351,62 @@ cudaError_t scatter_solution32(sc_ctx* c, const double* xb, const float* xi, dou
   return cudaGetLastError();
 }
 
-cudaError_t multidot(sc_ctx* c, const double* V, int nvec, size_t n, const double* w, double* out_dev) {
+template <int MODE>
+static cudaError_t gs_launch(sc_ctx* c, const double* V, int nvec, size_t n, double* w, const double* coef,
+                             double* out_dev) {
   if (nvec < 1 || nvec > c->restart_alloc + 1) return cudaErrorInvalidValue;
-  const int chunks = kDotChunks;
-  count_launch(c, 2);
   const int vec2 = n % 2 == 0 && ((reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(w)) & 15) == 0;
-  k_multidot_partial<<<dim3(chunks, nvec), 256, 0, c->stream>>>(V, n, w, c->partial, vec2);
-  k_multidot_final<<<nvec, 256, 0, c->stream>>>(c->partial, chunks, nvec, out_dev);
+  const int blocks = (int)std::max<size_t>(1, std::min<size_t>(kGsBlocks, (n + kGsTile - 1) / kGsTile));
+  const int units = MODE == GS_NORM ? 8 : nvec * gs_parts(nvec);
+  const size_t smem = ((size_t)kGsTile + nvec + 32 * units) * sizeof(double);
+  if (smem > 48 * 1024) {  // restart lengths above 170
+    cudaError_t e = cudaFuncSetAttribute(k_gs<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  count_launch(c);
+  k_gs<MODE><<<blocks, 256, smem, c->stream>>>(V, nvec, n, w, coef, c->partial, out_dev,
+                                             reinterpret_cast<unsigned*>(c->partial + (size_t)kGsBlocks * (c->restart_alloc + 2)),
+                                             vec2);
   return cudaGetLastError();
+}
+
+cudaError_t multidot(sc_ctx* c, const double* V, int nvec, size_t n, const double* w, double* out_dev) {
+  return gs_launch<GS_DOTS>(c, V, nvec, n, const_cast<double*>(w), nullptr, out_dev);  // w is only read
+}
+
+// Classical Gram-Schmidt twice: w is made orthogonal to V[0 .. nvec), the coefficients of the two
+// passes go to h1 and h2, <w, w> of the result to hn2 (all on the device).
+cudaError_t gram_schmidt(sc_ctx* c, const double* V, int nvec, size_t n, double* w, double* h1, double* h2, double* hn2) {
+  cudaError_t e = gs_launch<GS_DOTS>(c, V, nvec, n, w, nullptr, h1);
+  if (e == cudaSuccess) e = gs_launch<GS_UPDATE>(c, V, nvec, n, w, h1, h2);
+  if (e == cudaSuccess) e = gs_launch<GS_NORM>(c, V, nvec, n, w, h2, hn2);
+  return e;
+}
+
+cudaError_t vec_normalize(sc_ctx* c, double* dst, const double* w, size_t n, const double* norm2_dev) {
+  count_launch(c);
+  k_normalize<<<kDotBlocks, 256, 0, c->stream>>>(dst, w, n, norm2_dev);
+  return cudaGetLastError();
+}
+
+// Partial sums, the CTAs' ticket and the pinned copy of the Gram-Schmidt results for a restart length.
+cudaError_t alloc_gs(sc_ctx* c, int restart) {
+  const size_t np = (size_t)kGsBlocks * (restart + 2);
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&c->partial), (np + 1) * sizeof(double));
+  if (e == cudaSuccess) e = cudaMemset(c->partial + np, 0, sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&c->Hd), (3 * (size_t)(restart + 2) + 16) * sizeof(double));
+  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&c->h_gs), (2 * (size_t)(restart + 1) + 1) * sizeof(double));
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_gs, cudaEventDisableTiming);
+  return e;
+}
+
+void free_gs(sc_ctx* c) {
+  if (c->partial) cudaFree(c->partial);
+  if (c->Hd) cudaFree(c->Hd);
+  if (c->h_gs) cudaFreeHost(c->h_gs);
+  if (c->ev_gs) cudaEventDestroy(c->ev_gs);
+  c->partial = c->Hd = c->h_gs = nullptr;
+  c->ev_gs = nullptr;
 }
 
 cudaError_t vec_update(sc_ctx* c, double* w, const double* V, int nvec, size_t n, const double* coef_dev,

@@ -1264,8 +1264,7 @@ sc_status sc_mixed_create(const sc_config* cfg, void* cuda_stream, int n, double
   // Krylov workspace
   m->aux = new sc_ctx();
   m->aux->stream = m->stream; m->aux->cfg = *cfg; m->aux->restart_alloc = m->restart;
-  A(mx_alloc(&m->aux->partial, 152 * (size_t)(m->restart + 2)));
-  A(mx_alloc(&m->aux->Hd, 3 * (size_t)(m->restart + 2) + 16));
+  A(sc::alloc_gs(m->aux, m->restart));
   if (e != cudaSuccess) {
     sc_mixed_destroy(m);
     return SC_ERR_OOM;
@@ -1293,8 +1292,7 @@ void sc_mixed_destroy(sc_mixed* m) {
   if (m->fork) cudaEventDestroy(m->fork);
   for (cudaEvent_t ev : m->prof_ev) cudaEventDestroy(ev);
   if (m->aux) {
-    if (m->aux->partial) cudaFree(m->aux->partial);
-    if (m->aux->Hd) cudaFree(m->aux->Hd);
+    sc::free_gs(m->aux);
     delete m->aux;
   }
   delete m;
@@ -1511,7 +1509,8 @@ sc_status mx_gmres(sc_mixed* m, double tol, int max_iters, int* iters_out) {
   MX_CUDA(cudaMemsetAsync(m->xb, 0, n1 * sizeof(double), m->stream));
   MX_CUDA(cudaMemcpyAsync(m->Tb, m->gb, n1 * sizeof(double), cudaMemcpyDeviceToDevice, m->stream));
   double beta = mx_norm(m, m->Tb, n1);
-  std::vector<double> H((size_t)(mr + 1) * mr), cs(mr), sn(mr), gv(mr + 1), hbuf(2 * (mr + 1) + 1), y(mr);
+  std::vector<double> H((size_t)(mr + 1) * mr), cs(mr), sn(mr), gv(mr + 1), y(mr);
+  double* const hbuf = c->h_gs;
   int iters = 0;
   bool ok = beta <= tol;
   while (!ok && iters < max_iters) {
@@ -1519,21 +1518,28 @@ sc_status mx_gmres(sc_mixed* m, double tol, int max_iters, int* iters_out) {
     std::fill(gv.begin(), gv.end(), 0.0);
     gv[0] = beta;
     int k = 0;
+    bool ahead = false;  // w of this iteration is already under way
     for (int j = 0; j < mr && iters < max_iters; ++j) {
-      MX_CUDA(mx_precond(m, m->V + (size_t)j * n1, m->Zb));
-      MX_CUDA(mx_apply_S(m, m->Zb, m->Wv));
-      MX_CUDA(sc::multidot(c, m->V, j + 1, n1, m->Wv, h1));
-      MX_CUDA(sc::vec_update(c, m->Wv, m->V, j + 1, n1, h1, -1.0));
-      MX_CUDA(sc::multidot(c, m->V, j + 1, n1, m->Wv, h2));
-      MX_CUDA(sc::vec_update(c, m->Wv, m->V, j + 1, n1, h2, -1.0));
-      MX_CUDA(sc::multidot(c, m->Wv, 1, n1, m->Wv, hn2));
-      MX_CUDA(cudaMemcpyAsync(hbuf.data(), c->Hd, (2 * (mr + 1) + 1) * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-      MX_CUDA(cudaStreamSynchronize(m->stream));
+      if (!ahead) {
+        MX_CUDA(mx_precond(m, m->V + (size_t)j * n1, m->Zb));
+        MX_CUDA(mx_apply_S(m, m->Zb, m->Wv));
+      }
+      MX_CUDA(sc::gram_schmidt(c, m->V, j + 1, n1, m->Wv, h1, h2, hn2));
+      MX_CUDA(cudaMemcpyAsync(hbuf, c->Hd, (2 * (mr + 1) + 1) * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+      MX_CUDA(cudaEventRecord(c->ev_gs, m->stream));
+      if (j + 1 < mr) MX_CUDA(sc::vec_normalize(c, m->V + (size_t)(j + 1) * n1, m->Wv, n1, hn2));
+      // the next operator application is enqueued before the host sees this iteration's results,
+      // unless the last estimate says that this one may end the cycle
+      ahead = j + 1 < mr && iters + 1 < max_iters && std::fabs(gv[j]) > 1.5 * tol;
+      if (ahead) {
+        MX_CUDA(mx_precond(m, m->V + (size_t)(j + 1) * n1, m->Zb));
+        MX_CUDA(mx_apply_S(m, m->Zb, m->Wv));
+      }
+      MX_CUDA(cudaEventSynchronize(c->ev_gs));
       for (int i = 0; i <= j; ++i) H[(size_t)i * mr + j] = hbuf[i] + hbuf[(mr + 1) + i];
       const double hn = std::sqrt(std::max(hbuf[2 * (mr + 1)], 0.0));
       H[(size_t)(j + 1) * mr + j] = hn;
       if (!std::isfinite(hn)) return mfail(m, SC_ERR_NONFINITE, "non-finite value in GMRES");
-      if (hn > 0) MX_CUDA(sc::vec_axpby(c, m->V + (size_t)(j + 1) * n1, 1.0 / hn, m->Wv, 0.0, n1));
       for (int i = 0; i < j; ++i) {
         const double a = H[(size_t)i * mr + j], b = H[(size_t)(i + 1) * mr + j];
         H[(size_t)i * mr + j] = cs[i] * a + sn[i] * b;
