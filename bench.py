@@ -593,7 +593,7 @@ def run_mixed_mesh(args, world, rank, local):
     avg_ms = apps_ms / max(n_apps, 1)
     roof = {"bound": "hbm", "achieved": app_bytes / (avg_ms * 1e-3) / 1e9, "peak": float(peaks["hbm_gbs"]),
             "unit": "GB/s", "traffic": None,
-            "kernel": "block-Jacobi application (k_lu_solve_cta, one launch per order class, concurrent)",
+            "kernel": "block-Jacobi application (k_tri_apply, two launches per order class, concurrent)",
             "launches_timed": n_apps, "avg_launch_ms": avg_ms}
     roof["frac"] = roof["achieved"] / roof["peak"]
     clocks = sampler.stop() if sampler else None
