@@ -121,9 +121,10 @@ __global__ void __launch_bounds__(256) k_mlp_gemm(int M, int N, int K, const flo
 // K-major core matrices of 8 rows x 16 bytes): while the tensor cores work on one chunk, the threads split
 // and store the next and load the one after.  Thread t holds row t % 128 (its TMEM lane) and of every
 // 64 columns the half t / 128.  A wait that runs out leaves NaN in its samples' outputs.
-// 100,352 samples: 0.20 ms against 1.84 ms in three SIMT products (and 0.6 ms of host time for their
-// temporaries); 256 samples: 52 against 82 us.  Bound by the chain of one CTA's chunks (split, store,
-// multiply, collect) more than by the tensor cores.
+// 100,352 samples: 0.17 ms a call against 2.43 ms for three SIMT products and their temporaries; a
+// training batch of 256: about 50 us against 82.  Bound by the instruction stream of a CTA's eight warps
+// (split, store, collect), not by the tensor cores.  Tried: pieces of eight rows per warp load (0.21 ms
+// when the split cost more), activations written through shared memory (no gain).
 constexpr int kFwStage = 3 * 128 * 64 * 2 + 256 * 64 * 2;  // bytes
 constexpr int kCoreLbo = 128, kCoreSbo = 8 * kCoreLbo;
 __device__ __forceinline__ uint32_t bf16_core(int row, int k) {
@@ -176,6 +177,37 @@ __device__ __forceinline__ void tmem_add32(uint32_t taddr, float* acc) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 32; ++i) acc[i] += __uint_as_float(r[i >> 3][i & 7]);
+}
+
+// The three parts of eight values, packed in pairs: two subtractions and one byte permutation per pair
+// and part.  The remainders of a finite value are exact, so the sum of the last ones is NaN only if a
+// value is infinite or NaN; those take the careful split (100,352 samples: 209 us with it for all, now 167).
+__device__ __forceinline__ void split3x8(const float* x, uint32_t q[3][4]) {
+  float bad = 0.f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float r[2][2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float v = x[2 * j + h];
+      r[h][0] = v - __uint_as_float(__float_as_uint(v) & 0xffff0000u);
+      r[h][1] = r[h][0] - __uint_as_float(__float_as_uint(r[h][0]) & 0xffff0000u);
+      bad += r[h][1];
+    }
+    q[0][j] = __byte_perm(__float_as_uint(x[2 * j]), __float_as_uint(x[2 * j + 1]), 0x7632);
+    q[1][j] = __byte_perm(__float_as_uint(r[0][0]), __float_as_uint(r[1][0]), 0x7632);
+    q[2][j] = __byte_perm(__float_as_uint(r[0][1]), __float_as_uint(r[1][1]), 0x7632);
+  }
+  if (bad != bad) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      uint32_t lo[3], hi[3];
+      split3(x[2 * j], lo);
+      split3(x[2 * j + 1], hi);
+#pragma unroll
+      for (int s = 0; s < 3; ++s) q[s][j] = lo[s] | hi[s] << 16;
+    }
+  }
 }
 
 struct FwLane {  // what a thread of k_mlp_forward works on
@@ -251,14 +283,7 @@ __device__ __forceinline__ bool fw_layer(FwLane& f, float a[32], uint4 w[8], flo
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       uint32_t q[3][4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        uint32_t lo[3], hi[3];
-        split3(a[8 * i + 2 * j], lo);
-        split3(a[8 * i + 2 * j + 1], hi);
-#pragma unroll
-        for (int s = 0; s < 3; ++s) q[s][j] = lo[s] | hi[s] << 16;
-      }
+      split3x8(a + 8 * i, q);
 #pragma unroll
       for (int s = 0; s < 3; ++s)
         *reinterpret_cast<uint4*>(As + s * 16384 + bf16_core(f.row, 32 * f.half + 8 * i)) =
