@@ -447,9 +447,11 @@ sc_status sc_learned_features(sc_ctx* ctx, float* F, float* snorm);
 
 /* Training targets T[s][25] = ([S_ee^-1]_kk - [S_ee]_kk^-1) ||[S_ee]_kk||_F for every sample
    (row-major 5 x 5; elements of both colours): the correction of the inverse of the node block
-   to the node block of the face-block inverse, [S_ee^-1]_kk from unit solves with the
-   condensation's factors.  After sc_condense on the mixed arm.  Device pointer, K * nbn * 25
-   floats. */
+   to the node block of the face-block inverse, [S_ee^-1]_kk with the condensation's factors
+   (SC_PC_NONE and SC_PC_RB_SCHUR, whose condensation keeps no factors of every S_ee: with
+   factors formed for this call and temporaries of up to 256 elements; SC_ERR_SINGULAR_BLOCK
+   where one does not exist).  After sc_condense on the mixed arm.  Device pointer,
+   K * nbn * 25 floats. */
 sc_status sc_learned_targets(sc_ctx* ctx, float* T);
 
 /* Network parameters for SC_PC_LEARNED (device pointers, layout of sc_mlp_forward; copied

@@ -1780,9 +1780,37 @@ __global__ void __launch_bounds__(128) k_inv_node_blocks(int n, int nblk, const 
   if (lane < 5) out[(long long)smp * 25 + 5 * lane + var] = s[5 * a + lane];
 }
 
+// The same where the condensation kept no factors of every element (no preconditioner, or the
+// Schur-corrected sweep, which factorises the red and the corrected black blocks): the S_ee
+// blocks, which it then left as they were, are factorised here, some elements at a time.
+// *c->d_status: -1, or what the factorisation reported.
+static cudaError_t inverse_node_blocks_refactor(sc_ctx* c, float* out) {
+  const Geo& G = c->G;
+  const int chunk = std::min(G.K, 256);
+  const size_t per = (size_t)G.nb * G.lds;
+  struct Tmp { void* p[4] = {}; ~Tmp() { for (void* q : p) cudaFree(q); } } tmp;
+  cudaError_t e = cudaMalloc(&tmp.p[0], chunk * per * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&tmp.p[1], (size_t)chunk * ls_stride(G) * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&tmp.p[2], (size_t)chunk * G.nb * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&tmp.p[3], (size_t)chunk * G.nb * sizeof(int));
+  float *A = static_cast<float*>(tmp.p[0]), *LS = static_cast<float*>(tmp.p[1]);
+  int *piv = static_cast<int*>(tmp.p[2]), *rowperm = static_cast<int*>(tmp.p[3]);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0xff, sizeof(int), c->stream);
+  for (int e0 = 0; e0 < G.K && e == cudaSuccess; e0 += chunk) {
+    const int m = std::min(chunk, G.K - e0);
+    e = cudaMemcpyAsync(A, c->See32 + e0 * per, m * per * sizeof(float), cudaMemcpyDeviceToDevice, c->stream);
+    if (e == cudaSuccess)
+      e = factor_batch32(c, A, G.nb, G.lds, (long long)per, m, piv, rowperm, LS, c->d_status, true);
+    if (e == cudaSuccess) e = tri_node_blocks(c, LS, rowperm, m, out + (size_t)e0 * G.nbn * 25);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // before the buffers go
+  return e;
+}
+
 cudaError_t inverse_node_blocks32(sc_ctx* c, float* out) {
   const Geo& G = c->G;
-  if (c->ls_full || c->red_compact) return tri_node_blocks(c, c->Sls32, c->rowperm, out);
+  if (c->cfg.precond == SC_PC_NONE || c->red_compact) return inverse_node_blocks_refactor(c, out);
+  if (c->ls_full) return tri_node_blocks(c, c->Sls32, c->rowperm, G.K, out);
   const int nblk = ls_nblk(G);
   const size_t smem = (size_t)4 * nblk * 32 * sizeof(float);
   cudaError_t err = cudaFuncSetAttribute(k_inv_node_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

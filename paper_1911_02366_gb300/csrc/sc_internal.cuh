@@ -541,7 +541,7 @@ cudaError_t tri_solve(sc_ctx* c, const TS* LS, const int* rowperm, int compact, 
 cudaError_t tri_dense_inverse(sc_ctx* c, const float* LS, const int* rowperm, int count, float* out);
 cudaError_t dense_inverse_apply(sc_ctx* c, const float* inv, const int* elist, int count, const double* v, double* z,
                                 float* zt);
-cudaError_t tri_node_blocks(sc_ctx* c, const float* LS, const int* rowperm, float* out);
+cudaError_t tri_node_blocks(sc_ctx* c, const float* LS, const int* rowperm, int count, float* out);
 void build_learned_tables(sc_ctx* c);
 void build_explicit_tables(sc_ctx* c);
 cudaError_t upload_explicit_tables(sc_ctx* c);

@@ -403,9 +403,16 @@ sc_status sc_learned_targets(sc_ctx* c, float* T) {
     k_inverse_targets<<<(nsmp + 127) / 128, 128, 0, c->stream>>>(nsmp, Zex, c->Sdiag, T);
     e = cudaGetLastError();
   }
+  int bad = -1;  // of the factors formed for this call, if any
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   cudaFree(Zex);
-  return e == cudaSuccess ? SC_OK : SC_ERR_CUDA;
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return SC_ERR_OOM;
+  }
+  if (e != cudaSuccess || bad >= SC_TC_TIMEOUT) return SC_ERR_CUDA;
+  return bad >= 0 ? SC_ERR_SINGULAR_BLOCK : SC_OK;
 }
 
 sc_status sc_set_learned_correction(sc_ctx* c, const float* Y, float scale) {

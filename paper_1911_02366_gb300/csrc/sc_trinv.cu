@@ -401,6 +401,8 @@ __global__ void __launch_bounds__(128) k_tri_node_blocks(int n, const float* __r
   if (smp >= nsmp) return;
   const int nbn = n / 5, e = smp / nbn, a = smp % nbn, w = threadIdx.x >> 5;
   const int* rp = rowperm + (long long)e * n;
+  if (lane < 5) pos[w][lane] = n;  // a column that no row maps to meets no entry below
+  __syncwarp();
   for (int i = lane; i < n; i += 32) {
     const int d = __ldg(rp + i) - 5 * a;
     if (d >= 0 && d < 5) pos[w][d] = i;
@@ -526,9 +528,10 @@ cudaError_t dense_inverse_apply(sc_ctx* c, const float* inv, const int* elist, i
   return cudaGetLastError();
 }
 
-cudaError_t tri_node_blocks(sc_ctx* c, const float* LS, const int* rowperm, float* out) {
+// out: of `count` elements, 25 values per boundary node.
+cudaError_t tri_node_blocks(sc_ctx* c, const float* LS, const int* rowperm, int count, float* out) {
   const Geo& G = c->G;
-  const int nblk = (G.nb + 31) / 32, npad = (G.nb + 3) & ~3, nsmp = G.K * G.nbn;
+  const int nblk = (G.nb + 31) / 32, npad = (G.nb + 3) & ~3, nsmp = count * G.nbn;
   count_launch(c);
   k_tri_node_blocks<<<(nsmp + 3) / 4, 128, 0, c->stream>>>(G.nb, LS, (long long)nblk * 32 * npad, npad, rowperm, nsmp,
                                                          out);
