@@ -1490,9 +1490,9 @@ cudaError_t condense_t(sc_ctx* c, T* Aown, T* Ainv, T* Y, T* See, bool tc, bool 
   if (c->cfg.precond != SC_PC_NONE) {
     bool done = false;
     if constexpr (std::is_same<T, float>::value) {
-      if (tc && c->cfg.precond == SC_PC_RB_SCHUR && c->SeeL) {
+      if (c->cfg.precond == SC_PC_RB_SCHUR && c->SeeL) {
         // the Schur-corrected sweep factorises only the red blocks here; the black ones are
-        // factorised once, after their correction
+        // factorised once, after their correction (factor_batch32 heeds tensor_cores)
         err = red_factor32(c, See);
         if (err != cudaSuccess) return err;
         c->red_compact = true;
