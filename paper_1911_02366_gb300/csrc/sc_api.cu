@@ -225,7 +225,7 @@ sc_status sc_default_config(sc_config* cfg) {
 
 sc_status sc_create(const sc_config* cfg, void* cuda_stream, sc_ctx** out) {
   if (!cfg || !out) return SC_ERR_ARG;
-  if (cfg->gmres_restart < 1 || cfg->gmres_restart > 400 || cfg->gmres_max_iters < 1 || !(cfg->rel_tol > 0) ||
+  if (cfg->gmres_restart < 1 || cfg->gmres_restart > sc::kMaxRestart || cfg->gmres_max_iters < 1 || !(cfg->rel_tol > 0) ||
       !(cfg->Re > 0) || !(cfg->Ma > 0) || !(cfg->gamma > 1) || !(cfg->Pr > 0))
     return SC_ERR_ARG;
   if (cfg->precision != SC_PREC_FP64 && cfg->precision != SC_PREC_MIXED) return SC_ERR_ARG;

@@ -651,7 +651,9 @@ inline unsigned blocks_for(size_t n, int bs) { return (unsigned)((n + bs - 1) / 
 
 namespace sc {
 
-// Shared memory of the residual kernels per CTA.
+// Shared memory of the residual kernels per CTA, and what order 6 takes (one element per CTA, the most of all).
+constexpr int kPointSmemMax = (64 + kMaxNodes * 20) * (int)sizeof(double);
+constexpr int kRowsSmemMax = (64 + kMaxNodes * 20 + 30 * kMaxP * kMaxP) * (int)sizeof(double);
 static size_t point_smem(const Geo& G) { return (64 + (size_t)group_elems(G) * G.nn * 20) * sizeof(double); }
 static size_t rows_smem(const Geo& G) {
   return (64 + (size_t)group_elems(G) * (G.nn * 20 + 30 * G.p * G.p)) * sizeof(double);
@@ -660,7 +662,7 @@ static size_t rows_smem(const Geo& G) {
 template <bool IP>
 static cudaError_t launch_point(sc_ctx* c, const Geo& G, const double* Q, bool store_grad, unsigned long long* spd) {
   const int ge = group_elems(G);
-  cudaError_t e = cudaFuncSetAttribute(k_point<IP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)point_smem(G));
+  cudaError_t e = cudaFuncSetAttribute(k_point<IP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPointSmemMax);
   if (e != cudaSuccess) return e;
   count_launch(c);
   k_point<IP><<<(G.K + ge - 1) / ge, group_threads(G), point_smem(G), c->stream>>>(
@@ -671,7 +673,7 @@ static cudaError_t launch_point(sc_ctx* c, const Geo& G, const double* Q, bool s
 template <bool IP, bool RK>
 static cudaError_t launch_rows(sc_ctx* c, const Geo& G, const double* Q, const double* Qh, double* out, const RkStage& st) {
   const int ge = group_elems(G);
-  cudaError_t e = cudaFuncSetAttribute(k_rows<IP, RK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem(G));
+  cudaError_t e = cudaFuncSetAttribute(k_rows<IP, RK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmemMax);
   if (e != cudaSuccess) return e;
   count_launch(c);
   k_rows<IP, RK><<<(G.K + ge - 1) / ge, group_threads(G), rows_smem(G), c->stream>>>(G, ge, Q, Qh, c->F, c->Floc, c->diss, c->d_nbr,

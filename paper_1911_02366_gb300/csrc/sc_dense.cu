@@ -1324,7 +1324,8 @@ namespace sc {
 template <class T>
 static cudaError_t lu_blocked_simt(sc_ctx* c, int n, T* A, long long stride, int lda, int batch, int* piv, int* status) {
   const size_t smem = (size_t)n * (PW + 1) * sizeof(T);
-  cudaError_t err = cudaFuncSetAttribute(k_lu_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t err = cudaFuncSetAttribute(k_lu_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxNb<T> * (PW + 1) * (int)sizeof(T));
   if (err != cudaSuccess) return err;
   for (int k0 = 0; k0 < n; k0 += PW) {
     const int bw = min(PW, n - k0), rest = n - k0 - bw;
@@ -1349,7 +1350,8 @@ static cudaError_t lu_blocked_tf32_batch(sc_ctx* c, float* See, int K, int* piv,
   const long long sS = (long long)nb * lds;
   const size_t smem = (size_t)nb * (PW + 1) * sizeof(float);
   const bool reg = nb <= LPR_ROWS, reg2 = !reg && nb <= LPR2_ROWS;
-  cudaError_t err = cudaFuncSetAttribute(k_lu_panel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t err = cudaFuncSetAttribute(k_lu_panel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxNb<float> * (PW + 1) * (int)sizeof(float));
   if (err != cudaSuccess) return err;
   for (int k0 = 0; k0 < nb; k0 += PW) {
     const int bw = min(PW, nb - k0), rest = nb - k0 - bw;
@@ -1434,7 +1436,7 @@ cudaError_t condense_t(sc_ctx* c, T* Aown, T* Ainv, T* Y, T* See, bool tc, bool 
       done = true;
     }
     if (!done) {
-      err = cudaFuncSetAttribute(k_gj_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      err = cudaFuncSetAttribute(k_gj_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGjSmemMax);
       if (err != cudaSuccess) return err;
       ProfScope ps(c, SCK_GJ_INV);
       k_gj_inv<T><<<K, 256, smem, c->stream>>>(ni, Aown, sA, lda, Ainv, (long long)ni * ldi, ldi, c->d_status);
@@ -1680,7 +1682,8 @@ cudaError_t grouped_lu_panel(cudaStream_t st, const CondItem* items, int n, int 
     k_lu_panel_reg2_grouped<<<nbig, 32 * LPR2_W, 0, st>>>(items, k0);
   } else if (nbig > 0) {
     const size_t smem = (size_t)max_nb * (PW + 1) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_lu_panel_grouped, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_lu_panel_grouped, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxNb<float> * (PW + 1) * (int)sizeof(float));
     if (e != cudaSuccess) return e;
     k_lu_panel_grouped<<<nbig, 256, smem, st>>>(items, k0);
   }
@@ -1813,7 +1816,8 @@ cudaError_t inverse_node_blocks32(sc_ctx* c, float* out) {
   if (c->ls_full) return tri_node_blocks(c, c->Sls32, c->rowperm, G.K, out);
   const int nblk = ls_nblk(G);
   const size_t smem = (size_t)4 * nblk * 32 * sizeof(float);
-  cudaError_t err = cudaFuncSetAttribute(k_inv_node_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t err = cudaFuncSetAttribute(k_inv_node_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         4 * ((kMaxNb<float> + 31) / 32) * 32 * (int)sizeof(float));
   if (err != cudaSuccess) return err;
   count_launch(c);
   const long long nw = (long long)G.K * G.nbn * 5;

@@ -474,6 +474,16 @@ constexpr int SC_PACK_VIOLATION = (1 << 30) + 1;
 constexpr int SC_EXPLICIT_PATTERN = (1 << 30) + 2;
 
 namespace sc {
+// Dynamic shared-memory limits.  cudaFuncAttributeMaxDynamicSharedMemorySize belongs to a function,
+// not to a context: a host thread that set it to its own mesh's size could lower it between
+// another's set and launch.  So every launch sets the same value, the size of the largest mesh:
+// order 6 on the mixed arm, 5 on the FP64 arm (whose own blocks are FP64 on both arms).
+constexpr int kMaxP = 7, kMaxNodes = kMaxP * kMaxP * kMaxP, kMaxNi = 5 * (kMaxP - 2) * (kMaxP - 2) * (kMaxP - 2);
+constexpr int kMaxLda = (((kMaxNi + 3) & ~3) + 5 * kMaxNodes - kMaxNi + 3) & ~3;
+template <class T> constexpr int kMaxNb = 5 * (kMaxNodes - (kMaxP - 2) * (kMaxP - 2) * (kMaxP - 2));
+template <> constexpr int kMaxNb<double> = 5 * (216 - 64);
+constexpr int kMaxRestart = 400;
+
 // Gauss-Lobatto nodes x, weights w and differentiation matrix D[a][b] = l_b'(x_a) of order N.
 void gl_basis(int N, std::vector<double>& x, std::vector<double>& w, double D[SC_MAXP][SC_MAXP]);
 cudaError_t launch_residual(sc_ctx* c);

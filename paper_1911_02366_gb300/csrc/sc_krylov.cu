@@ -360,7 +360,8 @@ static cudaError_t gs_launch(sc_ctx* c, const double* V, int nvec, size_t n, dou
   const int units = MODE == GS_NORM ? 8 : nvec * gs_parts(nvec);
   const size_t smem = ((size_t)kGsTile + nvec + 32 * units) * sizeof(double);
   if (smem > 48 * 1024) {  // restart lengths above 170
-    cudaError_t e = cudaFuncSetAttribute(k_gs<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr int most = (kGsTile + (kMaxRestart + 1) * 33) * (int)sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(k_gs<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return e;
   }
   count_launch(c);

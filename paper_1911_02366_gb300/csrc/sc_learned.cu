@@ -322,7 +322,8 @@ cudaError_t learned_couplings(sc_ctx* c) {
   const Geo& G = c->G;
   const int nsmp = G.K * G.nbn;
   const size_t smem = (size_t)8 * (G.ni * 5 + 32) * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(k_learned_coupling, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_learned_coupling, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       8 * (kMaxNi * 5 + 32) * (int)sizeof(float));
   if (e != cudaSuccess) return e;
   count_launch(c);
   k_learned_coupling<<<(3 * nsmp + 7) / 8, 256, smem, c->stream>>>(G, c->Aown32, c->Ainv32, c->X, c->d_pptr,

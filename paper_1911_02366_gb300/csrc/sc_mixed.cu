@@ -1085,7 +1085,7 @@ sc_status sc_mixed_create(const sc_config* cfg, void* cuda_stream, int n, double
   if (n < 2 || n > 32 || !(L > 0)) return SC_ERR_ARG;
   if (cfg->precision != SC_PREC_MIXED || (cfg->precond != SC_PC_BLOCK_JACOBI && cfg->precond != SC_PC_NONE) ||
       cfg->visc_flux != SC_VISC_BR1 || (cfg->adv_flux != SC_FLUX_ROE && cfg->adv_flux != SC_FLUX_LF) ||
-      cfg->gmres_restart < 1 || cfg->gmres_restart > 400 || cfg->gmres_max_iters < 1 || !(cfg->rel_tol > 0) ||
+      cfg->gmres_restart < 1 || cfg->gmres_restart > sc::kMaxRestart || cfg->gmres_max_iters < 1 || !(cfg->rel_tol > 0) ||
       !(cfg->inner_tol > 0) || !(cfg->Re > 0) || !(cfg->Ma > 0) || !(cfg->gamma > 1) || !(cfg->Pr > 0))
     return SC_ERR_ARG;
   const int K = n * n * n;

@@ -456,7 +456,8 @@ template <class T>
 static cudaError_t pack_t(sc_ctx* c, T* Apk, float* dense32) {
   const Geo& G = c->G;
   const size_t smem = (size_t)8 * (G.lda + 4) * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(k_pack<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_pack<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       8 * (kMaxLda + 4) * (int)sizeof(double));
   if (e != cudaSuccess) return e;
   count_launch(c);
   const int split = std::max(1, std::min((G.ne + 7) / 8, (4 * 152 * 4 + G.K - 1) / G.K));

@@ -328,7 +328,8 @@ cudaError_t launch_tf32(cudaStream_t stream, int M, int N, int K, float alpha, c
   constexpr int kMaxCtas = 512 / (int)tmem_cols_for(BN);
   constexpr size_t kSmemSM = 228 * 1024, kMinSmem = kSmemSM / (kMaxCtas + 1) - 1024 + 16;
   const size_t smem = std::max(K <= TC_BK ? tc_stage_bytes<BN>() : smem2, kMinSmem);
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_tf32<BN, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_gemm_tf32<BN, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)std::max(smem2, kMinSmem));
   if (e != cudaSuccess) return e;
   dim3 grid((N + BN - 1) / BN, (M + TC_BM - 1) / TC_BM, batch);
   k_gemm_tf32<BN, TA, TB><<<grid, 128, smem, stream>>>(M, N, K, alpha, A, sA, lda, B, sB, ldb, beta, C, sC, ldc, flags,

@@ -459,7 +459,7 @@ cudaError_t tri_inverse(sc_ctx* c, int n, const T* LU, long long stride, int lda
   const int nblk = (n + 31) / 32, npad = (n + 3) & ~3;
   const long long ls = (long long)nblk * 32 * npad;
   cudaError_t e = cudaFuncSetAttribute(k_tri_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)tri_inv_smem<T>(nblk));
+                                       (int)tri_inv_smem<T>((kMaxNb<T> + 31) / 32));
   if (e != cudaSuccess) return e;
   return tri_inv_halves(nblk, [&](int x0, int nx, int blocks) {
     count_launch(c);
@@ -476,7 +476,7 @@ cudaError_t grouped_tri_inverse(cudaStream_t st, const CondItem* items, int coun
   if (count <= 0) return cudaSuccess;
   const int nblk = (nb + 31) / 32;
   cudaError_t e = cudaFuncSetAttribute(k_tri_inv_grouped, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)tri_inv_smem<float>(nblk));
+                                       (int)tri_inv_smem<float>((kMaxNb<float> + 31) / 32));
   if (e != cudaSuccess) return e;
   return tri_inv_halves(nblk, [&](int x0, int nx, int blocks) {
     k_tri_inv_grouped<<<dim3(nx, count, 2), 32 * TiWarps<float>::v, tri_inv_smem<float>(blocks), st>>>(items, x0);
