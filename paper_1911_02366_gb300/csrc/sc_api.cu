@@ -462,6 +462,7 @@ sc_status sc_set_mesh(sc_ctx* c, int n, double L, int N) {
   SC_CUDA(cudaMemset(c->Aown, 0, (size_t)G.K * own_stride(G) * sizeof(double)));
   if (c->Ainv) SC_CUDA(cudaMemset(c->Ainv, 0, (size_t)G.K * G.ni * G.ldi * sizeof(double)));
   if (c->Ainv32) SC_CUDA(cudaMemset(c->Ainv32, 0, (size_t)G.K * G.ni * G.ldi * sizeof(float)));
+  SC_CUDA(sc::finish_setup());
   c->has_mesh = true;
   return SC_OK;
 }

@@ -237,6 +237,7 @@ sc_status sc_batch_create(sc_ctx* const* ctxs, int nctx, sc_batch** out) {
     e = cudaMemcpy(b->d_items, b->items.data(), b->items.size() * sizeof(CondItem), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemcpy(b->d_ptrs, b->h_ptrs.data(), b->h_ptrs.size() * sizeof(void*), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = sc::finish_setup();
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming);

@@ -639,6 +639,7 @@ sc_status direct_factor_t(sc_ctx* c, int which, double* ms_form, double* ms_fact
   for (int i = 0; i < n; ++i) perm[i] = i;
   for (int j = 0; j < n; ++j) std::swap(perm[j], perm[piv[j]]);
   DC_CUDA(cudaMemcpy(c->d_dpiv, perm.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice));
+  DC_CUDA(sc::finish_setup());
   c->direct_n = n;
   c->direct_ld = (int)ldd;
   c->direct_which = which;

@@ -486,6 +486,9 @@ constexpr int kMaxRestart = 400;
 
 // Gauss-Lobatto nodes x, weights w and differentiation matrix D[a][b] = l_b'(x_a) of order N.
 void gl_basis(int N, std::vector<double>& x, std::vector<double>& w, double D[SC_MAXP][SC_MAXP]);
+// Set-up copies and fills go through the legacy stream, and a copy from pageable memory may return
+// before its data has arrived; a caller's non-blocking stream is ordered behind neither.
+inline cudaError_t finish_setup() { return cudaStreamSynchronize(cudaStreamLegacy); }
 cudaError_t launch_residual(sc_ctx* c);
 // -R(Q) with the geometry G (c0 = 0 gives -H(Q), the spatial operator alone) into out;
 // fills c->grad (and c->gloc) and uses c->F as scratch.

@@ -1265,6 +1265,7 @@ sc_status sc_mixed_create(const sc_config* cfg, void* cuda_stream, int n, double
   m->aux = new sc_ctx();
   m->aux->stream = m->stream; m->aux->cfg = *cfg; m->aux->restart_alloc = m->restart;
   A(sc::alloc_gs(m->aux, m->restart));
+  A(sc::finish_setup());
   if (e != cudaSuccess) {
     sc_mixed_destroy(m);
     return SC_ERR_OOM;
@@ -1369,7 +1370,7 @@ sc_status sc_mixed_own_block(sc_mixed* m, int e, double* block) {
   cudaError_t ce = mx_alloc(&scr, (size_t)(nwork * slot));
   if (ce == cudaSuccess) ce = mx_alloc(&d_work, nwork);
   if (ce == cudaSuccess) ce = mx_alloc(&d_next, 1);
-  if (ce == cudaSuccess) ce = cudaMemcpy(d_work, work.data(), nwork * sizeof(int2), cudaMemcpyHostToDevice);
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(d_work, work.data(), nwork * sizeof(int2), cudaMemcpyHostToDevice, m->stream);
   if (ce == cudaSuccess) ce = mx_alloc(&blk, (size_t)ne * ne);
   if (ce == cudaSuccess) ce = mx_alloc(&outp, 1);
   if (ce == cudaSuccess) ce = mx_alloc(&el, 1);
