@@ -382,7 +382,8 @@ sc_status sc_hessenberg_eigvals(int m, const double* H, double* re, double* im);
    b = [b1 (256) | b2 (256) | b3 (25)], FP32.  Layers: h1 = relu(W1 x + b1),
    h2 = relu(W2 h1 + b2), y = W3 h2 + b3; FP32 arithmetic.  All pointers are device pointers
    unless stated; work is enqueued on cuda_stream and synchronised before return.
-   SC_ERR_ARG for null pointers or bad sizes, SC_ERR_CUDA for launch failures. */
+   SC_ERR_ARG for null pointers or bad sizes, SC_ERR_CUDA for launch failures and for a wait on
+   the tensor cores that runs out (sc_mlp_train then stops before the update). */
 
 /* y[n x 25] = net(X[n x 128]).  cache: NULL, or 4 n x 256 floats that receive z1, h1, z2,
    h2 (pre- and post-activations) for sc_mlp_backward. */

@@ -374,7 +374,7 @@ cudaError_t learned_correction(sc_ctx* c) {
   const int nsmp = G.K * G.nbn;
   cudaError_t e = learned_features(c, c->Feat, c->Snorm);
   if (e == cudaSuccess)
-    e = mlp_forward(c->stream, c->Wbf16, c->Wbias, c->Feat, nsmp, c->Ynet);
+    e = mlp_forward(c->stream, c->Wbf16, c->Wbias, c->Feat, nsmp, c->Ynet, c->d_status);
   if (e == cudaSuccess) e = assemble_correction(c, c->Ynet, kNetworkDamping);
   return e;
 }

@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256) k_mlp_gemm(int M, int N, int K, const flo
 // staged in two shared-memory buffers (three 128 x 64 parts and a 256 x 64 piece of the weights,
 // K-major core matrices of 8 rows x 16 bytes): while the tensor cores work on one chunk, the threads split
 // and store the next and load the one after.  Thread t holds row t % 128 (its TMEM lane) and of every
-// 64 columns the half t / 128.  A wait that runs out leaves NaN in its samples' outputs.
+// 64 columns the half t / 128.  A wait that runs out leaves SC_TC_TIMEOUT in *status and NaN in its samples' outputs.
 // 100,352 samples: 0.17 ms a call against 2.43 ms for three SIMT products and their temporaries; a
 // training batch of 256: about 50 us against 82.  Bound by the instruction stream of a CTA's eight warps
 // (split, store, collect), not by the tensor cores.  Tried: pieces of eight rows per warp load (0.21 ms
@@ -143,10 +143,15 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
 constexpr uint32_t idesc_bf16(int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
-__device__ __forceinline__ bool wait_bounded(uint64_t* bar, uint32_t parity) {
-  for (long long it = 0; it <= kWaitLimit; ++it)
-    if (mbar_try_wait(bar, parity)) return true;
-  return false;
+// Polls of the forward pass's waits before it gives up (a build with -1 gives up at once).
+#ifndef SC_MLP_WAIT_POLLS
+#define SC_MLP_WAIT_POLLS kWaitLimit
+#endif
+// The same for all lanes of a warp.
+__device__ __forceinline__ bool wait_bounded(uint64_t* bar, uint32_t parity, long long limit) {
+  bool done = false;
+  for (long long it = 0; it <= limit && !done; ++it) done = mbar_try_wait(bar, parity);
+  return __all_sync(0xffffffffu, done);
 }
 // x = p[0] + p[1] + p[2] in BF16 (bit patterns); infinities and NaN stay in the first part.
 __device__ __forceinline__ void split3(float x, uint32_t p[3]) {
@@ -262,7 +267,8 @@ __device__ __forceinline__ bool fw_layer(FwLane& f, float a[32], uint4 w[8], flo
 #pragma unroll
   for (int i = 0; i < 32 * NQ; ++i) acc[i] = 0.f;
   auto collect = [&]() {  // the products of the chunk before
-    ok = ok && wait_bounded(f.bar, (f.step - 1) & 1);
+    ok = ok && wait_bounded(f.bar, (f.step - 1) & 1, SC_MLP_WAIT_POLLS);
+    if (!ok) return;  // as a condition of the loads below: 2.5 us of 167 per 100,352 samples
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (L < 2 || f.half == 0)
 #pragma unroll
@@ -356,7 +362,7 @@ __global__ void __launch_bounds__(256, 1) k_mlp_forward(int n, const __nv_bfloat
                                                         const float* __restrict__ bias, const float* __restrict__ X,
                                                         float* __restrict__ Y, float* __restrict__ z1,
                                                         float* __restrict__ h1, float* __restrict__ z2,
-                                                        float* __restrict__ h2, int flags) {
+                                                        float* __restrict__ h2, int flags, int* status) {
   extern __shared__ __align__(1024) unsigned char stage_mem[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_s;
@@ -387,7 +393,13 @@ __global__ void __launch_bounds__(256, 1) k_mlp_forward(int n, const __nv_bfloat
     fw_activate(f, bias_s + OFF_B2, acc, z2, h2);
     ok = fw_layer<2>(f, a, w, acc);
   }
-  if (!ok && f.step > 0) wait_bounded(&mbar, (f.step - 1) & 1);  // products still in flight
+  if (!ok) {
+    if (f.step > 0) wait_bounded(&mbar, (f.step - 1) & 1, kWaitLimit);  // products still in flight
+    if (tid == 0) {  // device memory or a mapped host word
+      *reinterpret_cast<volatile int*>(status) = SC_TC_TIMEOUT;
+      __threadfence_system();
+    }
+  }
   if (f.half == 0 && f.gr < n)
 #pragma unroll
     for (int i = 0; i < NO; ++i)
@@ -398,12 +410,13 @@ __global__ void __launch_bounds__(256, 1) k_mlp_forward(int n, const __nv_bfloat
 }
 
 cudaError_t forward(cudaStream_t st, const __nv_bfloat16* W, const float* bias, const float* X, int n, float* Y,
-                    float* z1, float* h1, float* z2, float* h2) {
+                    float* z1, float* h1, float* z2, float* h2, int* status) {
   auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   const int flags = (a16(X) ? 1 : 0) | (a16(W) ? 2 : 0) | (a16(z1) && a16(h1) && a16(z2) && a16(h2) ? 4 : 0);
   cudaError_t e = cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kFwStage);
   if (e != cudaSuccess) return e;
-  k_mlp_forward<<<(unsigned)((n + 127) / 128), 256, 2 * kFwStage, st>>>(n, W, bias, X, Y, z1, h1, z2, h2, flags);
+  k_mlp_forward<<<(unsigned)((n + 127) / 128), 256, 2 * kFwStage, st>>>(n, W, bias, X, Y, z1, h1, z2, h2, flags,
+                                                                         status);
   return cudaGetLastError();
 }
 
@@ -507,16 +520,49 @@ uint64_t splitmix64_next(uint64_t& state) {
   return z ^ (z >> 31);
 }
 
+// The word in which a forward pass of this host thread reports a wait that ran out: mapped host memory, so
+// that reading it after the call's synchronisation costs no copy; given back with the thread.
+struct StatusWord {
+  int* p = nullptr;
+  ~StatusWord() { if (p) cudaFreeHost(p); }
+};
+cudaError_t status_word(int** host, int** device) {
+  static thread_local StatusWord w;
+  void* d = nullptr;
+  if (w.p && cudaHostGetDevicePointer(&d, w.p, 0) != cudaSuccess) {  // gone with a device reset
+    (void)cudaGetLastError();
+    w.p = nullptr;
+  }
+  if (!w.p) {
+    // another thread may be capturing a graph
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return e;
+    void* q = nullptr;
+    e = cudaHostAlloc(&q, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped);
+    const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess || back != cudaSuccess) return e != cudaSuccess ? e : back;
+    w.p = static_cast<int*>(q);
+    e = cudaHostGetDevicePointer(&d, w.p, 0);
+    if (e != cudaSuccess) return e;
+  }
+  *host = w.p;
+  *device = static_cast<int*>(d);
+  return cudaSuccess;
+}
+
 constexpr char kMlpMagic[8] = {'S', 'C', 'M', 'L', 'P', '0', '0', '1'};
 
 }  // namespace
 
 namespace sc {
 
-// Inference: Y = net(X).
-cudaError_t mlp_forward(cudaStream_t st, const uint16_t* Wbf16, const float* bias, const float* X, int n, float* Y) {
+// Inference: Y = net(X); *status (device) <- SC_TC_TIMEOUT if a wait runs out.
+cudaError_t mlp_forward(cudaStream_t st, const uint16_t* Wbf16, const float* bias, const float* X, int n, float* Y,
+                        int* status) {
   if (n <= 0) return cudaSuccess;
-  return forward(st, reinterpret_cast<const __nv_bfloat16*>(Wbf16), bias, X, n, Y, nullptr, nullptr, nullptr, nullptr);
+  return forward(st, reinterpret_cast<const __nv_bfloat16*>(Wbf16), bias, X, n, Y, nullptr, nullptr, nullptr, nullptr,
+                 status);
 }
 
 }  // namespace sc
@@ -531,9 +577,13 @@ sc_status sc_mlp_forward(const uint16_t* Wbf16, const float* bias, const float* 
   const __nv_bfloat16* W = reinterpret_cast<const __nv_bfloat16*>(Wbf16);
   // cache: [z1 | h1 | z2 | h2], each n x 256 (pre- and post-activations)
   auto part = [&](int i) { return cache ? cache + (size_t)i * n * NH : nullptr; };
-  cudaError_t e = forward(st, W, bias, X, n, Y, part(0), part(1), part(2), part(3));
+  int *word = nullptr, *dword = nullptr;
+  cudaError_t e = status_word(&word, &dword);
+  if (e != cudaSuccess) return SC_ERR_CUDA;
+  *word = 0;
+  e = forward(st, W, bias, X, n, Y, part(0), part(1), part(2), part(3), dword);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  return e == cudaSuccess ? SC_OK : SC_ERR_CUDA;
+  return e == cudaSuccess && *static_cast<volatile int*>(word) == 0 ? SC_OK : SC_ERR_CUDA;
 }
 
 sc_status sc_mlp_backward(const uint16_t* Wbf16, const float* X, const float* cache, const float* dY, int n,
