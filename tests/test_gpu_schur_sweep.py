@@ -81,3 +81,14 @@ def test_red_inverses_solve_the_element_schur_blocks(N, tc):
         ze, ve = z[e * nb:(e + 1) * nb], v[e * nb:(e + 1) * nb]
         scale = np.abs(S).sum(axis=1).max() * np.abs(ze).max() + np.abs(ve).max()
         assert np.abs(S @ ze - ve).max() <= (2e-3 if tc else 1e-4) * scale, e
+
+
+def test_measured_solves_are_those_with_factors():
+    """The block-solve span of one application: the black elements' solve, not the product with the red
+    inverses, which is another kernel."""
+    from paper_1911_02366_gb300 import sc
+    Q, dt, p, ctx = _system(4, 2, precond=sc.SC_PC_RB_SCHUR)
+    K, _, _, nb = ctx.sc_sizes()
+    ctx.sc_profile_kernel(sc.SC_KERNEL_LU_SOLVE)
+    _apply(ctx, np.ones(K * nb))
+    assert (ctx.sc_profile_read()[0], ctx.sc_profile_elements()) == (1, K // 2)
