@@ -71,8 +71,8 @@ enum { SC_VISC_BR1 = 0, SC_VISC_SIPG = 1 };
      couplings.  The forward sweep's preconditioned operator has the spectrum of D^-1 times
      the black Schur complement, so this D takes the red couplings out of the black blocks
      (on the Taylor-Green systems about 0.7 times the sweep's iterations).  sc_condense forms
-     the red blocks' inverses (n_b solves per red element with their factors; n_red n_b^2
-     floats of device memory) and factorises the corrected black blocks; if that
+     the red blocks' inverses (products of their inverted triangles; n_red n_b floats times n_b
+     rounded up to a multiple of 4 of device memory) and factorises the corrected black blocks; if that
      factorisation meets a singular block the plain sweep runs. */
 enum { SC_PC_BLOCK_JACOBI = 0, SC_PC_NONE = 1, SC_PC_LEARNED = 2, SC_PC_RED_BLACK = 3, SC_PC_RB_SCHUR = 4 };
 

@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(352) k_rows(Geo G, int ge, const double* __res
       const double rhs = -G.dx * r[k];  // M_jj = (h/2)^3 W_j
       mx = rhs == rhs ? fmax(mx, fabs(rhs)) : INFINITY;
       const size_t i = (first + t) * 5 + k;
-      double dq = st.dt ? dt * rhs : 0.0;
+      double dq = dt * rhs;
       if (st.a != 0.0 && live) dq = fma(st.a, st.dq[i], dq);
       if (live) st.dq[i] = dq;
       y[k] = fma(st.b, dq, q[k]);

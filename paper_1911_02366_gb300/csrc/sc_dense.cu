@@ -1314,8 +1314,6 @@ inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) /
 
 namespace sc {
 
-// Blocked LU of the S_ee blocks with the trailing updates A22 -= L21 U12 as batched TF32
-// tensor-core GEMMs (mixed arm): per panel one k_lu_panel launch and one GEMM.
 // LU with partial pivoting of `batch` n x n blocks on the CUDA cores: per 32 columns one panel step per
 // block, then the trailing updates of all blocks as one batched product.  FP64-pipe bound (FP32 without
 // tensor cores: FMA bound); the panels are latency bound.  With the updates in the panel's CTA 64
@@ -1560,8 +1558,15 @@ inline long long ls_stride(const Geo& G) { return (long long)ls_nblk(G) * 32 * l
 // Below these counts the warp-per-element solve cannot fill the chip and its chain of block rows
 // sets the time, so the condensation inverts the whole triangles (sc_trinv.cu): launches over
 // every element of the mesh, and over element lists (one colour of the sweep).  Above them the
-// chains of many elements overlap: a list of 2048 elements of n_b = 490 runs at 0.83 of the HBM
-// rate, and inverting the triangles would cost more per system than the solves gain.
+// chains of many elements overlap.  Both sides measured, mixed arm: time of one application with
+// inverted / partitioned triangles, and the applications after which the inversion is paid for.
+//   block Jacobi   512 elements  N=2 24 / 36 us, 7      N=4 113 / 446 us, 7      N=6 0.39 / 1.73 ms, 23
+//                 1000           N=2 32 / 38, 27        N=4 192 / 455, 17        N=6 0.74 / 1.78, 57
+//                 1728           N=2 54 / 72, 17        N=4 311 / 482, 44        N=6 1.24 / 1.92, 151
+//                 2744           N=2 82 / 77, never     N=4 473 / 536, 186       N=5 1.02 / 1.15, 453
+//   one sweep    2 x 864         N=2 115 / 116, 164     N=4 524 / 756, 32        N=6 2.15 / 3.34, 86
+//                2 x 1372        N=2 149 / 136, never   N=4 768 / 878, 107       N=5 1.58 / 1.92, 177
+// A system takes 100 to 400 applications, so the lines lie where the inversion stops paying at most orders.
 constexpr int kSolveFullMaxElems = 2048;
 constexpr int kSolveFullMaxList = 1024;
 bool solve_full_inverse(int per_launch, bool list) {
@@ -1715,7 +1720,6 @@ cudaError_t grouped_finish(cudaStream_t st, const CondItem* items, const std::ve
   return e;
 }
 
-// C = A B for `batch` row-major FP32 blocks on the CUDA cores.
 // C -= A B for one large row-major problem on the CUDA cores (64 x 64 tiles).
 template <class T>
 cudaError_t gemm_update(sc_ctx* c, int M, int N, int K, const T* A, int lda, const T* B, int ldb, T* C, int ldc) {
@@ -1728,6 +1732,7 @@ cudaError_t gemm_update(sc_ctx* c, int M, int N, int K, const T* A, int lda, con
 template cudaError_t gemm_update<float>(sc_ctx*, int, int, int, const float*, int, const float*, int, float*, int);
 template cudaError_t gemm_update<double>(sc_ctx*, int, int, int, const double*, int, const double*, int, double*, int);
 
+// C = A B for `batch` row-major FP32 blocks on the CUDA cores.
 cudaError_t gemm_fp32(sc_ctx* c, int M, int N, int K, const float* A, long long sA, int lda, const float* B,
                       long long sB, int ldb, float* C, long long sC, int ldc, int batch) {
   dim3 g(cdiv(N, 64), cdiv(M, 64), batch);

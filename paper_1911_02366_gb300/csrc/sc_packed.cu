@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(256, PkOcc<T>::v) k_cond_boundary_pk(Geo G, co
 // CTAs per element of a pass over `count` elements and `nodes` nodes (8 per CTA at a time): enough
 // for four waves of the CTAs that reside at once, so that small meshes fill the chip and the last
 // wave is short.  With one CTA per element the boundary pass took 0.32 ms for 216 elements of order
-// 6 and 65 us for 64 of order 3 in FP64, now 0.13 ms (0.86 of HBM) and 19 us.
+// 6 and 65 us for 64 of order 3 in FP64, now 0.137 ms (0.83 of HBM) and 19 us.
 int pk_splits(int count, int nodes) {
   constexpr int kTarget = 4 * 6 * 152;
   return std::max(1, std::min((nodes + 7) / 8, (kTarget + count - 1) / count));

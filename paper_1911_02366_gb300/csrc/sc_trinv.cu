@@ -203,8 +203,8 @@ __global__ void __launch_bounds__(32 * TiWarps<float>::v) k_tri_inv_grouped(cons
 // x = L^-1 P (v - vsub) (UPPER = false, x compact per list entry) or z = U^-1 x: CTA (p, i) forms
 // the block rows p and nblk - 1 - p of list entry i, which together read the same number of
 // entries for every p; its warps share the 4-column groups and meet in shared memory.
-// HBM bound where the factors exceed L2: 365 elements of n_b = 760 (0.84 GB) take 0.15 ms
-// against 0.38 ms for the chain of block rows, 216 of n_b = 1090 (1.03 GB) 0.18 against 0.62 ms.
+// HBM bound where the factors exceed L2: 364 elements of n_b = 760 (0.84 GB) take 0.155 ms
+// (0.84 of HBM) against 0.38 ms for the chain of block rows, 216 of n_b = 1090 (1.03 GB) 0.178 (0.89) against 0.62 ms.
 constexpr int kTaWarps = 8;  // one per 4-column group of a diagonal block
 // T: arithmetic, TS: storage of the factors.
 template <class T, class TS, bool UPPER>
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(256) k_tri_product(int n, const float* __restr
 
 // z = S_ee^-1 v with the dense inverses: CTA (t, i) forms rows 128 t .. of list entry i, each lane
 // four rows, the warps sharing the columns.  HBM bound: 2048 elements of n_b = 490 (1.98 GB)
-// take 0.29 ms against 0.35 ms for the partitioned-inverse solve with the factors.
+// take 0.294 ms (0.99 of HBM) against 0.35 ms (0.87) for the partitioned-inverse solve with the factors.
 constexpr int kIgWarps = 8;
 __global__ void __launch_bounds__(32 * kIgWarps) k_inv_gemv(int n, int ldz, const float* __restrict__ Zinv,
                                                             const double* __restrict__ v, double* __restrict__ z,
