@@ -1815,9 +1815,11 @@ static cudaError_t inverse_node_blocks_refactor(sc_ctx* c, float* out) {
   return e;
 }
 
+bool node_blocks_refactored(const sc_ctx* c) { return c->cfg.precond == SC_PC_NONE || c->red_compact; }
+
 cudaError_t inverse_node_blocks32(sc_ctx* c, float* out) {
   const Geo& G = c->G;
-  if (c->cfg.precond == SC_PC_NONE || c->red_compact) return inverse_node_blocks_refactor(c, out);
+  if (node_blocks_refactored(c)) return inverse_node_blocks_refactor(c, out);
   if (c->ls_full) return tri_node_blocks(c, c->Sls32, c->rowperm, G.K, out);
   const int nblk = ls_nblk(G);
   const size_t smem = (size_t)4 * nblk * 32 * sizeof(float);

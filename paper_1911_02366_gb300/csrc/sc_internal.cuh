@@ -625,5 +625,7 @@ template <class T>
 cudaError_t gemm_update(sc_ctx* c, int M, int N, int K, const T* A, int lda, const T* B, int ldb, T* C, int ldc);
 void free_direct_factors(sc_ctx* c);
 // [S_ee^-1]_kk for every (element, boundary node) sample from the condensation's factors
+// whether that call has to form factors of its own (and reports on them in *c->d_status)
+bool node_blocks_refactored(const sc_ctx* c);
 cudaError_t inverse_node_blocks32(sc_ctx* c, float* out);
 }  // namespace sc

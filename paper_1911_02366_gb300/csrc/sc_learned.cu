@@ -404,8 +404,9 @@ sc_status sc_learned_targets(sc_ctx* c, float* T) {
     k_inverse_targets<<<(nsmp + 127) / 128, 128, 0, c->stream>>>(nsmp, Zex, c->Sdiag, T);
     e = cudaGetLastError();
   }
-  int bad = -1;  // of the factors formed for this call, if any
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+  int bad = -1;  // of the factors formed for this call; the word may hold an earlier call's report otherwise
+  if (e == cudaSuccess && sc::node_blocks_refactored(c))
+    e = cudaMemcpyAsync(&bad, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   cudaFree(Zex);
   if (e == cudaErrorMemoryAllocation) {
