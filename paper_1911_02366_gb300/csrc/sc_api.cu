@@ -402,8 +402,9 @@ sc_status sc_set_mesh(sc_ctx* c, int n, double L, int N) {
   }
   const bool sweep = c->cfg.precond == SC_PC_RED_BLACK || c->cfg.precond == SC_PC_LEARNED ||
                      c->cfg.precond == SC_PC_RB_SCHUR;
-  c->ls_full = sc::solve_full_inverse(sweep ? G.K / 2 : G.K, sweep);
-  c->black_full = sc::solve_full_inverse(c->n_black, true);
+  const bool fp64 = c->cfg.precision == SC_PREC_FP64;
+  c->ls_full = sc::solve_full_inverse(sweep ? G.K / 2 : G.K, sweep, G.nb, fp64);
+  c->black_full = sc::solve_full_inverse(c->n_black, true, G.nb, fp64);
   {
     const size_t len = (size_t)G.K * ((G.nb + 31) / 32 * 32);
     A(cudaMalloc(&c->tri_x, len * (c->cfg.precision == SC_PREC_MIXED ? sizeof(float) : sizeof(double))));

@@ -9,10 +9,13 @@
 //   k_lu_panel  one 32-column panel of the right-looking LU with partial pivoting of a batch of blocks
 //               in global memory (32-column panels factorised in shared memory).
 //   k_solve_prep  partitioned inverses of the LU factors in the solve layout (below).
+//   k_lu        the whole LU of a block per CTA (FP64, many or small blocks).
 //   k_lu_solve    z = (P^T L U)^-1 v for every element, one warp per element, one lane
-//                 per row of each 32-row block.
+//                 per row of each 32-row block; k_lu_solve_cta: eight warps per element.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "sc_internal.cuh"
@@ -390,6 +393,52 @@ __device__ void lu_panel(int n, int k0, T* __restrict__ Mx, int lda, int* __rest
     }
   }
   __syncthreads();
+}
+
+// Whole LU of one element block per CTA: panel steps with the trailing update
+// A22 -= L21 U12 done by the same CTA in 4 x 4 register tiles.
+template <class T>
+__global__ void __launch_bounds__(256) k_lu(int n, T* __restrict__ A, long long stride, int lda,
+                                            int* __restrict__ piv_all, int* __restrict__ status) {
+  extern __shared__ unsigned char smem_raw[];
+  T* P = reinterpret_cast<T*>(smem_raw);  // panel [n][PW+1]
+  constexpr int pld = PW + 1;
+  __shared__ int s_p;
+  __shared__ int s_bad;
+  const int e = blockIdx.x;
+  T* Mx = A + (long long)e * stride;
+  int* piv = piv_all + (long long)e * n;
+  if (threadIdx.x == 0) s_bad = 0;
+  __syncthreads();
+  for (int k0 = 0; k0 < n; k0 += PW) {
+    lu_panel<T>(n, k0, Mx, lda, piv, P, &s_p, &s_bad);
+    const int bw = min(PW, n - k0), rest = n - k0 - bw;
+    if (rest > 0) {
+      // A22 -= L21 U12, 4x4 register tiles
+      const int tr = (rest + 3) / 4, tcn = (rest + 3) / 4;
+      for (int t = threadIdx.x; t < tr * tcn; t += blockDim.x) {
+        const int bi = (t / tcn) * 4, bj = (t % tcn) * 4;
+        T acc[4][4];
+        for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+        for (int c = 0; c < bw; ++c) {
+          T l[4], u[4];
+          for (int a = 0; a < 4; ++a) l[a] = (bi + a < rest) ? P[(bw + bi + a) * pld + c] : T(0);
+          for (int b = 0; b < 4; ++b)
+            u[b] = (bj + b < rest) ? Mx[(long long)(k0 + c) * lda + k0 + bw + bj + b] : T(0);
+          for (int a = 0; a < 4; ++a) for (int b = 0; b < 4; ++b) acc[a][b] = fma(l[a], u[b], acc[a][b]);
+        }
+        for (int a = 0; a < 4; ++a) {
+          if (bi + a >= rest) continue;
+          for (int b = 0; b < 4; ++b) {
+            if (bj + b >= rest) continue;
+            Mx[(long long)(k0 + bw + bi + a) * lda + k0 + bw + bj + b] -= acc[a][b];
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0 && s_bad) atomicCAS(status, -1, e);
 }
 
 // One panel step for every element (the trailing update is a separate batched GEMM).
@@ -1260,9 +1309,128 @@ __device__ __forceinline__ void ls_solve_warp_pf(int n, int nblk, const TS* __re
   }
 }
 
-// Element lists (red-black sweep): warp i serves element elist[i] (all elements when elist is
-// null); its factors are number i of LS / rowperm when compact, else number e; vsub (optional)
-// is subtracted from v on input.
+// The same solve by W warps: they share a block row's long dot product, the first one ends the row.
+template <class T, class TS, int W>
+__device__ __forceinline__ void ls_solve_cta(int n, int nblk, const TS* __restrict__ Le, int npad, T* s, T* red) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nq = npad / 4;
+  for (int b = 0; b < nblk; ++b) {  // forward
+    const int i0 = 32 * b, R = i0 + lane;
+    const bool live = R < n;
+    const TS* row = Le + (long long)b * 32 * npad + 4 * lane;
+    T a0 = T(0), a1 = T(0);
+    if (live) {
+#pragma unroll 4
+      for (int q = w; q < i0 / 4; q += W) {
+        Quad<T, TS> m;
+        m.load(row + (long long)q * 128);
+        a0 = fma(m.v[0], s[4 * q], a0);
+        a1 = fma(m.v[1], s[4 * q + 1], a1);
+        a0 = fma(m.v[2], s[4 * q + 2], a0);
+        a1 = fma(m.v[3], s[4 * q + 3], a1);
+      }
+    }
+    red[w * 32 + lane] = a0 + a1;
+    __syncthreads();
+    if (w == 0) {
+      T d = s[R];
+      const int qd = min(i0 / 4 + 8, nq);
+#pragma unroll
+      for (int q = i0 / 4; q < qd; ++q) {
+        if (live && 4 * q < R) {
+          Quad<T, TS> m;
+          m.load(row + (long long)q * 128);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (4 * q + j < R) d = fma(m.v[j], s[4 * q + j], d);
+        }
+      }
+      T sum = T(0);
+#pragma unroll
+      for (int k = 0; k < W; ++k) sum += red[k * 32 + lane];
+      __syncwarp();
+      if (live) s[R] = d - sum;
+    }
+    __syncthreads();
+  }
+  for (int b = nblk - 1; b >= 0; --b) {  // backward
+    const int i0 = 32 * b, R = i0 + lane;
+    const bool live = R < n;
+    const TS* row = Le + (long long)b * 32 * npad + 4 * lane;
+    T a0 = T(0), a1 = T(0);
+    if (live) {
+#pragma unroll 4
+      for (int q = i0 / 4 + 8 + w; q < nq; q += W) {
+        Quad<T, TS> m;
+        m.load(row + (long long)q * 128);
+        a0 = fma(m.v[0], s[4 * q], a0);
+        a1 = fma(m.v[1], s[4 * q + 1], a1);
+        a0 = fma(m.v[2], s[4 * q + 2], a0);
+        a1 = fma(m.v[3], s[4 * q + 3], a1);
+      }
+    }
+    red[w * 32 + lane] = a0 + a1;
+    __syncthreads();
+    if (w == 0) {
+      T d = T(0);
+      const int qd = min(i0 / 4 + 8, nq);
+#pragma unroll
+      for (int q = i0 / 4; q < qd; ++q) {
+        if (live && 4 * q + 3 >= R) {
+          Quad<T, TS> m;
+          m.load(row + (long long)q * 128);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (4 * q + j >= R) d = fma(m.v[j], s[4 * q + j], d);
+        }
+      }
+      T sum = T(0);
+#pragma unroll
+      for (int k = 0; k < W; ++k) sum += red[k * 32 + lane];
+      __syncwarp();
+      if (live) s[R] = d - sum;
+    }
+    __syncthreads();
+  }
+}
+
+constexpr int kSolveCtaWarps = 8;
+
+// Element lists (red-black sweep): CTA / warp i serves element elist[i] (all elements when
+// elist is null); its factors are number i of LS / rowperm when compact, else number e;
+// vsub (optional) is subtracted from v on input.
+template <class T, class TS, int W = kSolveCtaWarps>
+__global__ void __launch_bounds__(32 * W) k_lu_solve_cta(int n, int nblk, const TS* __restrict__ LS,
+                                                                      long long lsstride, int npad,
+                                                                      const int* __restrict__ rowperm,
+                                                                      const double* __restrict__ v,
+                                                                      double* __restrict__ z, T* __restrict__ zt,
+                                                                      const int* __restrict__ elist, int compact,
+                                                                      const double* __restrict__ vsub) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int e = elist ? __ldg(elist + blockIdx.x) : blockIdx.x, ls = nblk * 32;
+  const int f = compact ? blockIdx.x : e;
+  T* s = reinterpret_cast<T*>(smem_raw);
+  T* red = s + ls;
+  const int* rp = rowperm + (long long)f * n;
+  const double* ve = v + (long long)e * n;
+  const double* we = vsub ? vsub + (long long)e * n : nullptr;
+  for (int i = threadIdx.x; i < ls; i += blockDim.x) {
+    T val = T(0);
+    if (i < n) {
+      const int r = __ldg(rp + i);
+      val = we ? (T)(ve[r] - we[r]) : (T)ve[r];
+    }
+    s[i] = val;
+  }
+  __syncthreads();
+  ls_solve_cta<T, TS, W>(n, nblk, LS + (long long)f * lsstride, npad, s, red);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    if (z) z[(long long)e * n + i] = (double)s[i];
+    if (zt) zt[(long long)e * n + i] = s[i];
+  }
+}
+
 // z = (P^T L U)^-1 v, one warp per element (4 per CTA); the running vector (v, then x,
 // then z) sits in shared memory.  Arithmetic in the factor precision T; v in double,
 // outputs z (double) and / or zt (T).
@@ -1318,10 +1486,24 @@ namespace sc {
 // block, then the trailing updates of all blocks as one batched product.  FP64-pipe bound (FP32 without
 // tensor cores: FMA bound); the panels are latency bound.  With the updates in the panel's CTA 64
 // blocks of n_b = 280 kept 64 SMs at FP64 rate and the others idle (3.2 ms; now 1.6 ms of panels and
-// the products on all SMs).
+// the products on all SMs).  FP64 blocks keep the one-CTA form (k_lu) where it is the faster one: three
+// blocks per SM fill the chip by themselves, and the single panels of small blocks do not pay their
+// launches.  Condensations with k_lu / by panels: n_b = 130: 64 elements 1.13 / 1.25 ms, 512 3.26 / 4.21;
+// 280: 64 5.1 / 4.2, 343 13.6 / 13.8, 512 19.1 / 21.0, 1000 34 / 39; 490: 125 29.2 / 29.2, 343 80.9 / 80.1,
+// 512 112.5 / 116, 1000 208 / 221; 760: 64 92 / 72, 512 486 / 481, 729 653 / 671.  In FP32 the panels are
+// never slower (512 elements, n_b = 130 to 760: 0.96 / 0.99, 3.8 / 3.7, 18.0 / 15.4, 63 / 50 ms).
 template <class T>
-static cudaError_t lu_blocked_simt(sc_ctx* c, int n, T* A, long long stride, int lda, int batch, int* piv, int* status) {
+static cudaError_t lu_simt(sc_ctx* c, int n, T* A, long long stride, int lda, int batch, int* piv, int* status) {
   const size_t smem = (size_t)n * (PW + 1) * sizeof(T);
+  if constexpr (std::is_same<T, double>::value) {
+    if (n <= 130 || batch >= 3 * 152) {
+      cudaError_t e = cudaFuncSetAttribute(k_lu<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           kMaxNb<T> * (PW + 1) * (int)sizeof(T));
+      if (e != cudaSuccess) return e;
+      k_lu<T><<<batch, 256, smem, c->stream>>>(n, A, stride, lda, piv, status);
+      return cudaGetLastError();
+    }
+  }
   cudaError_t err = cudaFuncSetAttribute(k_lu_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kMaxNb<T> * (PW + 1) * (int)sizeof(T));
   if (err != cudaSuccess) return err;
@@ -1506,7 +1688,7 @@ cudaError_t condense_t(sc_ctx* c, T* Aown, T* Ainv, T* Y, T* See, bool tc, bool 
     }
     if (!done) {
       ProfScope ps(c, SCK_LU);
-      err = lu_blocked_simt<T>(c, nb, See, (long long)nb * lds, lds, K, c->piv, c->d_status);
+      err = lu_simt<T>(c, nb, See, (long long)nb * lds, lds, K, c->piv, c->d_status);
       if (err != cudaSuccess) return err;
     }
     count_launch(c, 2);
@@ -1555,22 +1737,32 @@ inline int ls_nblk(const Geo& G) { return (G.nb + 31) / 32; }
 inline int ls_npad(const Geo& G) { return (G.nb + 3) & ~3; }
 inline long long ls_stride(const Geo& G) { return (long long)ls_nblk(G) * 32 * ls_npad(G); }
 
-// Below these counts the warp-per-element solve cannot fill the chip and its chain of block rows
-// sets the time, so the condensation inverts the whole triangles (sc_trinv.cu): launches over
-// every element of the mesh, and over element lists (one colour of the sweep).  Above them the
-// chains of many elements overlap.  Both sides measured, mixed arm: time of one application with
-// inverted / partitioned triangles, and the applications after which the inversion is paid for.
-//   block Jacobi   512 elements  N=2 24 / 36 us, 7      N=4 113 / 446 us, 7      N=6 0.39 / 1.73 ms, 23
-//                 1000           N=2 32 / 38, 27        N=4 192 / 455, 17        N=6 0.74 / 1.78, 57
-//                 1728           N=2 54 / 72, 17        N=4 311 / 482, 44        N=6 1.24 / 1.92, 151
-//                 2744           N=2 82 / 77, never     N=4 473 / 536, 186       N=5 1.02 / 1.15, 453
-//   one sweep    2 x 864         N=2 115 / 116, 164     N=4 524 / 756, 32        N=6 2.15 / 3.34, 86
-//                2 x 1372        N=2 149 / 136, never   N=4 768 / 878, 107       N=5 1.58 / 1.92, 177
-// A system takes 100 to 400 applications, so the lines lie where the inversion stops paying at most orders.
-constexpr int kSolveFullMaxElems = 2048;
-constexpr int kSolveFullMaxList = 1024;
-bool solve_full_inverse(int per_launch, bool list) {
-  return per_launch < (list ? kSolveFullMaxList : kSolveFullMaxElems);
+// Block solves with the S_ee factors take one of three forms: with inverted triangles (sc_trinv.cu), with the
+// partitioned inverses by a CTA per element, or by a warp per element.  From kSolveCtaMaxElems elements per
+// launch on (kSolveCtaMaxList for element lists, one colour of the sweep) the chains of block rows of many
+// elements overlap and a warp per element is fastest.  Below, a chain sets the time, and inverted
+// triangles, which have none, solve two to five times as fast; but the condensation pays 2/3 n_b^3 flops
+// per element for them.  Applications after which they have paid (CTA form against inverted
+// triangles, milliseconds of inversion over the difference of one application; a sweep is two lists):
+//   FP32 elements  512: N=4 2.3 / 0.11 (21), N=5 11 / 0.17 (66), N=6 31 / 0.27 (111)
+//                 1000: N=5 22 / 0.37 (59), N=6 59 / 0.62 (96)
+//                 1728: N=4 7.5 / 0.14 (53), N=5 38 / 0.19 (203), N=6 103 / 0.26 (393)
+//   FP32 lists     500: N=6 59 / 0.71 (84)   864: N=4 7.5 / 0.12 (62), N=5 38 / 0.22 (173), N=6 103 / 0.32 (325)
+//   FP64 elements   64: N=3 1.1 / 0.054 (21), N=5 20 / 0.46 (44)   125: N=4 12 / 0.21 (54), N=5 38 / 0.40 (94)
+//                  216: N=4 19 / 0.19 (102), N=5 64 / 0.33 (193)   512: N=2 1.1 / 0.008, N=3 6.1 / 0.063 (97), N=4 45 / 0.13 (338)
+//                 1000: N=2 2.0 / 0.058 (34), N=3 12 / 0.13 (90), N=4 86 / 0.26 (332)   1728: N=2 3.2 / 0.039 (82)
+//   FP64 lists     172: N=4 30 / 0.55 (55), N=5 101 / 1.06 (95)   256: N=3 6.2 / 0.20 (31), N=4 45 / 0.47 (95)
+//                  500: N=3 12 / 0.23 (51), N=4 86 / 0.50 (171)   864: N=2 3.2 / 0.076 (43), N=3 20 / 0.17 (113)
+// A system takes 110 to 190 applications with block Jacobi (CFL 10 and 20), half as many with a sweep.
+// FP64, whose inversion runs at 1.2 TFLOP/s, therefore stops at count n_b^1.5 = 5e6 (1067 elements of
+// N = 3, 461 of 4, 238 of 5; all of 2), lists at half of that; FP32 at two thirds of the CTA form's range
+// for N = 5 and 6.
+constexpr int kSolveCtaMaxElems = 2048;
+constexpr int kSolveCtaMaxList = 1024;
+bool solve_full_inverse(int count, bool list, int nb, bool fp64) {
+  const int cta = list ? kSolveCtaMaxList : kSolveCtaMaxElems;
+  if (count >= cta) return false;
+  return fp64 ? count * (nb * std::sqrt((double)nb)) <= (list ? 2.5e6 : 5e6) : nb < 700 || count < 2 * cta / 3;
 }
 
 template <class T, class TS>
@@ -1578,6 +1770,12 @@ cudaError_t lu_solve_t(sc_ctx* c, const TS* LS, const double* v, double* z, T* z
   const Geo& G = c->G;
   ProfScope ps(c, SCK_LU_SOLVE);
   if (c->ls_full) return tri_solve<T, TS>(c, LS, c->rowperm, 0, nullptr, G.K, v, nullptr, z, zt);
+  if (G.K < kSolveCtaMaxElems) {
+    const size_t csm = (size_t)(ls_nblk(G) + kSolveCtaWarps) * 32 * sizeof(T);
+    k_lu_solve_cta<T, TS><<<G.K, 32 * kSolveCtaWarps, csm, c->stream>>>(G.nb, ls_nblk(G), LS, ls_stride(G), ls_npad(G),
+                                                                       c->rowperm, v, z, zt, nullptr, 0, nullptr);
+    return cudaGetLastError();
+  }
   const size_t smem = (size_t)4 * ls_nblk(G) * 32 * sizeof(T);
   k_lu_solve<T, TS><<<cdiv(G.K, 4), 128, smem, c->stream>>>(G.nb, ls_nblk(G), LS, ls_stride(G), ls_npad(G),
                                                             c->rowperm, v, z, zt, G.K, nullptr, 0, nullptr);
@@ -1593,6 +1791,12 @@ cudaError_t lu_solve_list_t(sc_ctx* c, const T* LS, const int* rowperm, int comp
   if (nlist <= 0) return cudaSuccess;
   ProfScope ps(c, SCK_LU_SOLVE, nlist);
   if (full) return tri_solve<T, T>(c, LS, rowperm, compact, elist, nlist, v, vsub, z, zt);
+  if (nlist < kSolveCtaMaxList) {
+    const size_t csm = (size_t)(ls_nblk(G) + kSolveCtaWarps) * 32 * sizeof(T);
+    k_lu_solve_cta<T, T><<<nlist, 32 * kSolveCtaWarps, csm, c->stream>>>(G.nb, ls_nblk(G), LS, ls_stride(G), ls_npad(G),
+                                                                        rowperm, v, z, zt, elist, compact, vsub);
+    return cudaGetLastError();
+  }
   const size_t smem = (size_t)4 * ls_nblk(G) * 32 * sizeof(T);
   // FP32 factors: loads issued ahead (128 registers, 4 CTAs per SM hold one colour of 16^3)
   constexpr bool pf = std::is_same<T, float>::value;
@@ -1751,7 +1955,7 @@ cudaError_t factor_batch32(sc_ctx* c, float* A, int n, int lda, long long stride
     if (err != cudaSuccess) return err;
     count_launch(c, 3);
   } else {
-    err = lu_blocked_simt<float>(c, n, A, stride, lda, batch, piv, status);
+    err = lu_simt<float>(c, n, A, stride, lda, batch, piv, status);
     if (err != cudaSuccess) return err;
     count_launch(c, 4);
   }

@@ -542,8 +542,8 @@ void build_packed_pattern(sc_ctx* c);
 long long solve_layout_stride(const Geo& G);
 cudaError_t factor_batch32(sc_ctx* c, float* A, int n, int lda, long long stride, int batch, int* piv, int* rowperm,
                            float* LS, int* status, bool full);
-// Meshes whose block solves use the inverted triangles: `per_launch` elements per solve launch.
-bool solve_full_inverse(int per_launch, bool list);
+// Whether block solves of `count` elements per launch (a list: one colour of the sweep) use the inverted triangles.
+bool solve_full_inverse(int count, bool list, int nb, bool fp64);
 template <class T>
 cudaError_t tri_inverse(sc_ctx* c, int n, const T* LU, long long stride, int lda, T* LS, int count,
                         __half* LS16 = nullptr, int* ovf = nullptr);

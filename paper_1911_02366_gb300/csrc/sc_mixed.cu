@@ -1189,7 +1189,7 @@ sc_status sc_mixed_create(const sc_config* cfg, void* cuda_stream, int n, double
     c.view = new sc_ctx();
     c.view->G = Gc; c.view->stream = c.st; c.view->cfg = *cfg;
     c.view->rowperm = c.rowperm;
-    c.view->ls_full = sc::solve_full_inverse(c.count, true);
+    c.view->ls_full = sc::solve_full_inverse(c.count, true, c.nb, false);
     float* tx = nullptr;
     A(mx_alloc(&tx, k * (size_t)((c.nb + 31) / 32 * 32)));
     c.view->tri_x = tx;
